@@ -1,5 +1,6 @@
 // otm_api.cu -- the C ABI (include/otm.h): workspace layout, initialisation, the step driver
 // (Algorithm 1 as a fixed kernel sequence on one stream) and state transfer.
+#include <math.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -31,6 +32,7 @@ struct otm_handle {
     bool adj_swap;
     bool adj_shape_swap;           // the two state-shape buffers of the adjoint workspace trade roles
     int64_t adj_shape_step;        // state whose shape functions the spare buffer holds (-1: none)
+    bool state_fix;                // the state's shape functions come from fixed-point evaluations
     bool contrib_stale;            // node-major contributions not regenerated by the last load
     void *keep_buf;                // otm_keep_last_good: snapshot of the state before the running step
     // phase timing
@@ -98,6 +100,7 @@ static size_t layout(int64_t nn, int64_t nn_cap, int64_t nm, int S, int precisio
     TAKE(d.spos, double4_32a, nn_cap);
     TAKE(d.spos32, float4, nn_cap);
     TAKE(d.du32, float4, nn_cap);
+    TAKE(d.xfix, longlong4_32a, nn_cap);
     TAKE(d.nflags, uint8_t, nn_cap);
     TAKE(d.ngid, int64_t, nn_cap);
     TAKE(d.ncount, int32_t, nn_cap);
@@ -134,6 +137,7 @@ static size_t layout(int64_t nn, int64_t nn_cap, int64_t nm, int S, int precisio
     TAKE(d.failed, uint8_t, nm);
     TAKE(d.lme_fail, uint8_t, nm);
     TAKE(d.n_fail, int32_t, 1);
+    TAKE(d.fstart, FixStart, nm);
     TAKE(d.lme_defer, int32_t, nm);
     TAKE(d.n_defer, int32_t, 1);
     TAKE(d.flag, int32_t, 1);
@@ -198,6 +202,10 @@ static void fill_params(Dev &D, const otm_params *P)
     D.rs2 = P->rs2;
     D.cell = P->cell_size;
     D.sc = make_search_const(P->cell_size, P->rs2);
+    D.fix = make_fix_const(P->beta, P->rs2);
+    // FP64 path: log of the weights' sum of a regular cloud of spacing h, plus ln 2.8: the first sums
+    // start near 0.35, inside the fixed-point evaluation's window
+    D.logz0 = P->precision == OTM_PRECISION_FP64 ? 1.5 * log(3.141592653589793 / (P->beta * P->h * P->h)) + 1.04 : 0.0;
     D.dt = P->dt;
     D.tol_abs = P->newton_tol * P->h;
     D.eps_stab = P->eps_stab;
@@ -234,6 +242,19 @@ static int read_error(otm_handle *h, int32_t *code, int64_t *id)
     return c;
 }
 
+// The LME solve of the current positions and supports. A solve that only regenerates the shape functions
+// of the state (kLmeKeep) evaluates them as the solve that led to the state did, whichever path that
+// was, and so repeats them bit for bit; any other solve evaluates as this handle's path does.
+static int solve_lme(otm_handle *h, int lme_mode)
+{
+    Dev &D = h->D;
+    D.lme_mode = lme_mode;
+    if (lme_mode != kLmeKeep) h->state_fix = D.precision == OTM_PRECISION_FP64 && D.fix.on;
+    D.lme_fix = h->state_fix && D.fix.on;
+    CK(launch_lme(D, h->stream, &h->launches));
+    return OTM_OK;
+}
+
 // steps 5-6 of Algorithm 1 plus the node-major lists for the next step's step 1; with `insert`,
 // MPs whose LME solve fails are flagged for node insertion instead of stopping the step
 static int rebuild_supports(otm_handle *h, bool insert, int lme_mode)
@@ -241,7 +262,6 @@ static int rebuild_supports(otm_handle *h, bool insert, int lme_mode)
     Dev &D = h->D;
     cudaStream_t s = h->stream;
     D.insert_mode = insert ? 1 : 0;
-    D.lme_mode = lme_mode;
     {
         PhaseScope ps(h, OTM_PHASE_GRID);
         CK(launch_grid_build(D, s, &h->launches));
@@ -258,7 +278,8 @@ static int rebuild_supports(otm_handle *h, bool insert, int lme_mode)
     }
     {
         PhaseScope ps(h, OTM_PHASE_LME);
-        CK(launch_lme(D, s, &h->launches));
+        const int rc = solve_lme(h, lme_mode);
+        if (rc != OTM_OK) return rc;
     }
     D.insert_mode = 0;
     return OTM_OK;
@@ -372,8 +393,8 @@ static int regenerate_contributions(otm_handle *h)
     if (!h->contrib_stale) return OTM_OK;
     Dev &D = h->D;
     CK(cudaMemsetAsync(D.emax, 0x80, 2 * sizeof(int), h->stream));
-    D.lme_mode = kLmeKeep;
-    CK(launch_lme(D, h->stream, &h->launches));
+    const int rc = solve_lme(h, kLmeKeep);
+    if (rc != OTM_OK) return rc;
     h->contrib_stale = false;
     return OTM_OK;
 }
@@ -405,8 +426,8 @@ static int enqueue_step(otm_handle *h)
         CK(cudaMemsetAsync(D.emax, 0x80, 2 * sizeof(int), s));
         {
             PhaseScope ps(h, OTM_PHASE_LME);
-            D.lme_mode = kLmeStep;
-            CK(launch_lme(D, s, &h->launches));
+            const int rc = solve_lme(h, kLmeStep);
+            if (rc != OTM_OK) return rc;
         }
         h->step++;
         return OTM_OK;
@@ -435,8 +456,8 @@ static int enqueue_step(otm_handle *h)
         {
             PhaseScope ps(h, OTM_PHASE_LME);
             D.insert_mode = h->P.max_insert > 0 ? 1 : 0;
-            D.lme_mode = kLmeStep;
-            CK(launch_lme(D, s, &h->launches));
+            const int rc = solve_lme(h, kLmeStep);
+            if (rc != OTM_OK) return rc;
             D.insert_mode = 0;
         }
         if (h->P.max_insert > 0) {
@@ -814,8 +835,8 @@ static int replay_step(otm_handle *h, Place place)
     }
     {
         PhaseScope ps(h, OTM_PHASE_LME);
-        D.lme_mode = kLmeStep;
-        CK(launch_lme(D, s, &h->launches));
+        const int rc = solve_lme(h, kLmeStep);
+        if (rc != OTM_OK) return rc;
     }
     h->step++;
     return read_error(h, nullptr, nullptr);
@@ -951,6 +972,7 @@ extern "C" void otm_destroy(otm_handle *h)
 struct SnapHeader {
     int64_t nn, nm, step, magic, n_inserted;
     int64_t nn_cap, nm_cap, S;     // the layout the snapshot was written with
+    int64_t state_fix;             // its shape functions come from fixed-point evaluations
 };
 struct SnapField {
     void *p;
@@ -996,7 +1018,8 @@ extern "C" int otm_snapshot_save(otm_handle *h, void *dst)
     if (!h || !dst || (((uintptr_t)dst) & 255)) return OTM_ERR_ARG;
     SnapField f[32];
     const int n = snap_fields(h, f);
-    SnapHeader hd = {h->D.nn, h->D.nm, h->step, 0x4f544d53, h->n_inserted, h->nn_cap, h->nm0, h->D.S};
+    SnapHeader hd = {h->D.nn, h->D.nm, h->step, 0x4f544d53, h->n_inserted, h->nn_cap, h->nm0, h->D.S,
+                     h->state_fix ? 1 : 0};
     CK(cudaMemcpyAsync(dst, &hd, sizeof(hd), cudaMemcpyDefault, h->stream));
     char *o = (char *)dst + 256;
     for (int i = 0; i < n; i++) {
@@ -1025,6 +1048,7 @@ static int snapshot_load_impl(otm_handle *h, const void *src, const double4_32a 
     h->D.nm = hd.nm;
     h->step = hd.step;
     h->n_inserted = hd.n_inserted;
+    h->state_fix = hd.state_fix != 0;
     SnapField f[32];
     const int n = snap_fields(h, f);
     const char *o = (const char *)src + 256;
@@ -1051,8 +1075,8 @@ static int snapshot_load_impl(otm_handle *h, const void *src, const double4_32a 
         CK(cudaMemcpyAsync(D.Kinv, K, (size_t)D.nm * 48, cudaMemcpyDeviceToDevice, h->stream));
         h->contrib_stale = true;
     } else {
-        D.lme_mode = kLmeKeep;
-        CK(launch_lme(D, h->stream, &h->launches));
+        const int rc = solve_lme(h, kLmeKeep);
+        if (rc != OTM_OK) return rc;
         h->contrib_stale = false;
     }
     return read_error(h, nullptr, nullptr);

@@ -14,6 +14,7 @@
 #include <stdint.h>
 
 #include "../../include/otm.h"
+#include "otm_fix.cuh"
 
 namespace otm {
 
@@ -48,7 +49,14 @@ struct SearchConst {
     float rs2_rd, rs2_ru;  // rs2 rounded down / up to FP32
 };
 
+// the start of one MP's fixed-point LME solve (k_lme_prep -> k_lme_fix, copied word by word)
+struct FixStart {
+    double trial[3];
+    i64 xp[3], v[3], cst, ok, pad;
+};
+
 SearchConst make_search_const(double cell, double rs2);
+FixConst make_fix_const(double beta, double rs2);
 
 struct Dev {
     // sizes and parameters
@@ -58,6 +66,9 @@ struct Dev {
     int max_cells;
     double h, beta, rs2, cell, dt, tol_abs, eps_stab;
     SearchConst sc;
+    FixConst fix;                    // fixed-point LME evaluation
+    int lme_fix;                     // 1: this LME launch evaluates in fixed point (see launch_lme)
+    double logz0;                    // exponent shift of the first solve
     int max_newton;
     int wall, tool, allow_erode;
     int insert_mode;                 // 1: an MP whose LME solve fails is flagged for node insertion
@@ -69,6 +80,7 @@ struct Dev {
     // nodes
     double4_32a *x, *x_prev, *du, *mr;   // mr = (mass, force xyz) of the last node update
     float4 *du32;
+    longlong4_32a *xfix;             // fixed-point node positions of the running LME solve (otm_fix.cuh)
     uint8_t *nflags;
     int64_t *ngid;
     int32_t *ncount, *noff;          // influence counts (atomics) and node-major offsets
@@ -87,6 +99,7 @@ struct Dev {
     uint8_t *failed;                 // fracture flags of the step
     uint8_t *lme_fail;               // LME failures of the step (node insertion)
     int32_t *n_fail;                 // their count
+    FixStart *fstart;                // starts of the fixed-point LME solves
     int32_t *lme_defer;              // MPs whose support exceeds k_lme's shared-memory rows
     int32_t *n_defer;                // their count (k_lme_wide solves them)
     int32_t *flag;                   // one int of scratch for host-read checks (argument validation)
@@ -235,24 +248,25 @@ __device__ __forceinline__ T warp_reduce_scatter12(const T (&v)[12], int lane)
 // Reduce-scatter of 10 per-lane values in 12 additions per lane. Afterwards lane L holds the
 // warp total of value rs10_value(L); rs10_writer(L) picks one lane per value, and value j can
 // be read from lane {0, 2, 4, 8, 10, 16, 18, 20, 24, 26}[j].
-__device__ __forceinline__ double warp_reduce_scatter10(const double (&v)[10], int lane)
+template <typename T>
+__device__ __forceinline__ T warp_reduce_scatter10(const T (&v)[10], int lane)
 {
-    double a[5];
+    T a[5];
 #pragma unroll
     for (int i = 0; i < 5; i++) {
         const bool up = lane & 16;
-        const double mine = up ? v[5 + i] : v[i], other = up ? v[i] : v[5 + i];
+        const T mine = up ? v[5 + i] : v[i], other = up ? v[i] : v[5 + i];
         a[i] = mine + __shfl_xor_sync(0xffffffffu, other, 16);
     }
     const bool up8 = lane & 8;
-    const double b0 = (up8 ? a[3] : a[0]) + __shfl_xor_sync(0xffffffffu, up8 ? a[0] : a[3], 8);
-    const double b1 = (up8 ? a[4] : a[1]) + __shfl_xor_sync(0xffffffffu, up8 ? a[1] : a[4], 8);
-    const double b2 = a[2] + __shfl_xor_sync(0xffffffffu, a[2], 8);
+    const T b0 = (up8 ? a[3] : a[0]) + __shfl_xor_sync(0xffffffffu, up8 ? a[0] : a[3], 8);
+    const T b1 = (up8 ? a[4] : a[1]) + __shfl_xor_sync(0xffffffffu, up8 ? a[1] : a[4], 8);
+    const T b2 = a[2] + __shfl_xor_sync(0xffffffffu, a[2], 8);
     const bool up4 = lane & 4;
-    const double c0 = (up4 ? b2 : b0) + __shfl_xor_sync(0xffffffffu, up4 ? b0 : b2, 4);
-    const double c1 = b1 + __shfl_xor_sync(0xffffffffu, b1, 4);
+    const T c0 = (up4 ? b2 : b0) + __shfl_xor_sync(0xffffffffu, up4 ? b0 : b2, 4);
+    const T c1 = b1 + __shfl_xor_sync(0xffffffffu, b1, 4);
     const bool up2 = lane & 2;
-    const double dd = (up2 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, up2 ? c0 : c1, 2);
+    const T dd = (up2 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, up2 ? c0 : c1, 2);
     return dd + __shfl_xor_sync(0xffffffffu, dd, 1);
 }
 

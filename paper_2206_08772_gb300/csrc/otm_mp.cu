@@ -15,6 +15,7 @@
 #include <mutex>
 
 #include "otm_dev.cuh"
+#include "otm_fix.cuh"
 #include "otm_rm.cuh"
 
 namespace otm {
@@ -96,6 +97,7 @@ constexpr int kExpNmin = -1020 * 1024;                 // 2^(n >> 10) stays norm
 constexpr int kExpNmax = 1021 * 1024 + 1023;
 
 static __device__ double g_exp2_table[kExpTable];
+static __device__ u64 g_exp2_mant[kExpTable];          // 2^(j/1024) as 64-bit mantissas (fix_exp)
 
 // Fill g_exp2_table on the current device (first call per device; a synchronous copy, so it
 // belongs before any stream capture: otm_init and the stand-alone entries call it). With
@@ -121,6 +123,11 @@ cudaError_t exp_table_setup(bool verify)
     if (done[dev]) return cudaSuccess;
     double host[kExpTable];
     for (int j = 0; j < kExpTable; j++) host[j] = std::exp2((double)j / (double)kExpTable);
+    u64 mant[kExpTable];
+    for (int j = 0; j < kExpTable; j++)
+        mant[j] = (u64)std::floor(std::ldexp(std::exp2((long double)j / (long double)kExpTable), 63) + 0.5L);
+    e = cudaMemcpyToSymbol(g_exp2_mant, mant, sizeof(mant));
+    if (e != cudaSuccess) return e;
     e = cudaMemcpyToSymbol(g_exp2_table, host, sizeof(host));
     if (e == cudaSuccess) done[dev] = true;
     return e;
@@ -682,6 +689,8 @@ __device__ __forceinline__ void newton_fail(MpNewton &m)
 
 // the solve has converged at C (whose Hessian sums are FP64): J'^-1, 1/Z and the next shift for
 // the outputs
+// ZOFF: the binary exponent the next solve's Z starts below (see the end)
+template <int ZOFF>
 __device__ __forceinline__ void newton_finish(MpNewton &m)
 {
     const LmeSums c = sums_of(m.C);
@@ -691,14 +700,16 @@ __device__ __forceinline__ void newton_finish(MpNewton &m)
         return;
     }
     for (int i = 0; i < 6; i++) m.inv[i] = inv[i];
-    // the next solve's shift only has to keep the weights near 1: log Z to within ln 2, from the
-    // binary exponent of Z (Z > 0 and finite here)
+    // the next solve's shift only has to keep the weights in range: log Z + ZOFF ln 2 to within ln 2, from
+    // the binary exponent of Z (Z > 0 and finite here); ZOFF = 2 starts the next sums at Z in
+    // [1/4, 1/2), the middle of the fixed-point evaluation's window
     const int ez = ((__double2hiint(c.Z) >> 20) & 0x7ff) - 1023;
-    m.logz = fma((double)ez, 0x1.62e42fefa39efp-1, c.shift);
+    m.logz = fma((double)(ez + ZOFF), 0x1.62e42fefa39efp-1, c.shift);
     m.state = kNewtonDone;
 }
 
 // one scalar round after an evaluation (the damped Newton of lme_newton_loop, as a state machine)
+template <int ZOFF>
 __device__ void newton_round(MpNewton &m, double tol, int max_it)
 {
     if (m.state != kNewtonEval) return;
@@ -731,7 +742,7 @@ __device__ void newton_round(MpNewton &m, double tol, int max_it)
     }
     double inv[6];
     if (r2 <= tol * tol * c.Z * c.Z) {   // converged
-        newton_finish(m);
+        newton_finish<ZOFF>(m);
         return;
     }
     if (m.iters >= max_it || !lme_jinv(c, inv)) {
@@ -988,7 +999,7 @@ __device__ __forceinline__ void lme_record(const Dev &D, int64_t p, double l0, d
     D.lam[3 * p + 2] = l2;
 }
 
-// Shared-memory rows per MP in k_lme. With 336 slots a block of 4 MPs takes 55 KB and 4 blocks
+// Shared-memory rows per MP in k_lme and k_lme_fix. With 336 slots a block of 4 MPs takes 55 KB and 4 blocks
 // fit an SM (3 with full 384-slot rows), which hides more of the FP64 pipe's dependency and
 // barrier stalls; the supports of the benchmark rods stay below (at most 316 slots mid-run on the
 // 2.85 M-MP rod). MPs with larger supports are deferred to k_lme_wide, which runs the same block
@@ -996,6 +1007,108 @@ __device__ __forceinline__ void lme_record(const Dev &D, int64_t p, double l0, d
 constexpr int kLmeRows = 336;
 
 __host__ __device__ __forceinline__ int lme_rows(int S) { return S < kLmeRows ? S : kLmeRows; }
+
+// the solve's start: the warm start and an evaluation pending there
+__device__ __forceinline__ void lme_start(const Dev &D, int64_t p, MpNewton &M, double shift0)
+{
+    // Eq. 14: the warm start is the previous step's lambda, or (within a step) the cubic
+    // through the last four solutions: while the material deforms smoothly one Newton
+    // step from it meets the tolerance
+    double l0 = D.lam[3 * p], l1 = D.lam[3 * p + 1], l2 = D.lam[3 * p + 2];
+    if (D.lme_mode == kLmeStep) {
+        // cubic: 4 l_n - 6 l_{n-1} + 4 l_{n-2} - l_{n-3}
+        const double *a1 = D.lam_prev + 3 * p, *a2 = D.lam_prev2 + 3 * p, *a3 = D.lam_prev3 + 3 * p;
+        l0 = fma(4.0, l0 + a2[0], -fma(6.0, a1[0], a3[0]));
+        l1 = fma(4.0, l1 + a2[1], -fma(6.0, a1[1], a3[1]));
+        l2 = fma(4.0, l2 + a2[2], -fma(6.0, a1[2], a3[2]));
+    }
+    M.trial[0] = M.ws[0] = l0;
+    M.trial[1] = M.ws[1] = l1;
+    M.trial[2] = M.ws[2] = l2;
+    M.t = 1.0;
+    M.have_cur = M.iters = M.iters_total = M.halvings = M.retried = 0;
+    M.shift0 = shift0;
+    newton_set_trial(M);
+}
+
+// records the solve of MP p; false if it failed (nothing more to write for this MP)
+__device__ __forceinline__ bool lme_finish(const Dev &D, int64_t p, int cnt, const MpNewton &M, double shift0, int lane)
+{
+    const int st = M.state == kNewtonDone ? OTM_OK : OTM_ERR_LME_NOCONV;
+    if (lane == 0) {
+        D.newton_it[p] = M.iters_total;
+        if (st == OTM_OK) {
+            lme_record(D, p, M.lam[0], M.lam[1], M.lam[2]);
+            D.logz_in[p] = shift0;
+            D.logz[p] = M.logz;
+        } else if (D.insert_mode && cnt > 0) {
+            D.lme_fail[p] = 1;          // node insertion follows (lambda keeps the warm start)
+            atomicAdd(D.n_fail, 1);
+        } else {
+            raise_error(D.err, st, D.mgid[p]);
+        }
+    }
+    return st == OTM_OK;
+}
+
+// N_a = w_a / Z and grad N_a = -N_a J^-1 d_a = -K e_a with e_a = N_a d_a and K = J^-1 = Z J'^-1
+// (one symmetric 3x3 per MP). The pair rows keep (N_a, e_a) and the MP keeps K: whoever needs
+// grad N applies K once per MP (the kinematics gather sums du_a (x) e_a, and dF = 1 - G K
+// follows in the return map), so the per-pair work is N, e and the contributions.
+// Eq. 5 contributions of the next step, stored at the pair's place in its node's influence
+// list: mass m_p N_a, force -v_p sigma_p grad N_a = (v_p sigma_p K) e_a = Q e_a.
+__device__ __forceinline__ void lme_force_matrix(const Dev &D, int64_t p, const MpNewton &M, int lane, double (&Q)[9])
+{
+    const double vp = D.vol[p];
+    const double *sg = D.sig + 6 * p;
+    double Kc[6];
+    // lanes 0-5 form K (and store it), lanes 0-8 one entry of Q each; all lanes get both
+    const double kj = (lane < 6) ? M.inv[lane] * M.C[0] : 0.0;
+    if (lane < 6) D.Kinv[6 * p + lane] = kj;
+#pragma unroll
+    for (int i = 0; i < 6; i++) Kc[i] = __shfl_sync(0xffffffffu, kj, i);
+    // symmetric index of (i, j) in (xx, yy, zz, xy, yz, xz)
+    const int li = (lane < 9) ? lane / 3 : 0, lc = (lane < 9) ? lane % 3 : 0;
+    auto sym = [](int i, int j) { return i == j ? i : (i + j == 1 ? 3 : (i + j == 3 ? 4 : 5)); };
+    const double q = vp * (sg[sym(li, 0)] * Kc[sym(0, lc)] + sg[sym(li, 1)] * Kc[sym(1, lc)] +
+                           sg[sym(li, 2)] * Kc[sym(2, lc)]);
+#pragma unroll
+    for (int i = 0; i < 9; i++) Q[i] = __shfl_sync(0xffffffffu, q, i);
+}
+
+// stabilisation (Eq. 7-8): -eps N_a e_a / |x_a,n-1 - x_p,n-1|,
+// e_a = x_a - x_p - dF (x_a,n-1 - x_p,n-1), with dF the increment that led to this state
+template <bool STAB>
+struct LmeStab {
+    __device__ __forceinline__ void load(const Dev &, int64_t) {}
+    __device__ __forceinline__ void term(const Dev &, int, double, double, double, double, double &, double &, double &) const {}
+};
+
+template <>
+struct LmeStab<true> {
+    double xq0, xq1, xq2, F[9];
+    __device__ __forceinline__ void load(const Dev &D, int64_t p)
+    {
+        const double4_32a q = D.xp_prev[p];
+        xq0 = q.x; xq1 = q.y; xq2 = q.z;
+#pragma unroll
+        for (int i = 0; i < 9; i++) F[i] = D.dF[9 * p + i];
+    }
+    // (x, y, z) = x_p - x_a
+    __device__ __forceinline__ void term(const Dev &D, int id, double N, double x, double y, double z, double &sx,
+                                         double &sy, double &sz) const
+    {
+        const double4_32a a = D.x_prev[id];
+        const double q0 = a.x - xq0, q1 = a.y - xq1, q2 = a.z - xq2;
+        const double len = sqrt(q0 * q0 + q1 * q1 + q2 * q2);
+        if (len > 1e-12 * D.h) {
+            const double c = -D.eps_stab * N / len;
+            sx = c * (-x - (F[0] * q0 + F[1] * q1 + F[2] * q2));
+            sy = c * (-y - (F[3] * q0 + F[4] * q1 + F[5] * q2));
+            sz = c * (-z - (F[6] * q0 + F[7] * q1 + F[8] * q2));
+        }
+    }
+};
 
 // The LME solve of the block's MPs (one per warp; p the warp's MP, active whether it has one),
 // shared-memory rows of `rows` slots. Every thread of the block calls it (block barriers inside);
@@ -1028,24 +1141,7 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
             W.q[k] = fma(-beta_s, fma(z, z, fma(y, y, x * x)), -shift_s);
         }
         if (lane == 0) {
-            // Eq. 14: the warm start is the previous step's lambda, or (within a step) the cubic
-            // through the last four solutions: while the material deforms smoothly one Newton
-            // step from it meets the tolerance
-            double l0 = D.lam[3 * p], l1 = D.lam[3 * p + 1], l2 = D.lam[3 * p + 2];
-            if (D.lme_mode == kLmeStep) {
-                // cubic: 4 l_n - 6 l_{n-1} + 4 l_{n-2} - l_{n-3}
-                const double *a1 = D.lam_prev + 3 * p, *a2 = D.lam_prev2 + 3 * p, *a3 = D.lam_prev3 + 3 * p;
-                l0 = fma(4.0, l0 + a2[0], -fma(6.0, a1[0], a3[0]));
-                l1 = fma(4.0, l1 + a2[1], -fma(6.0, a1[1], a3[1]));
-                l2 = fma(4.0, l2 + a2[2], -fma(6.0, a1[2], a3[2]));
-            }
-            M.trial[0] = M.ws[0] = l0;
-            M.trial[1] = M.ws[1] = l1;
-            M.trial[2] = M.ws[2] = l2;
-            M.t = 1.0;
-            M.have_cur = M.iters = M.iters_total = M.halvings = M.retried = 0;
-            M.shift0 = shift0;
-            newton_set_trial(M);
+            lme_start(D, p, M, shift0);
             M.state = cnt > 0 ? kNewtonEval : kNewtonFail;
         }
     } else if (lane == 0) {
@@ -1061,70 +1157,24 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
         __syncthreads();
         bool pending = false;
         if (warp == 0 && lane < kLmeWarps) {
-            newton_round(NS[lane], D.tol_abs, D.max_newton);
+            newton_round<MIXED ? 0 : 2>(NS[lane], D.tol_abs, D.max_newton);
             pending = NS[lane].state == kNewtonEval;
         }
         if (!__syncthreads_or(pending)) break;
     }
     if (!active) return;
-    const int st = M.state == kNewtonDone ? OTM_OK : OTM_ERR_LME_NOCONV;
-    if (lane == 0) {
-        D.newton_it[p] = M.iters_total;
-        if (st == OTM_OK) {
-            lme_record(D, p, M.lam[0], M.lam[1], M.lam[2]);
-            D.logz_in[p] = shift0;
-            D.logz[p] = M.logz;
-        } else if (D.insert_mode && cnt > 0) {
-            D.lme_fail[p] = 1;          // node insertion follows (lambda keeps the warm start)
-            atomicAdd(D.n_fail, 1);
-        } else {
-            raise_error(D.err, st, D.mgid[p]);
-        }
-    }
-    double inv[6];
-    for (int i = 0; i < 6; i++) inv[i] = M.inv[i];
-    const double iZ = M.iZ;
-    if (st != OTM_OK) return;
+    if (!lme_finish(D, p, cnt, M, shift0, lane)) return;
 
-    // N_a = w_a / Z and grad N_a = -N_a J^-1 d_a = -K e_a with e_a = N_a d_a and K = J^-1 = Z J'^-1
-    // (one symmetric 3x3 per MP). The pair rows keep (N_a, e_a) and the MP keeps K: whoever needs
-    // grad N applies K once per MP (the kinematics gather sums du_a (x) e_a, and dF = 1 - G K
-    // follows in the return map), so the per-pair work here is N, e and the contributions.
-    // Eq. 5 contributions of the next step, stored at the pair's place in its node's influence
-    // list: mass m_p N_a, force -v_p sigma_p grad N_a = (v_p sigma_p K) e_a = Q e_a.
-    const double mp = D.mass[p], vp = D.vol[p];
-    const double *sg = D.sig + 6 * p;
-    double Kc[6], Q[9];
-    {
-        // lanes 0-5 form K (and store it), lanes 0-8 one entry of Q each; all lanes get both
-        const double Zc = M.C[0];
-        const double kj = (lane < 6) ? inv[lane] * Zc : 0.0;
-        if (lane < 6) D.Kinv[6 * p + lane] = kj;
-#pragma unroll
-        for (int i = 0; i < 6; i++) Kc[i] = __shfl_sync(0xffffffffu, kj, i);
-        // symmetric index of (i, j) in (xx, yy, zz, xy, yz, xz)
-        const int li = (lane < 9) ? lane / 3 : 0, lc = (lane < 9) ? lane % 3 : 0;
-        auto sym = [](int i, int j) { return i == j ? i : (i + j == 1 ? 3 : (i + j == 3 ? 4 : 5)); };
-        const double q = vp * (sg[sym(li, 0)] * Kc[sym(0, lc)] + sg[sym(li, 1)] * Kc[sym(1, lc)] +
-                               sg[sym(li, 2)] * Kc[sym(2, lc)]);
-#pragma unroll
-        for (int i = 0; i < 9; i++) Q[i] = __shfl_sync(0xffffffffu, q, i);
-    }
+    const double iZ = M.iZ, mp = D.mass[p];
+    double Q[9];
+    lme_force_matrix(D, p, M, lane, Q);
     int em = -2000, ef = -2000;   // largest binary exponents of the stored mass / force terms
     float Qf[9];
 #pragma unroll
     for (int i = 0; i < 9; i++) Qf[i] = MIXED ? (float)Q[i] : 0.f;
     const float mpf = MIXED ? (float)mp : 0.f;
-    // stabilisation (Eq. 7-8): -eps N_a e_a / |x_a,n-1 - x_p,n-1|,
-    // e_a = x_a - x_p - dF (x_a,n-1 - x_p,n-1), with dF the increment that led to this state
-    double xq0 = 0, xq1 = 0, xq2 = 0, F00 = 0, F01 = 0, F02 = 0, F10 = 0, F11 = 0, F12 = 0, F20 = 0, F21 = 0, F22 = 0;
-    if (STAB) {
-        const double4_32a q = D.xp_prev[p];
-        xq0 = q.x; xq1 = q.y; xq2 = q.z;
-        const double *Fd = D.dF + 9 * p;
-        F00 = Fd[0]; F01 = Fd[1]; F02 = Fd[2]; F10 = Fd[3]; F11 = Fd[4]; F12 = Fd[5]; F20 = Fd[6]; F21 = Fd[7];
-        F22 = Fd[8];
-    }
+    LmeStab<STAB> stab;
+    stab.load(D, p);
     for (int k = lane; k < cnt; k += kWarp) {
         const double wk = W.w[k];
         const double N = wk * iZ;
@@ -1146,17 +1196,7 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
         const int id = D.ids[base + k];
         const int64_t pos = (int64_t)D.noff[id] + D.rank[base + k];
         double sx = 0.0, sy = 0.0, sz = 0.0;
-        if (STAB) {
-            const double4_32a a = D.x_prev[id];
-            const double q0 = a.x - xq0, q1 = a.y - xq1, q2 = a.z - xq2;
-            const double len = sqrt(q0 * q0 + q1 * q1 + q2 * q2);
-            if (len > 1e-12 * D.h) {
-                const double c = -D.eps_stab * N / len;
-                sx = c * (-x - (F00 * q0 + F01 * q1 + F02 * q2));
-                sy = c * (-y - (F10 * q0 + F11 * q1 + F12 * q2));
-                sz = c * (-z - (F20 * q0 + F21 * q1 + F22 * q2));
-            }
-        }
+        stab.term(D, id, N, x, y, z, sx, sy, sz);
         if (MIXED) {
             const float c0 = mpf * fN;
             float c1 = fmaf(Qf[2], fez, fmaf(Qf[1], fey, Qf[0] * fex));
@@ -1222,25 +1262,503 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp) k_lme_wide(const Dev D)
     }
 }
 
+// ======================================================================== k_lme_fix
+// The LME solve with fixed-point evaluations (otm_fix.cuh): same block structure, Newton decisions and
+// outputs as k_lme, but the pair loops run in integers, so the FP64 pipe (2 lanes per clock and SM)
+// only sees the scalars and the force contributions.
+//
+// Bound: k_lme keeps the FP64 pipe 89 % busy (19 FP64 instructions a pair and evaluation). Here it is
+// 47 % busy (11 a pair for the force contributions and N, plus the rounds' scalars), and the integer
+// instructions (about 200 a pair and evaluation, two to four cycles of an SM quarter each) and their
+// latency at 16 warps an SM (128 registers; four blocks of 54 KB) bound the kernel.
+// Measured on the 202,752-MP rod (267 pairs an MP, 1.19 Newton iterations): k_lme 7.78 ms, this kernel
+// 2.96 ms (with k_lme_prep). Five blocks an SM (96 registers, the exp table in L1) take 3.40 ms: spills.
+struct MpFix {
+    i64 xp[3];         // X of the material point
+    i64 v[3];          // centre offset of the pending trial, lambda / (2 beta) in LSB
+    i64 cst;           // the trial's exponent constant, 46 fraction bits
+    i64 ok;            // the trial is inside the fixed-point range
+};
+static_assert(2 * kExpTable / kLmeWarps >= kLmeRows, "the exp table holds the warps' pair positions");
+static_assert(sizeof(FixStart) == 3 * sizeof(double) + sizeof(MpFix) + 8, "k_lme_fix copies FixStart word by word");
+
+// centre offset and constant of a trial with a shift; false out of range (or not finite): FP64 evaluation
+__device__ __forceinline__ bool fix_trial(const FixConst &C, const double *trial, double sh, i64 *v, i64 &cst)
+{
+    bool ok = true;
+    double l2 = 0.0;
+    for (int i = 0; i < 3; i++) {
+        const double x = trial[i] * C.i2b;
+        l2 = fma(trial[i], trial[i], l2);
+        ok = ok && fabs(x) < C.vmax;
+        v[i] = __double2ll_rn(x);
+    }
+    const double c = fma(l2, C.cy, -sh * kFixYScale);
+    cst = __double2ll_rn(c * kFixYOne);
+    return ok && fabs(c) < 65536.0;
+}
+
+// 1/x (x positive and normal): the hardware's approximate FP64 reciprocal (about 20 bits), refined by
+// STEPS Newton steps y += y (1 - x y), each of which doubles the bits. The division operator takes
+// about twice the FP64 instructions.
+template <int STEPS>
+__device__ __forceinline__ double recip(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+#pragma unroll
+    for (int i = 0; i < STEPS; i++) y = fma(y, fma(-x, y, 1.0), y);
+    return y;
+}
+
+// One scalar round after the block's evaluations (the damped Newton of newton_round), for the block's
+// kLmeWarps MPs at once by one warp, eight lanes per MP: the entries of J', of its cofactors and of
+// the step go to one lane each, so that a round takes about 45 FP64 instructions instead of 85 (an
+// FP64 instruction costs the pipe 16 cycles with one active lane as with 32). Halvings, failures and the
+// cold-start retry (rare) run on the group's first lane. Returns whether this lane's MP has an
+// evaluation pending.
+__device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixConst &C, double tol, int max_it, int lane)
+{
+    const int q = lane & 7, gb = lane & 24;
+    MpNewton &m = NS[lane >> 3];
+    MpFix &f = FS[lane >> 3];
+    const bool act = m.state == kNewtonEval;
+    if (!__any_sync(0xffffffffu, act)) return false;
+    auto from = [&](double v, int src) { return __shfl_sync(0xffffffffu, v, gb + src); };
+    auto nib = [&](unsigned tab) { return (int)((tab >> (4 * q)) & 7u); };   // lane q's entry of a table
+    const double Z = m.E[0], r0 = m.E[1], r1 = m.E[2], r2 = m.E[3];
+    const double rn = fma(r2, r2, fma(r1, r1, r0 * r0));
+    bool accept = act;
+    if (act && m.have_cur) {   // accept if log Z or the residual norm drops, else halve
+        const double cZ = m.C[0], c0 = m.C[1], c1 = m.C[2], c2 = m.C[3];
+        const double cn = fma(c2, c2, fma(c1, c1, c0 * c0));
+        const bool less = m.E[10] == m.C[10] ? Z < cZ : m.E[10] + log(Z) < m.C[10] + log(cZ);
+        accept = isfinite(Z) && (less || rn * (cZ * cZ) < cn * (Z * Z));
+    }
+    const bool finite = isfinite(rn) && isfinite(Z);
+    const bool conv = accept && finite && rn <= tol * tol * Z * Z;
+    const bool newton = accept && finite && !conv && m.iters < max_it;
+    // J' = A - r r^T / Z at the accepted point, lane q its entry (xx, yy, zz, xy, yz, xz); r r^T / Z is
+    // second order in the residual, so the approximate 1/Z does
+    const double iZ = recip<0>(Z);
+    const int ei = nib(0x010210), ej = nib(0x221210);
+    const double ri = ei == 0 ? r0 : (ei == 1 ? r1 : r2), rj = ej == 0 ? r0 : (ej == 1 ? r1 : r2);
+    const double J = q < 6 ? fma(-(ri * iZ), rj, m.E[4 + q]) : 0.0;
+    // cofactors, same order: J[p1] J[p2] - J[p3] J[p4]
+    const double cf = from(J, nib(0x335001)) * from(J, nib(0x454122)) - from(J, nib(0x503354)) * from(J, nib(0x142354));
+    const double det = fma(from(J, 5), from(cf, 5), fma(from(J, 3), from(cf, 3), from(J, 0) * from(cf, 0)));
+    const bool regular = det > 0.0 && isfinite(det);
+    const double inv = cf * recip<3>(det);
+    // the step -J'^-1 r, lane q < 3 its component, and the next trial
+    const double step = -fma(from(inv, nib(0x245)), r2, fma(from(inv, nib(0x413)), r1, from(inv, nib(0x530)) * r0));
+    const double lam = q < 3 ? m.trial[q] : 0.0;
+    const double trial = lam + step;
+    const double t0 = from(trial, 0), t1 = from(trial, 1), t2 = from(trial, 2);
+    const double l2 = fma(t2, t2, fma(t1, t1, t0 * t0)), v = trial * C.i2b;
+    const double sh = m.E[10], c = fma(l2, C.cy, -sh * kFixYScale);
+    const unsigned inside = __ballot_sync(0xffffffffu, q >= 3 || fabs(v) < C.vmax);
+    __syncwarp();
+    const bool finish = conv && regular, next = newton && regular;
+    if (accept) {
+        m.C[q] = m.E[q];
+        if (q < 3) {
+            m.C[8 + q] = m.E[8 + q];
+            m.lam[q] = lam;
+        }
+    }
+    if (next) {
+        if (q < 3) {
+            m.dir[q] = step;
+            m.trial[q] = trial;
+            f.v[q] = __double2ll_rn(v);
+        }
+        if (q == 0) {
+            m.t = 1.0;
+            m.sh = sh;
+            m.have_cur = 1;
+            m.halvings = 0;
+            m.iters++;
+            m.iters_total++;
+            f.cst = __double2ll_rn(c * kFixYOne);
+            f.ok = ((inside >> gb) & 0xffu) == 0xffu && fabs(c) < 65536.0;
+        }
+    } else if (finish) {
+        if (q < 6) m.inv[q] = inv;
+        if (q == 0) {
+            m.have_cur = 1;
+            m.iZ = recip<3>(Z);
+            // the next solve's shift: its Z then starts in [1/4, 1/2) (see newton_finish)
+            const int ez = ((__double2hiint(Z) >> 20) & 0x7ff) - 1023;
+            m.logz = fma((double)(ez + 2), 0x1.62e42fefa39efp-1, sh);
+            m.state = kNewtonDone;
+        }
+    } else if (act && q == 0) {
+        if (accept) {
+            m.have_cur = 1;
+            newton_fail(m);
+        } else if (++m.halvings >= 40) {
+            newton_fail(m);
+        } else {
+            m.t *= 0.5;
+            for (int i = 0; i < 3; i++) m.trial[i] = fma(m.t, m.dir[i], m.lam[i]);
+            newton_set_trial(m);
+        }
+        if (m.state == kNewtonEval) f.ok = fix_trial(C, m.trial, m.sh, f.v, f.cst) ? 1 : 0;
+    }
+    __syncwarp();
+    return m.state == kNewtonEval;
+}
+
+// shared-memory rows of one warp: the support nodes' X and the weights of the last evaluation (FP64 bits)
+struct FixSmem {
+    i64 x0[kLmeRows], x1[kLmeRows], x2[kLmeRows];
+    double w[kLmeRows];
+};
+
+// One evaluation in fixed point at the pending trial: weights into F.w, the sums into m.E. False if the
+// weights leave the window (a weight of 1 or more, Z outside [2^-11, 1), A too large): the caller then
+// evaluates in FP64. A function of the trial and the shift alone, so a restored state repeats it bit
+// for bit. Warp-uniform.
+template <bool LOLO>
+__device__ __forceinline__ bool lme_eval_fix(const FixConst &C, FixSmem &F, int n, MpNewton &m, const MpFix &f,
+                                             int lane, const u64 *T)
+{
+    FixSums s;
+    fix_sums_zero(s);
+    {
+        const i64 c0 = f.xp[0] - f.v[0], c1 = f.xp[1] - f.v[1], c2 = f.xp[2] - f.v[2], cst = f.cst;
+        const u64 bq = C.bq;
+#pragma unroll 1
+        for (int k = lane; k < n; k += kWarp)
+            F.w[k] = fix_pair<LOLO>(F.x0[k], F.x1[k], F.x2[k], c0, c1, c2, cst, bq, T, s);
+    }
+    const uint32_t tr = fix_trace(s);
+    if (__any_sync(0xffffffffu, s.top >= 0 || s.zc >= (1u << 26) || tr >= (1u << 30))) return false;
+    const uint32_t zs = __reduce_add_sync(0xffffffffu, s.zc), ts = __reduce_add_sync(0xffffffffu, tr >> 5);
+    if (zs < (1u << 15) || zs >= (1u << 26) - 1024u || ts >= (kFixTraceMax >> 5) - 64u) return false;
+    i64 v[10];
+    fix_combine(s, v);
+    i64 t = warp_reduce_scatter10(v, lane);
+    const i64 Z = __shfl_sync(0xffffffffu, t, 0);
+    const i64 r0 = __shfl_sync(0xffffffffu, t, 2), r1 = __shfl_sync(0xffffffffu, t, 4), r2 = __shfl_sync(0xffffffffu, t, 8);
+    // sums 1-3 are r, 4-9 A (00, 11, 22, 01, 12, 02): moved from the centre to the material point
+    const int j = rs10_value(lane);
+    const int a = j < 4 ? 0 : (j < 7 ? j - 4 : (j == 8 ? 1 : 0));
+    const int b = j < 4 ? (j > 0 ? j - 1 : 0) : (j < 7 ? j - 4 : (j == 7 ? 1 : 2));
+    const i64 ra = a == 0 ? r0 : (a == 1 ? r1 : r2), vb = f.v[b];
+    const i64 rd = fix_r_about(Z, b == 0 ? r0 : (b == 1 ? r1 : r2), vb);
+    if (j >= 4) t = fix_a_about(t, ra, rd, f.v[a], vb);
+    else if (j >= 1) t = rd;
+    const double d = (double)t * (j == 0 ? 0x1p-63 : (j < 4 ? C.r_unit : C.a_unit));
+    if (rs10_writer(lane)) m.E[j] = d;
+    if (lane == 0) m.E[10] = m.sh;
+    return true;
+}
+
+// the same evaluation in FP64, for trials outside the fixed-point range: coordinates from global
+// memory, shift handling as lme_eval_block
+__device__ __noinline__ void lme_eval64(const double4_32a *x, const int32_t *ids, double4_32a xp, double beta_s, double *w,
+                                        int n, MpNewton &m, int lane)
+{
+    const double s0 = m.trial[0] * kExpScale, s1 = m.trial[1] * kExpScale, s2 = m.trial[2] * kExpScale;
+    double sh = m.sh, v[10], t = 0.0;
+    for (int pass = 0; pass < 2; pass++) {
+        const double sh_s = sh * kExpScale;
+#pragma unroll
+        for (int i = 0; i < 10; i++) v[i] = 0.0;
+        for (int k = lane; k < n; k += kWarp) {
+            const double4_32a a = x[ids[k]];
+            const double dx = xp.x - a.x, dy = xp.y - a.y, dz = xp.z - a.z;
+            const double q = fma(-beta_s, fma(dz, dz, fma(dy, dy, dx * dx)), -sh_s);
+            const double wk = exp_scaled(fma(s2, dz, fma(s1, dy, fma(s0, dx, q))), g_exp2_table);
+            w[k] = wk;
+            const double wx = wk * dx, wy = wk * dy, wz = wk * dz;
+            v[0] += wk;
+            v[1] += wx; v[2] += wy; v[3] += wz;
+            v[4] = fma(wx, dx, v[4]); v[5] = fma(wy, dy, v[5]); v[6] = fma(wz, dz, v[6]);
+            v[7] = fma(wx, dy, v[7]); v[8] = fma(wy, dz, v[8]); v[9] = fma(wx, dz, v[9]);
+        }
+        t = warp_reduce_scatter10(v, lane);
+        const double Z = __shfl_sync(0xffffffffu, t, 0);
+        if (pass == 1 || (Z > 1e-200 && Z < 1e200)) break;
+        double mx = -INFINITY;   // over- or underflow: once more with the largest exponent as the shift
+        for (int k = lane; k < n; k += kWarp) {
+            const double4_32a a = x[ids[k]];
+            const double dx = xp.x - a.x, dy = xp.y - a.y, dz = xp.z - a.z;
+            mx = fmax(mx, fma(s2, dz, fma(s1, dy, s0 * dx)) - beta_s * fma(dz, dz, fma(dy, dy, dx * dx)));
+        }
+        sh = warp_max(mx) * (1.0 / kExpScale);
+    }
+    if (rs10_writer(lane)) m.E[rs10_value(lane)] = t;
+    if (lane == 0) m.E[10] = sh;
+}
+
+// shared memory of one block: the exp table, the warps' rows (a compile-time stride, so that a slot's four
+// words share one address register) and the solves' states
+struct FixBlock {
+    u64 table[kExpTable];
+    FixSmem rows[kLmeWarps];
+    MpNewton newton[kLmeWarps];
+    MpFix fix[kLmeWarps];
+};
+
+template <bool MIXED, bool STAB>
+__global__ void __launch_bounds__(kLmeWarps * kWarp, 4) k_lme_fix(const __grid_constant__ Dev D)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t p = (int64_t)blockIdx.x * kLmeWarps + warp;
+    const int rows = lme_rows(D.S), S = D.S;
+    const FixConst &C = D.fix;
+    FixBlock &B = *(FixBlock *)smem_raw;
+    u64 *T = B.table;
+    for (int j = threadIdx.x; j < kExpTable; j += kLmeWarps * kWarp) T[j] = g_exp2_mant[j];
+    FixSmem &F = B.rows[warp];
+    MpNewton &M = B.newton[warp];
+    MpFix &X = B.fix[warp];
+    bool active = (p < D.nm) && !has_error(D.err);
+    if (active && D.cnt[p] > rows) {   // solved by k_lme_wide
+        if (lane == 0) D.lme_defer[atomicAdd(D.n_defer, 1)] = (int32_t)p;
+        active = false;
+    }
+    const int64_t base = p * (int64_t)S;
+    int cnt = 0;
+    double shift0 = 0;
+    if (active) {
+        cnt = D.cnt[p];
+        shift0 = D.logz[p];
+        for (int k = lane; k < cnt; k += kWarp) {
+            const longlong4_32a a = D.xfix[D.ids[base + k]];
+            F.x0[k] = a.x; F.x1[k] = a.y; F.x2[k] = a.z;
+        }
+        if (lane < 11) {   // the start formed by k_lme_prep
+            const i64 v = ((const i64 *)&D.fstart[p])[lane];
+            if (lane < 3) M.trial[lane] = M.ws[lane] = fx_bits_d((u64)v);
+            else ((i64 *)&X)[lane - 3] = v;
+        }
+        if (lane == 0) {
+            M.t = 1.0;
+            M.have_cur = M.iters = M.iters_total = M.halvings = M.retried = 0;
+            M.shift0 = M.sh = shift0;
+            M.state = cnt > 0 ? kNewtonEval : kNewtonFail;
+        }
+    } else if (lane == 0) {
+        M.state = kNewtonIdle;
+    }
+    __syncthreads();
+    for (;;) {
+        if (M.state == kNewtonEval) {
+            __syncwarp();
+            if (!(X.ok && lme_eval_fix<!MIXED>(C, F, cnt, M, X, lane, T)))
+                lme_eval64(D.x, D.ids + base, D.xp[p], D.beta * kExpScale, F.w, cnt, M, lane);
+        }
+        __syncthreads();
+        const bool pending = warp == 0 && fix_round(B.newton, B.fix, C, D.tol_abs, D.max_newton, lane);
+        if (!__syncthreads_or(pending)) break;
+    }
+    if (!active) return;
+    if (!lme_finish(D, p, cnt, M, shift0, lane)) return;
+    // the pairs' node-major positions hang on two dependent loads: gathered ahead of the output loop, four
+    // passes in flight, into this warp's share of the exp table (every warp of the block is past its
+    // last evaluation)
+    int32_t *pos = (int32_t *)B.table + warp * (2 * kExpTable / kLmeWarps);
+    for (int k0 = lane; k0 < cnt; k0 += 4 * kWarp) {
+        int id[4], r[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int k = k0 + j * kWarp;
+            id[j] = k < cnt ? D.ids[base + k] : 0;
+            r[j] = k < cnt ? D.rank[base + k] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) r[j] += D.noff[id[j]];
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            if (k0 + j * kWarp < cnt) pos[k0 + j * kWarp] = r[j];
+    }
+    const double iZ = M.iZ, mp = D.mass[p];
+    double Q[9];
+    lme_force_matrix(D, p, M, lane, Q);
+    const i64 xp0 = X.xp[0], xp1 = X.xp[1], xp2 = X.xp[2];
+    const int fb = C.fb;
+    LmeStab<STAB> st;
+    st.load(D, p);
+    // largest magnitudes of the stored mass / force terms by their high words (exponents at the end)
+    unsigned hm = 0, hf = 0;
+#pragma unroll 1
+    for (int k = lane; k < cnt; k += kWarp) {
+        const double N = F.w[k] * iZ;
+        const i64 d0 = xp0 - F.x0[k], d1 = xp1 - F.x1[k], d2 = xp2 - F.x2[k];
+        double sx = 0.0, sy = 0.0, sz = 0.0;
+        if (STAB) {
+            const int id = D.ids[base + k];
+            const double4_32a a = D.x[id], xp = D.xp[p];
+            st.term(D, id, N, xp.x - a.x, xp.y - a.y, xp.z - a.z, sx, sy, sz);
+        }
+        if (MIXED) {
+            // e = N d in FP32 (every consumer of the mixed path's rows rounds them to FP32),
+            // stored widened exactly; N stays FP64
+            const float fN = f32_round_bits(N);
+            const float ex = fN * fix_to_float(d0, fb), ey = fN * fix_to_float(d1, fb), ez = fN * fix_to_float(d2, fb);
+            D.shape[base + k] = make_double4_32a(N, df_widen(ex), df_widen(ey), df_widen(ez));
+            const float c0 = (float)mp * fN;
+            float c1 = fmaf((float)Q[2], ez, fmaf((float)Q[1], ey, (float)Q[0] * ex));
+            float c2 = fmaf((float)Q[5], ez, fmaf((float)Q[4], ey, (float)Q[3] * ex));
+            float c3 = fmaf((float)Q[8], ez, fmaf((float)Q[7], ey, (float)Q[6] * ex));
+            if (STAB) {
+                c1 += f32_round_bits(sx);
+                c2 += f32_round_bits(sy);
+                c3 += f32_round_bits(sz);
+            }
+            D.contrib32[pos[k]] = make_float4(c0, c1, c2, c3);
+            hm = max(hm, __float_as_uint(c0) & 0x7fffffffu);
+            hf = max(max(hf, __float_as_uint(c1) & 0x7fffffffu),
+                     max(__float_as_uint(c2) & 0x7fffffffu, __float_as_uint(c3) & 0x7fffffffu));
+        } else {
+            double ex, ey, ez;
+            {
+                const u64 nb = fx_d_bits(N);
+                const u64 nm = ((nb & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
+                const int en = (int)(nb >> 52);
+                // a component within 2^-31 of the range (the last 32 bits of D), or N subnormal: FP64
+                const int least = min(min(abs((int)(d0 >> 32)), abs((int)(d1 >> 32))), abs((int)(d2 >> 32)));
+                if (least > 1 && en > 0) {
+                    ex = fix_mul_double(nm, en, d0, fb);
+                    ey = fix_mul_double(nm, en, d1, fb);
+                    ez = fix_mul_double(nm, en, d2, fb);
+                } else {
+                    const double Nu = N * C.r_unit;
+                    ex = Nu * (double)d0; ey = Nu * (double)d1; ez = Nu * (double)d2;
+                }
+            }
+            D.shape[base + k] = make_double4_32a(N, ex, ey, ez);
+            const double cm = mp * N;
+            double fx = Q[0] * ex + Q[1] * ey + Q[2] * ez;
+            double fy = Q[3] * ex + Q[4] * ey + Q[5] * ez;
+            double fz = Q[6] * ex + Q[7] * ey + Q[8] * ez;
+            if (STAB) {
+                fx += sx;
+                fy += sy;
+                fz += sz;
+            }
+            D.contrib64[pos[k]] = make_double4_32a(cm, fx, fy, fz);
+            hm = max(hm, (unsigned)__double2hiint(cm) & 0x7fffffffu);
+            hf = max(max(hf, (unsigned)__double2hiint(fx) & 0x7fffffffu),
+                     max((unsigned)__double2hiint(fy) & 0x7fffffffu, (unsigned)__double2hiint(fz) & 0x7fffffffu));
+        }
+    }
+    hm = __reduce_max_sync(0xffffffffu, hm);
+    hf = __reduce_max_sync(0xffffffffu, hf);
+    if (lane == 0) {
+        // binary exponents; zero and subnormal terms count as -2000
+        const int sft = MIXED ? 23 : 20, bias = MIXED ? 127 : 1023;
+        atomicMax(&D.emax[0], (hm >> sft) ? (int)(hm >> sft) - bias : -2000);
+        atomicMax(&D.emax[1], (hf >> sft) ? (int)(hf >> sft) - bias : -2000);
+    }
+}
+
+// Before k_lme_fix: the nodes' fixed-point coordinates, the empty list of deferred MPs and, one thread
+// per MP, the start of each solve (warm start, its centre and constant): about 30 FP64 instructions
+// that would cost 16 cycles each in the MP's own warp and cost half a cycle a lane here.
+__global__ void __launch_bounds__(256) k_lme_prep(const __grid_constant__ Dev D)
+{
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    const FixConst &C = D.fix;
+    if (t0 == 0) *D.n_defer = 0;
+    for (int64_t i = t0; i < D.nn; i += nt) {
+        const double4_32a a = D.x[i];
+        longlong4_32a f;
+        f.x = fix_from_double(a.x, C.fb);
+        f.y = fix_from_double(a.y, C.fb);
+        f.z = fix_from_double(a.z, C.fb);
+        f.w = 0;
+        D.xfix[i] = f;
+    }
+    for (int64_t p = t0; p < D.nm; p += nt) {
+        // Eq. 14: the warm start is the previous step's lambda, or (within a step) the cubic through the
+        // last four solutions, 4 l_n - 6 l_{n-1} + 4 l_{n-2} - l_{n-3}
+        FixStart s;
+        for (int i = 0; i < 3; i++) {
+            double l = D.lam[3 * p + i];
+            if (D.lme_mode == kLmeStep)
+                l = fma(4.0, l + D.lam_prev2[3 * p + i], -fma(6.0, D.lam_prev[3 * p + i], D.lam_prev3[3 * p + i]));
+            s.trial[i] = l;
+        }
+        const double4_32a x = D.xp[p];
+        s.xp[0] = fix_from_double(x.x, C.fb);
+        s.xp[1] = fix_from_double(x.y, C.fb);
+        s.xp[2] = fix_from_double(x.z, C.fb);
+        s.ok = fix_trial(C, s.trial, D.logz[p], s.v, s.cst) ? 1 : 0;
+        s.pad = 0;
+        D.fstart[p] = s;
+    }
+}
+
+// The fixed-point evaluation's constants: fb so that the support radius lies between 2^63/4.4 and
+// 2^63/2.2 LSB (a trial's centre may then move by 0.45 support radii or more per axis before it leaves
+// the range). Off where the exponent scale does not fit 64 bits (support tolerances below about
+// 2e-10) or for length scales outside the exponent arithmetic's range.
+FixConst make_fix_const(double beta, double rs2)
+{
+    FixConst c = {};
+    const double rs = std::sqrt(rs2);
+    int ex = 0;
+    std::frexp(2.2 * rs, &ex);                      // 2^63 LSB = 2^ex >= 2.2 rs
+    c.fb = 63 - ex;
+    const double a = std::ldexp(1.0, 32 - c.fb);
+    const long double bq = std::ldexp((long double)beta * 256.0L / std::log(2.0L) * a * a, 46 + 63);
+    c.on = std::isfinite((double)bq) && bq < 0x1p64L && bq >= 0x1p32L && c.fb > -60 && c.fb < 120;
+    if (!c.on) return c;
+    c.bq = (u64)bq;
+    c.i2b = std::ldexp(1.0, c.fb) / (2.0 * beta);
+    c.cy = 64.0 / (beta * std::log(2.0));
+    c.vmax = kFixT - std::ldexp(rs, c.fb) * (1.0 + 1e-9);
+    c.r_unit = std::ldexp(1.0, -c.fb);
+    c.a_unit = a * a / 16.0;
+    return c;
+}
+
 static size_t lme_block_smem(int rows)
 {
     return (size_t)kLmeWarps * 5 * (size_t)rows * sizeof(double) + (size_t)kLmeWarps * sizeof(MpNewton);
 }
 
+// Which kernel (D.lme_fix, set by the step driver): the fixed-point one for the FP64 path's solves where
+// its exponent range covers the problem (fix.on), and for regenerating the shape functions of a state
+// that such a solve left, in either path. The mixed path's own solves keep k_lme: its FP32 increments
+// turn a last-bit change of N into an FP32 ulp of a node's increment (1e-7 of the stress it leads to),
+// so that recorded mixed runs would not be reproduced.
 template <bool MIXED, bool STAB>
-static cudaError_t launch_lme_t(const Dev &D, cudaStream_t s, unsigned blocks)
+static cudaError_t launch_lme_t(const Dev &D, cudaStream_t s, unsigned blocks, long long *launches)
 {
-    const size_t smem = lme_block_smem(lme_rows(D.S)), smem_wide = lme_block_smem(D.S);
-    cudaError_t e = cudaFuncSetAttribute(k_lme<MIXED, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_lme_wide<MIXED, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_wide);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(D.n_defer, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess) return e;
-    k_lme<MIXED, STAB><<<blocks, kLmeWarps * kWarp, smem, s>>>(D);
-    // one persistent round of blocks over the deferred MPs (none on most steps: the launch then
-    // returns at once)
-    k_lme_wide<MIXED, STAB><<<152 * 3, kLmeWarps * kWarp, smem_wide, s>>>(D);
+    cudaError_t e;
+    if (D.lme_fix) {
+        const size_t smem = sizeof(FixBlock);
+        e = cudaFuncSetAttribute(k_lme_fix<MIXED, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        int64_t pb = ((D.nn > D.nm ? D.nn : D.nm) + 255) / 256;
+        if (pb > 152 * 8) pb = 152 * 8;
+        k_lme_prep<<<(unsigned)pb, 256, 0, s>>>(D);
+        k_lme_fix<MIXED, STAB><<<blocks, kLmeWarps * kWarp, smem, s>>>(D);
+        if (launches) *launches += 2;
+    } else {
+        const size_t smem = lme_block_smem(lme_rows(D.S));
+        e = cudaFuncSetAttribute(k_lme<MIXED, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        e = cudaMemsetAsync(D.n_defer, 0, sizeof(int32_t), s);
+        if (e != cudaSuccess) return e;
+        k_lme<MIXED, STAB><<<blocks, kLmeWarps * kWarp, smem, s>>>(D);
+        if (launches) *launches += 1;
+    }
+    if (D.S > kLmeRows) {
+        // one persistent round of blocks over the deferred MPs (none on most steps: the launch then
+        // returns at once)
+        const size_t smem = lme_block_smem(D.S);
+        e = cudaFuncSetAttribute(k_lme_wide<MIXED, STAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k_lme_wide<MIXED, STAB><<<152 * 3, kLmeWarps * kWarp, smem, s>>>(D);
+        if (launches) *launches += 1;
+    }
     return cudaGetLastError();
 }
 
@@ -1249,10 +1767,9 @@ cudaError_t launch_lme(const Dev &D, cudaStream_t s, long long *launches)
     const unsigned blocks = (unsigned)((D.nm + kLmeWarps - 1) / kLmeWarps);
     if (blocks == 0) return cudaSuccess;
     const bool mixed = D.precision == OTM_PRECISION_MIXED, stab = D.eps_stab > 0.0;
-    cudaError_t e = mixed ? (stab ? launch_lme_t<true, true>(D, s, blocks) : launch_lme_t<true, false>(D, s, blocks))
-                          : (stab ? launch_lme_t<false, true>(D, s, blocks) : launch_lme_t<false, false>(D, s, blocks));
-    if (launches) *launches += 2;
-    return e;
+    return mixed ? (stab ? launch_lme_t<true, true>(D, s, blocks, launches) : launch_lme_t<true, false>(D, s, blocks, launches))
+                 : (stab ? launch_lme_t<false, true>(D, s, blocks, launches)
+                         : launch_lme_t<false, false>(D, s, blocks, launches));
 }
 
 // (N, grad N) of every slot of a padded row set, for state export: already stored in shape[]

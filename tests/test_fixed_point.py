@@ -1,0 +1,135 @@
+"""The fixed-point arithmetic of the FP64 path's LME evaluation (csrc/otm_fix.cuh), compiled for the host
+and checked against 60-digit decimal arithmetic: exponent, weights, the sums Z, r, A and N d."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+from decimal import Decimal, getcontext
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2206_08772_gb300", "csrc")
+
+SRC = r'''
+#include <cmath>
+#include <cstdlib>
+#include <vector>
+#include "otm_fix.cuh"
+using namespace otm;
+// the sums of one evaluation (32 lanes) as the kernel forms them; out: Z, r, A in physical units, then the
+// weights; prod: N d; returns 0, 1 centre out of range, 2 weights out of the window
+extern "C" int eval(int n, const double *x, const double *xp, const double *lam, double beta, double shift, int fb,
+                    const u64 *table, u64 bq, double *out, double *w, double *prod)
+{
+    std::vector<i64> X(3 * n);
+    for (int k = 0; k < 3 * n; k++) X[k] = fix_from_double(x[k], fb);
+    i64 P[3], v[3];
+    double l2 = 0;
+    for (int i = 0; i < 3; i++) {
+        P[i] = fix_from_double(xp[i], fb);
+        const double c = lam[i] * std::ldexp(1.0, fb) / (2 * beta);
+        if (!(std::fabs(c) < kFixT)) return 1;
+        v[i] = std::llrint(c);
+        l2 += lam[i] * lam[i];
+    }
+    const i64 cst = std::llrint((l2 * 64.0 / (beta * std::log(2.0)) - shift * kFixYScale) * kFixYOne);
+    i64 t[10] = {0};
+    for (int lane = 0; lane < 32; lane++) {
+        FixSums s;
+        fix_sums_zero(s);
+        for (int k = lane; k < n; k += 32)
+            w[k] = fix_pair<true>(X[3 * k], X[3 * k + 1], X[3 * k + 2], P[0] - v[0], P[1] - v[1], P[2] - v[2], cst, bq, table, s);
+        if (s.top >= 0) return 2;
+        i64 c[10];
+        fix_combine(s, c);
+        for (int i = 0; i < 10; i++) t[i] += c[i];
+    }
+    const int I[6] = {0, 1, 2, 0, 1, 0}, J[6] = {0, 1, 2, 1, 2, 2};
+    out[0] = std::ldexp((double)t[0], -63);
+    for (int i = 0; i < 3; i++) out[1 + i] = std::ldexp((double)fix_r_about(t[0], t[1 + i], v[i]), -fb);
+    for (int q = 0; q < 6; q++) {
+        const i64 rd = fix_r_about(t[0], t[1 + J[q]], v[J[q]]);
+        out[4 + q] = std::ldexp((double)fix_a_about(t[4 + q], t[1 + I[q]], rd, v[I[q]], v[J[q]]), 60 - 2 * fb);
+    }
+    for (int k = 0; k < n; k++)
+        for (int i = 0; i < 3; i++) {
+            const i64 D = P[i] - X[3 * k + i];
+            const u64 nb = fx_d_bits(w[k]);
+            prod[3 * k + i] = llabs(D) >= (2LL << 32)
+                                  ? fix_mul_double(((nb & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11, (int)(nb >> 52), D, fb)
+                                  : w[k] * std::ldexp((double)D, -fb);
+        }
+    return 0;
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("no host compiler")
+    d = tmp_path_factory.mktemp("fix")
+    (d / "fix.cpp").write_text(SRC)
+    so = str(d / "fix.so")
+    subprocess.run([gxx, "-O2", "-std=gnu++17", "-shared", "-fPIC", "-I", CSRC, str(d / "fix.cpp"), "-o", so], check=True)
+    L = C.CDLL(so)
+    L.eval.argtypes = [C.c_int] + [C.c_void_p] * 3 + [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_uint64] + [C.c_void_p] * 3
+    return L
+
+
+# spacing, origin in spacings, whole ball or a corner of the body, centre offset lambda h, support tolerance
+@pytest.mark.parametrize("h,origin,corner,lam_h,tol", [
+    (0.12e-3, 100.0, False, 0.0, 1e-6), (0.17e-3, 0.0, False, 0.3, 1e-6), (1.0, -3000.0, False, 0.1, 1e-6),
+    (0.23e-3, 40.0, True, 0.8, 1e-6), (3.0e-3, 7.0, False, 0.05, 1e-9), (5.0e-3, 1.0, False, 0.0, 1e-2)])
+def test_fixed_point_evaluation(lib, h, origin, corner, lam_h, tol):
+    getcontext().prec = 60
+    rng = np.random.default_rng(int(1e6 * h) + int(corner))
+    beta = 0.8 / (h * h)
+    rs = np.sqrt(np.log(1 / tol) / beta)
+    m = int(rs / h) + 2
+    g = np.arange(0 if corner else -m, m + 1)
+    x = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3) * h + origin * h
+    x = x + rng.uniform(-0.02, 0.02, x.shape) * h
+    xp = (origin + (0.3 if corner else 0.0)) * h + rng.uniform(-0.2, 0.2, 3) * h
+    x = np.ascontiguousarray(x[((xp - x) ** 2).sum(1) <= rs * rs][:384])
+    lam = rng.uniform(-1, 1, 3) * lam_h / h
+    n = len(x)
+    # constants as the library derives them: 2^63 units = 2^ex >= 2.2 support radii
+    fb = 63 - int(np.frexp(2.2 * rs)[1])
+    D = Decimal
+    ln2 = D(2).ln()
+    a = D(2) ** (32 - fb)
+    bq = int(D(beta) * 256 / ln2 * a * a * D(2) ** 109)
+    assert bq < 2 ** 64
+    table = np.array([int((D(2) ** (D(j) / 1024)) * D(2) ** 63 + D("0.5")) for j in range(1024)], np.uint64)
+    d = [[D(float(xp[i])) - D(float(x[k, i])) for i in range(3)] for k in range(n)]
+    # the kernel's centre is lambda / (2 beta) in whole units: the reference takes that lambda
+    v = [int(np.rint(lam[i] * 2.0 ** fb / (2 * beta))) for i in range(3)]
+    ld = [D(v[i]) * D(2) ** -fb * 2 * D(beta) for i in range(3)]
+    f = [-D(beta) * sum(c * c for c in dk) + sum(l * c for l, c in zip(ld, dk)) for dk in d]
+    shift = float(sum(t.exp() for t in f).ln()) + 1.0
+    wr = [(t - D(shift)).exp() for t in f]
+    out, w, prod = np.zeros(10), np.zeros(n), np.zeros((n, 3))
+    ptr = lambda t: t.ctypes.data_as(C.c_void_p)
+    st = lib.eval(n, ptr(x), ptr(xp), ptr(lam), beta, shift, fb, ptr(table), bq, ptr(out), ptr(w), ptr(prod))
+    assert st == 0
+    Z = sum(wr)
+    # weights relative to Z: half an ulp of the FP64 weight and Z each, 2e-17 per exponent unit, truncation
+    for k in range(n):
+        assert abs(D(float(w[k])) / D(float(out[0])) * Z / wr[k] - 1) <= D("8e-16")
+    ij = [(0, 0), (1, 1), (2, 2), (0, 1), (1, 2), (0, 2)]
+    tr = sum(wk * sum(c * c for c in dk) for wk, dk in zip(wr, d)) / Z
+    for i in range(3):
+        ref = sum(wk * dk[i] for wk, dk in zip(wr, d)) / Z
+        assert abs(D(float(out[1 + i])) / D(float(out[0])) - ref) <= D("4e-16") * tr.sqrt()
+    for q, (i, j) in enumerate(ij):
+        ref = sum(wk * dk[i] * dk[j] for wk, dk in zip(wr, d)) / Z
+        assert abs(D(float(out[4 + q])) / D(float(out[0])) - ref) <= D("2e-15") * tr
+    for k in range(n):
+        for i in range(3):
+            ref = D(float(w[k])) * d[k][i]
+            # half an ulp, and half a unit of each coordinate
+            assert abs(D(float(prod[k, i])) - ref) <= D(2) ** -53 * abs(ref) + D(float(w[k])) * D(2) ** (1 - fb)

@@ -226,3 +226,57 @@ def test_internal_exp_against_cuda_exp():
                               C.c_void_p(ro.data_ptr()), C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
     torch.cuda.synchronize()
     assert mo.cpu().numpy().tolist() == [0.0, np.inf, 0.0, np.inf, 0.0, np.inf]
+
+
+@pytest.mark.parametrize("h,gamma,tol,offset,S", [
+    (0.8e-3, 0.8, 1e-6, 0.0, 384), (0.8e-3, 0.8, 1e-6, 3.7, 384),      # the default, far from the origin
+    (0.7e-3, 1.6, 1e-6, 0.0, 128), (0.9e-3, 4.0, 1e-6, 0.0, 64),       # small supports (32 slots and below)
+    (0.8e-3, 0.72, 1e-6, -0.5, 384), (0.8e-3, 0.62, 1e-6, 0.0, 512),   # supports about and above 336 slots
+    (0.8e-3, 1.2, 3e-10, 0.0, 384), (0.8e-3, 1.4, 1e-12, 0.0, 384)])   # at and past the fixed-point range
+def test_step_shape_functions_vs_oracle(orc, h, gamma, tol, offset, S):
+    """The FP64 step's shape functions (fixed-point evaluations where their range covers the problem, FP64
+    elsewhere) against the oracle's LME at the GPU's own positions, after steps that deform the body, and
+    with points moved close to the hull, where lambda leaves the fixed-point range. Bound: both
+    solves stop at |r| <= 1e-14 h, which moves N by up to |J^-1 r . d| = 2 gamma 1e-14 sqrt(ln(1/tol)/gamma)
+    of itself each (2.6e-13 at most here), times 4 for the condition of J near the surface: 1e-12."""
+    from paper_2206_08772_gb300.otm import OTM
+    p = scenarios.taylor_rod(h=h, L=8 * h, gamma=gamma, support_tol=tol, material=scenarios.copper_jc())
+    p.node_x[:] += offset
+    p.mp_x[:] += offset
+    p.contact.wall_point = (0.0, 0.0, offset)
+    rng = np.random.default_rng(3)
+    p.node_du0[:] += rng.normal(0, 2e-3 * h, p.node_du0.shape)
+    sim = OTM(p, max_support=S)
+    assert sim.step(3) == 0, sim.error()
+
+    def check(points, bound):
+        x, xp, cnt = sim.get("node_x"), sim.get("mp_x"), sim.get("support_count")
+        ids, sh = sim.get_rows("support_ids", points), sim.get_rows("shape", points)
+        for r, q in enumerate(points):
+            d = xp[q] - x[ids[r, :cnt[q]]]
+            assert ((d * d).sum(1) <= p.rs2).all()
+            st, N, dN, _, _ = orc.lme(d, p.beta, p.newton_tol * p.h)
+            assert st == 0
+            assert rel(sh[r, :cnt[q], 0], N) <= bound
+            assert rel(sh[r, :cnt[q], 1:], dN) <= 10 * bound
+        return cnt
+
+    cnt = check(np.arange(0, p.n_mps, max(1, p.n_mps // 60)), 1e-12)
+    if gamma < 0.75:
+        assert (cnt > 336).any()
+    # the first point of each of a few cells towards the nearest corner node of the bottom face: lambda grows
+    x, xp = sim.get("node_x"), sim.get("mp_x")
+    corner = x[np.argmax(x[:, 0] - x[:, 2])]
+    near = np.argsort(((xp - corner) ** 2).sum(1))[:3]
+    for k, q in enumerate(near):
+        xp[q] = corner + (xp[q] - corner) * (0.3, 0.05, 0.01)[k]
+    sim.set("mp_x", xp)
+    assert sim.refresh() == 0, sim.error()
+    lam = sim.get("lam")[near]
+    check(near, 1e-9)     # J is near-singular there: conditioned by (distance / h)^-2, at most 1e4 above
+    if gamma == 0.8:      # a sharper prior needs less lambda to reach the hull
+        assert np.abs(lam).max() * h > 3.0
+    # a restored state repeats the solve bit for bit, on whichever path it ran
+    snap, before = sim.snapshot(), sim.get("shape")
+    sim.restore(snap)
+    assert np.array_equal(before, sim.get("shape"))
