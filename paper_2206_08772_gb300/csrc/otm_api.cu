@@ -223,7 +223,10 @@ static void fill_params(Dev &D, const otm_params *P)
     D.tool_clear = P->tool_clear;
     D.tool_v = P->tool_v;
     D.friction = P->friction;
-    for (int i = 0; i < 4; i++) D.mat[i] = P->mat[i];
+    for (int i = 0; i < 4; i++) {
+        D.mat[i] = P->mat[i];
+        D.rmc[i] = make_rm_const(P->mat[i], P->dt);
+    }
 }
 
 static int read_error(otm_handle *h, int32_t *code, int64_t *id)

@@ -55,7 +55,14 @@ struct FixStart {
     i64 xp[3], v[3], cst, ok, pad;
 };
 
+// a material's derived constants (return_map_small)
+struct RmConst {
+    double K, mu, i3mu, ih;          // bulk and shear modulus, 1 / (3 mu), 1 / (2 mu + 2 H / 3)
+    double idt, idte, ispan, heat;   // 1 / dt, 1 / (dt eps_dot0), 1 / (T_melt - T_room), chi / (rho0 cp)
+};
+
 SearchConst make_search_const(double cell, double rs2);
+RmConst make_rm_const(const otm_material &M, double dt);
 FixConst make_fix_const(double beta, double rs2);
 
 struct Dev {
@@ -76,6 +83,7 @@ struct Dev {
     double wall_p[3], wall_n[3];
     double tool_x0, tool_tip_y, tool_rake, tool_clear, tool_v, friction;
     otm_material mat[4];
+    RmConst rmc[4];
 
     // nodes
     double4_32a *x, *x_prev, *du, *mr;   // mr = (mass, force xyz) of the last node update

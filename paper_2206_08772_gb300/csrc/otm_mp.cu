@@ -98,6 +98,7 @@ constexpr int kExpNmax = 1021 * 1024 + 1023;
 
 static __device__ double g_exp2_table[kExpTable];
 static __device__ u64 g_exp2_mant[kExpTable];          // 2^(j/1024) as 64-bit mantissas (fix_exp)
+static __device__ double2 g_log_table[kExpTable];      // (r, -log r), see log_pos
 
 // Fill g_exp2_table on the current device (first call per device; a synchronous copy, so it
 // belongs before any stream capture: otm_init and the stand-alone entries call it). With
@@ -127,6 +128,15 @@ cudaError_t exp_table_setup(bool verify)
     for (int j = 0; j < kExpTable; j++)
         mant[j] = (u64)std::floor(std::ldexp(std::exp2((long double)j / (long double)kExpTable), 63) + 0.5L);
     e = cudaMemcpyToSymbol(g_exp2_mant, mant, sizeof(mant));
+    if (e != cudaSuccess) return e;
+    double2 lg[kExpTable];   // (r, -log r), r ~ 1/m at the middle of the interval (1 exactly about m = 1)
+    for (int j = 0; j < kExpTable; j++) {
+        double m = 1.0 + (j + 0.5) / kExpTable;
+        if (j >= 424) m *= 0.5;
+        const double r = (j == 0 || j == kExpTable - 1) ? 1.0 : 1.0 / m;
+        lg[j] = make_double2(r, (double)-std::log((long double)r));
+    }
+    e = cudaMemcpyToSymbol(g_log_table, lg, sizeof(lg));
     if (e != cudaSuccess) return e;
     e = cudaMemcpyToSymbol(g_exp2_table, host, sizeof(host));
     if (e == cudaSuccess) done[dev] = true;
@@ -1348,7 +1358,7 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
     const double cf = from(J, nib(0x335001)) * from(J, nib(0x454122)) - from(J, nib(0x503354)) * from(J, nib(0x142354));
     const double det = fma(from(J, 5), from(cf, 5), fma(from(J, 3), from(cf, 3), from(J, 0) * from(cf, 0)));
     const bool regular = det > 0.0 && isfinite(det);
-    const double inv = cf * recip<3>(det);
+    const double inv = cf * recip<2>(det);
     // the step -J'^-1 r, lane q < 3 its component, and the next trial
     const double step = -fma(from(inv, nib(0x245)), r2, fma(from(inv, nib(0x413)), r1, from(inv, nib(0x530)) * r0));
     const double lam = q < 3 ? m.trial[q] : 0.0;
@@ -1386,7 +1396,7 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
         if (q < 6) m.inv[q] = inv;
         if (q == 0) {
             m.have_cur = 1;
-            m.iZ = recip<3>(Z);
+            m.iZ = recip<2>(Z);
             // the next solve's shift: its Z then starts in [1/4, 1/2) (see newton_finish)
             const int ez = ((__double2hiint(Z) >> 20) & 0x7ff) - 1023;
             m.logz = fma((double)(ez + 2), 0x1.62e42fefa39efp-1, sh);
@@ -1816,7 +1826,255 @@ cudaError_t launch_kinematics(const Dev &D, cudaStream_t s, long long *launches)
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(128) k_return_map(const Dev D)
+// ======================================================================== return map without eigenvectors
+// Logarithm after P. T. P. Tang ("Table-driven implementation of the logarithm function in IEEE
+// floating-point arithmetic", ACM TOMS 16(4), 1990), for positive normal arguments: x = 2^e m with m in
+// [0.7, 1.4), r ~ 1/m from a 1024-entry table, t = m r - 1 (one rounding, |t| < 2^-9.9), and log x = e ln 2 -
+// log r + (t - t^2/2 + t^3/3 - t^4/4 + t^5/5). The table holds (r, -log r); absolute error below
+// 1e-16 max(1, |log x|). About 11 FP64 instructions; the library's log takes the pipe time of 33.
+
+__device__ __forceinline__ double log_pos(double x)
+{
+    const int hi = __double2hiint(x);
+    int e = (hi >> 20) - 1023;
+    const int j = (hi >> 10) & 1023;
+    const bool up = j >= 424;          // m >= 1.414: m / 2 and e + 1, so that arguments about 1 have e = 0
+    e += up;
+    const double m = __hiloint2double((hi & 0xfffff) | (up ? 0x3fe00000 : 0x3ff00000), __double2loint(x));
+    const double2 c = g_log_table[j];
+    const double t = fma(m, c.x, -1.0);
+    const double t2 = t * t;
+    const double q = fma(t, fma(t, fma(t, 0.2, -0.25), 0x1.5555555555555p-2), -0.5);
+    // the integer e as a double by its bits (a conversion costs an FP64 instruction as well; this one
+    // is a subtraction of two exactly known values)
+    const double ed = __hiloint2double(0x43300000, 0x40000000 + e) - 0x1.0000040000000p52;
+    return fma(ed, 0x1.62e42fefa39efp-1, fma(ed, 0x1.abc9e3b39803fp-56, c.y + fma(t2, q, t)));
+}
+
+__device__ __forceinline__ double exp_of(double v) { return exp_scaled(v * kExpScale, g_exp2_table); }
+
+// x^n for x > 0 by exp(n log x): relative error about (1 + |n log x|) 2e-16
+__device__ __forceinline__ double pow_pos(double x, double n) { return exp_of(n * log_pos(x)); }
+
+// Johnson-Cook flow stress at E = ebar_n + x (x > 0) and its derivative in x, as jc_sigma_y
+__device__ __forceinline__ void jc_flow(const otm_material &M, double E, double x, double inv_dte, double therm, double &sy,
+                                        double &dsy)
+{
+    const double ixE = recip<2>(x * E), ix = E * ixE, iE = x * ixE;
+    const double rstar = x * inv_dte;
+    double rate = 1.0, drate = 0.0;
+    if (rstar > 1.0) {
+        rate = fma(M.C, log_pos(rstar), 1.0);
+        drate = M.C * ix;
+    }
+    const double bp = M.B * pow_pos(E, M.n), hard = M.A + bp;
+    sy = hard * rate * therm;
+    dsy = fma(M.n * bp * iE, rate, hard * drate) * therm;
+}
+
+// The consistency condition's root in FP32 (Newton inside the bracket [0, hi]): within about 1e-5 of
+// the FP64 root, where two FP64 evaluations finish. All stresses divided by 3 mu.
+__device__ __forceinline__ float jc_root32(const otm_material &M, float s3, float ebar, float inv_dte, float therm, float hi,
+                                           float x)
+{
+    const float A = (float)M.A * s3 * therm, B = (float)M.B * s3 * therm, n = (float)M.n, C = (float)M.C;
+    float lo = 0.f, up = hi;
+    for (int it = 0; it < 6; it++) {
+        const float E = ebar + x, p = B * exp2f(n * __log2f(E)), hard = A + p, rs = x * inv_dte;
+        const bool on = rs > 1.f;
+        const float rate = on ? fmaf(C, __logf(rs), 1.f) : 1.f;
+        const float g = hi - x - hard * rate;
+        const float d = 1.f + __fdividef(n * p, E) * rate + (on ? __fdividef(hard * C, x) : 0.f);
+        if (g > 0.f) lo = x; else up = x;
+        const float xn = x + __fdividef(g, d);
+        const float y = (xn > lo && xn < up) ? xn : 0.5f * (lo + up);
+        if (fabsf(y - x) <= 1e-6f * y) { x = y; break; }
+        x = y;
+    }
+    return x;
+}
+
+// The constitutive update (return_map_point) for points whose deviatoric elastic strain is small,
+// without the eigen decomposition: with b_tr = (1 + p)(I + Y), Y traceless and |Y| <= 1/32,
+//   log b_tr = log(1 + p) I + log(I + Y),   b^e = (1 + p) exp(w) exp(2 rho dev e)
+// by their power series reduced with Cayley-Hamilton (Y^3 = -I2 Y + I3 I: two FMAs a term); the radial
+// return scales the deviator by rho, so neither needs principal axes. b_tr - I is formed from dF - I
+// and b^e - I, free of the rounding about 1. Metals stay below the bound: it is a shear strain of
+// about 1 %, ten times a copper's yield strain; anything else (and non-finite input) returns false
+// and takes return_map_point.
+//
+// FP64 pipe bound. Measured (two thirds of the points plastic, Johnson-Cook): 1,000,003 stand-alone points
+// 3.02 -> 0.78 ms a call; k_return_map on the 202,752-MP rod 1.40 -> 0.45 ms.
+__device__ __forceinline__ bool return_map_small(const otm_material &M, const RmConst &R, const RmIn &in, RmOut &out, int &status)
+{
+    double y[6], H[9];   // b_tr - I as (xx, yy, zz, xy, yz, xz)
+    {
+        const double g[9] = {in.dF[0] - 1.0, in.dF[1], in.dF[2], in.dF[3], in.dF[4] - 1.0, in.dF[5],
+                             in.dF[6], in.dF[7], in.dF[8] - 1.0};
+        const double b[6] = {in.be[0] - 1.0, in.be[1] - 1.0, in.be[2] - 1.0, in.be[3], in.be[4], in.be[5]};
+        // H = g (I + b), y = b + H + H^T + H g^T
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const double gx = g[3 * i], gy = g[3 * i + 1], gz = g[3 * i + 2];
+            H[3 * i] = gx + fma(gx, b[0], fma(gy, b[3], gz * b[5]));
+            H[3 * i + 1] = gy + fma(gx, b[3], fma(gy, b[1], gz * b[4]));
+            H[3 * i + 2] = gz + fma(gx, b[5], fma(gy, b[4], gz * b[2]));
+        }
+        const int I[6] = {0, 1, 2, 0, 1, 0}, J[6] = {0, 1, 2, 1, 2, 2};
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const int i = I[c], j = J[c];
+            y[c] = b[c] + (H[3 * i + j] + H[3 * j + i]) +
+                   fma(H[3 * i], g[3 * j], fma(H[3 * i + 1], g[3 * j + 1], H[3 * i + 2] * g[3 * j + 2]));
+        }
+    }
+    const double p = (y[0] + y[1] + y[2]) * (1.0 / 3.0);
+    if (!(fabs(p) < 0.5)) return false;
+    const double ip = recip<2>(1.0 + p);
+    double Y[6];
+#pragma unroll
+    for (int c = 0; c < 6; c++) Y[c] = (c < 3 ? y[c] - p : y[c]) * ip;
+    // Y^2, I2 = -tr(Y^2)/2, I3 = det Y
+    double Y2[6];
+    Y2[0] = fma(Y[0], Y[0], fma(Y[3], Y[3], Y[5] * Y[5]));
+    Y2[1] = fma(Y[1], Y[1], fma(Y[3], Y[3], Y[4] * Y[4]));
+    Y2[2] = fma(Y[2], Y[2], fma(Y[4], Y[4], Y[5] * Y[5]));
+    Y2[3] = fma(Y[0], Y[3], fma(Y[3], Y[1], Y[5] * Y[4]));
+    Y2[4] = fma(Y[3], Y[5], fma(Y[1], Y[4], Y[4] * Y[2]));
+    Y2[5] = fma(Y[0], Y[5], fma(Y[3], Y[4], Y[5] * Y[2]));
+    const double t2 = Y2[0] + Y2[1] + Y2[2];
+    if (!(t2 <= 1.0 / 1024.0)) return false;
+    const double h2 = 0.5 * t2;    // -I2
+    const double I3 = fma(Y[0], fma(Y[1], Y[2], -Y[4] * Y[4]), fma(Y[3], fma(Y[4], Y[5], -Y[3] * Y[2]),
+                                                                   Y[5] * fma(Y[3], Y[4], -Y[1] * Y[5])));
+    // log(I + Y) = c0 I + c1 Y + c2 Y^2, Horner from the 11th term (|eigenvalue| < 0.0256: rest below 1e-20)
+    double c0 = 1.0 / 11.0, c1 = 0.0, c2 = 0.0;
+#pragma unroll
+    for (int k = 10; k >= 0; k--) {   // (c0 + c1 Y + c2 Y^2) Y + a_k, a_k = -(-1)^k / k, a_0 = 0
+        const double a = k == 0 ? 0.0 : ((k & 1) ? 1.0 : -1.0) / (k == 0 ? 1 : k);
+        const double n0 = fma(c2, I3, a), n1 = fma(c2, h2, c0);
+        c2 = c1;
+        c1 = n1;
+        c0 = n0;
+    }
+    const double w = fma(c2, t2, 3.0 * c0) * (1.0 / 3.0);   // tr log(I + Y) / 3
+    const double q1 = 1.0 + p;
+    const double tr = 1.5 * (log_pos(q1) + (p - (q1 - 1.0)) * ip + w);    // tr e
+    double e[6];   // dev e
+#pragma unroll
+    for (int c = 0; c < 6; c++) e[c] = 0.5 * fma(c2, c < 3 ? Y2[c] - t2 * (1.0 / 3.0) : Y2[c], c1 * Y[c]);
+    const double mu = R.mu;
+    const double en2 = fma(2.0, fma(e[3], e[3], fma(e[4], e[4], e[5] * e[5])), fma(e[0], e[0], fma(e[1], e[1], e[2] * e[2])));
+    const double sn = 2.0 * mu * sqrt(en2);
+    const double q_tr = 1.2247448713915890491 * sn;   // sqrt(3/2) |s|
+    double dep = 0.0;
+    if (M.model == 0) {
+        const double f_tr = sn - 0.81649658092772603273 * (M.sigma_y0 + M.H * in.ebar);
+        if (f_tr > 0.0) dep = 0.81649658092772603273 * f_tr * R.ih;
+    } else {
+        const double tstar = fmin(fmax((in.T - M.T_room) * R.ispan, 0.0), 1.0);
+        const double therm = tstar > 1e-300 ? 1.0 - pow_pos(tstar, M.m) : 1.0 - pow(tstar, M.m);
+        const double pe = in.ebar > 1e-300 ? pow_pos(in.ebar, M.n) : pow(in.ebar, M.n);
+        if (q_tr - (M.A + M.B * pe) * therm > 0.0) {
+            // g(x) = q_tr - 3 mu x - sigma_y(x) on [0, q_tr / (3 mu)]: Newton safeguarded by bisection from the
+            // FP32 root
+            double lo = 0.0, hi = q_tr * R.i3mu;
+            double x = (in.guess > 0.0 && in.guess < hi) ? in.guess : 0.5 * hi;
+            const float x32 = jc_root32(M, (float)R.i3mu, (float)in.ebar, (float)R.idte, (float)therm, (float)hi, (float)x);
+            if (x32 > 0.f && (double)x32 < hi) x = (double)x32;
+            const double tol = 1e-12 * q_tr;
+            bool ok = false;
+            for (int it = 0; it < 300; it++) {
+                double sy, dsy;
+                jc_flow(M, in.ebar + x, x, R.idte, therm, sy, dsy);
+                const double g = q_tr - 3.0 * mu * x - sy;
+                const double xn = fma(g, recip<2>(fma(3.0, mu, dsy)), x);
+                if (fabs(g) <= tol) {   // one more Newton step fixes the accepted iterate to rounding
+                    if (xn > lo && xn < hi) x = xn;
+                    ok = true;
+                    break;
+                }
+                if (g > 0.0) lo = x; else hi = x;
+                if (hi - lo <= 4e-16 * hi) { ok = true; break; }
+                x = (xn > lo && xn < hi) ? xn : 0.5 * (lo + hi);
+            }
+            if (!ok) {
+                status = OTM_ERR_RETURNMAP_NOCONV;
+                return true;
+            }
+            dep = x;
+        }
+    }
+    const double qn = q_tr - 3.0 * mu * dep;
+    const double rho = dep > 0.0 ? 1.0 - 2.0 * mu * (1.2247448713915890491 * dep) / sn : 1.0;
+    const double iJ = 1.0 / in.J, kt = R.K * tr, m2 = 2.0 * mu * rho;
+#pragma unroll
+    for (int c = 0; c < 6; c++) out.sig[c] = (c < 3 ? fma(m2, e[c], kt) : m2 * e[c]) * iJ;
+    if (dep > 0.0) {
+        // b^e = (1 + p) exp(w) exp(D), D = 2 rho dev e traceless: both by their Taylor series (D to the 9th
+        // term, below 1e-19)
+        double D[6], D2[6];
+#pragma unroll
+        for (int c = 0; c < 6; c++) D[c] = 2.0 * rho * e[c];
+        D2[0] = fma(D[0], D[0], fma(D[3], D[3], D[5] * D[5]));
+        D2[1] = fma(D[1], D[1], fma(D[3], D[3], D[4] * D[4]));
+        D2[2] = fma(D[2], D[2], fma(D[4], D[4], D[5] * D[5]));
+        D2[3] = fma(D[0], D[3], fma(D[3], D[1], D[5] * D[4]));
+        D2[4] = fma(D[3], D[5], fma(D[1], D[4], D[4] * D[2]));
+        D2[5] = fma(D[0], D[5], fma(D[3], D[4], D[5] * D[2]));
+        const double d2 = 0.5 * (D2[0] + D2[1] + D2[2]);
+        const double d3 = fma(D[0], fma(D[1], D[2], -D[4] * D[4]), fma(D[3], fma(D[4], D[5], -D[3] * D[2]),
+                                                                       D[5] * fma(D[3], D[4], -D[1] * D[5])));
+        constexpr double kInvFact[10] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040,
+                                         1.0 / 40320, 1.0 / 362880};
+        double a0 = kInvFact[9], a1 = 0.0, a2 = 0.0;
+#pragma unroll
+        for (int k = 8; k >= 0; k--) {
+            const double n0 = fma(a2, d3, k == 0 ? 0.0 : kInvFact[k]), n1 = fma(a2, d2, a0);
+            a2 = a1;
+            a1 = n1;
+            a0 = n0;
+        }
+        // exp(D) - I = a0 I + a1 D + a2 D^2; (1 + p) exp(w) - 1 = p + (1 + p)(exp(w) - 1), |w| < 5e-4
+        const double ew = w * fma(w, fma(w, fma(w, fma(w, 1.0 / 120, 1.0 / 24), 1.0 / 6), 0.5), 1.0);
+        const double v = fma(q1, ew, p), sc = 1.0 + v;
+#pragma unroll
+        for (int c = 0; c < 6; c++) {
+            const double x = fma(a2, D2[c], a1 * D[c]);
+            out.be[c] = c < 3 ? 1.0 + (v + sc * (x + a0)) : sc * x;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 6; c++) out.be[c] = c < 3 ? 1.0 + y[c] : y[c];
+    }
+    out.ebar = in.ebar + dep;
+    out.rate = dep * R.idt;
+    out.T = in.T;
+    if (M.model == 1 && M.chi > 0.0 && dep > 0.0) out.T = fma(R.heat * qn, dep, in.T);
+    out.failed = jc_fractured(M, kt * iJ, qn, iJ, out);
+    status = OTM_OK;
+    for (int c = 0; c < 6; c++)
+        if (!isfinite(out.sig[c])) status = OTM_ERR_NONFINITE;
+    return true;
+}
+
+RmConst make_rm_const(const otm_material &M, double dt)
+{
+    RmConst r;
+    r.K = M.E / (3.0 * (1.0 - 2.0 * M.nu));
+    r.mu = M.E / (2.0 * (1.0 + M.nu));
+    r.i3mu = 1.0 / (3.0 * r.mu);
+    r.ih = 1.0 / (2.0 * r.mu + 2.0 * M.H / 3.0);
+    r.idt = 1.0 / dt;
+    r.idte = 1.0 / (dt * M.eps_dot0);
+    r.ispan = 1.0 / (M.T_melt - M.T_room);
+    r.heat = M.chi / (M.rho0 * M.cp);
+    return r;
+}
+
+// SMALL: the FP64 path; the mixed path keeps return_map_point (see launch_lme_t on its FP32 increments)
+template <bool SMALL>
+__global__ void __launch_bounds__(128) k_return_map(const __grid_constant__ Dev D)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= D.nm) return;
@@ -1857,11 +2115,16 @@ __global__ void __launch_bounds__(128) k_return_map(const Dev D)
     in.ebar = D.ebar[p];
     in.T = D.T[p];
     in.guess = D.rate[p] * D.dt;   // the previous step's plastic increment
-    double Q0[9];
-    for (int i = 0; i < 9; i++) Q0[i] = D.Qe[9 * p + i];
-    in.Q0 = Q0;
     RmOut o;
-    const int st = return_map_point(D.mat[D.mat_id[p]], D.dt, in, o);
+    int st = OTM_OK;
+    if (!SMALL || !return_map_small(D.mat[D.mat_id[p]], D.rmc[D.mat_id[p]], in, o, st)) {
+        double Q0[9];
+        for (int i = 0; i < 9; i++) Q0[i] = D.Qe[9 * p + i];
+        in.Q0 = Q0;
+        st = return_map_point(D.mat[D.mat_id[p]], D.dt, in, o);
+        if (st == OTM_OK)
+            for (int i = 0; i < 9; i++) D.Qe[9 * p + i] = o.Q[i];
+    }
     if (st != OTM_OK) {
         raise_error(D.err, st, D.mgid[p]);
         return;
@@ -1873,7 +2136,6 @@ __global__ void __launch_bounds__(128) k_return_map(const Dev D)
     D.ebar[p] = o.ebar;
     D.T[p] = o.T;
     D.rate[p] = o.rate;
-    for (int i = 0; i < 9; i++) D.Qe[9 * p + i] = o.Q[i];
     D.failed[p] = (uint8_t)(o.failed && D.allow_erode);
 }
 
@@ -1881,7 +2143,10 @@ cudaError_t launch_return_map(const Dev &D, cudaStream_t s, long long *launches)
 {
     const unsigned blocks = (unsigned)((D.nm + 127) / 128);
     if (blocks == 0) return cudaSuccess;
-    k_return_map<<<blocks, 128, 0, s>>>(D);
+    if (D.precision == OTM_PRECISION_MIXED)
+        k_return_map<false><<<blocks, 128, 0, s>>>(D);
+    else
+        k_return_map<true><<<blocks, 128, 0, s>>>(D);
     if (launches) *launches += 1;
     return cudaGetLastError();
 }
@@ -2029,7 +2294,7 @@ cudaError_t launch_exp_selftest(const double *x, int64_t n, double *mine, double
 }
 
 __global__ void __launch_bounds__(128)
-    k_return_map_only(const otm_material M, double dt, int64_t nm, const double *dF, const double *F_new, double *be,
+    k_return_map_only(const __grid_constant__ otm_material M, const __grid_constant__ RmConst R, double dt, int64_t nm, const double *dF, const double *F_new, double *be,
                       double *ebar, double *T, double *sigma, double *rate, uint8_t *failed, int32_t *status)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2045,7 +2310,8 @@ __global__ void __launch_bounds__(128)
     in.J = Fn[0] * (Fn[4] * Fn[8] - Fn[5] * Fn[7]) - Fn[1] * (Fn[3] * Fn[8] - Fn[5] * Fn[6]) +
            Fn[2] * (Fn[3] * Fn[7] - Fn[4] * Fn[6]);
     RmOut o;
-    const int st = return_map_point(M, dt, in, o);
+    int st = OTM_OK;
+    if (!return_map_small(M, R, in, o, st)) st = return_map_point(M, dt, in, o);
     if (st != OTM_OK) {
         atomicCAS(status, 0, st);
         return;
@@ -2066,7 +2332,7 @@ cudaError_t launch_return_map_only(const otm_material *mat, double dt, int64_t n
 {
     const unsigned blocks = (unsigned)((nm + 127) / 128);
     if (blocks == 0) return cudaSuccess;
-    k_return_map_only<<<blocks, 128, 0, s>>>(*mat, dt, nm, dF, F_new, be, ebar, T, sigma, rate, failed, status);
+    k_return_map_only<<<blocks, 128, 0, s>>>(*mat, make_rm_const(*mat, dt), dt, nm, dF, F_new, be, ebar, T, sigma, rate, failed, status);
     return cudaGetLastError();
 }
 

@@ -81,6 +81,22 @@ struct RmOut {
     bool failed;
 };
 
+// the Johnson-Cook fracture criterion (Sec. 4.2) for an updated point: pressure pr, von Mises Kirchhoff
+// stress qn, 1/J, and the updated ebar, T and rate in out
+__device__ __forceinline__ bool jc_fractured(const otm_material &M, double pr, double qn, double iJ, const RmOut &out)
+{
+    if (!(M.model == 1 && M.fracture && out.ebar > 0.0)) return false;
+    const double sv = fmax(qn, 0.0) * iJ;
+    // triaxiality; its limit sign(p) * inf where no deviatoric stress is left (melted point)
+    const double eta = (sv > 1e-12 * fabs(pr)) ? pr / sv : (pr > 0.0 ? INFINITY : (pr < 0.0 ? -INFINITY : 0.0));
+    const double texp = (M.d3 == 0.0) ? 1.0 : exp(M.d3 * eta);
+    const double rstar = out.rate / M.eps_dot0;
+    const double lr = (rstar > 1.0) ? log(rstar) : 0.0;
+    const double tstar = fmin(fmax((out.T - M.T_room) / (M.T_melt - M.T_room), 0.0), 1.0);
+    const double ef = (M.d1 + M.d2 * texp) * (1.0 + M.d4 * lr) * (1.0 + M.d5 * tstar);
+    return out.ebar >= ef;
+}
+
 // returns OTM_OK or an error code
 __device__ inline int return_map_point(const otm_material &M, double dt, const RmIn &in, RmOut &out)
 {
@@ -200,19 +216,7 @@ __device__ inline int return_map_point(const otm_material &M, double dt, const R
     out.rate = dep / dt;
     out.T = in.T;
     if (M.model == 1 && M.chi > 0.0 && dep > 0.0) out.T = in.T + M.chi * qn * dep / (M.rho0 * M.cp);
-    out.failed = false;
-    if (M.model == 1 && M.fracture && out.ebar > 0.0) {
-        const double pr = K * tr * iJ;
-        const double sv = fmax(qn, 0.0) * iJ;
-        // triaxiality; its limit sign(p) * inf where no deviatoric stress is left (melted point)
-        const double eta = (sv > 1e-12 * fabs(pr)) ? pr / sv : (pr > 0.0 ? INFINITY : (pr < 0.0 ? -INFINITY : 0.0));
-        const double texp = (M.d3 == 0.0) ? 1.0 : exp(M.d3 * eta);
-        const double rstar = out.rate / M.eps_dot0;
-        const double lr = (rstar > 1.0) ? log(rstar) : 0.0;
-        const double tstar = fmin(fmax((out.T - M.T_room) / (M.T_melt - M.T_room), 0.0), 1.0);
-        const double ef = (M.d1 + M.d2 * texp) * (1.0 + M.d4 * lr) * (1.0 + M.d5 * tstar);
-        out.failed = (out.ebar >= ef);
-    }
+    out.failed = jc_fractured(M, K * tr * iJ, qn, iJ, out);
     for (int c = 0; c < 6; c++)
         if (!isfinite(out.sig[c])) return OTM_ERR_NONFINITE;
     return OTM_OK;

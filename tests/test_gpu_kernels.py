@@ -280,3 +280,57 @@ def test_step_shape_functions_vs_oracle(orc, h, gamma, tol, offset, S):
     snap, before = sim.snapshot(), sim.get("shape")
     sim.restore(snap)
     assert np.array_equal(before, sim.get("shape"))
+
+
+@pytest.mark.parametrize("model", ["j2", "jc", "ti64"])
+@pytest.mark.parametrize("strain,pressure", [(0.0, 0.0), (1e-6, 0.0), (1e-3, 0.0), (7e-3, 0.0), (0.012, 0.0),
+                                             (1e-3, 0.04), (1e-3, -0.2), (1e-3, 0.7), (0.3, 0.0)])
+def test_return_map_series_and_eigenvectors_vs_oracle(orc, otm, model, strain, pressure):
+    """Points on both sides of the bound |dev b| <= 1/32 between the series form and the eigen decomposition
+    (strain 0.007 and 0.012 straddle it), under pressure, at rest, virgin and hardened, cold, hot and
+    melted. Stress bound: the FP64 rounding of b^e about 1 is 1.1e-16, seen through the moduli (largest
+    of K and 2 mu) in either implementation, times 20 for the sums; plus 1e-10 of the stress, the bar of
+    the other return map tests."""
+    mat = {"j2": scenarios.copper_j2, "jc": scenarios.copper_jc, "ti64": scenarios.ti64_jc}[model]()
+    rng = np.random.default_rng(11)
+    n, dt = 300, 5e-9
+    dF = np.eye(3) + rng.normal(0, 1, (n, 3, 3)) * 0.3 * strain
+    F = dF @ (np.eye(3) + rng.normal(0, 0.02, (n, 3, 3)))
+    be = np.concatenate([1 + pressure + rng.normal(0, 1, (n, 3)) * strain, rng.normal(0, 0.5, (n, 3)) * strain], 1)
+    be[:, :3] = np.maximum(be[:, :3], 0.2)
+    ebar = np.where(rng.uniform(size=n) < 0.3, 0.0, np.abs(rng.normal(0, 0.1, n)))
+    T = rng.choice([mat.T_room, mat.T_room + 60.0, 0.5 * (mat.T_room + mat.T_melt), mat.T_melt, mat.T_melt + 40.0], n)
+    ref = [orc.return_map(mat, dt, dF[k], be[k], ebar[k], T[k], np.linalg.det(F[k])) for k in range(n)]
+    good = np.array([r[0] == 0 for r in ref])
+    assert good.mean() > 0.5
+    dF, F, be, ebar, T = dF[good], F[good], be[good], ebar[good], T[good]
+    ref = [r for r in ref if r[0] == 0]
+    be_t, eb_t, T_t = dev(be.copy()), dev(ebar.copy()), dev(T.copy())
+    sig, rate, failed, status = otm.return_map(mat, dt, dev(dF.reshape(-1, 9)), dev(F.reshape(-1, 9)), be_t, eb_t, T_t)
+    assert status.item() == 0
+    K, mu = mat.E / (3 * (1 - 2 * mat.nu)), mat.E / (2 * (1 + mat.nu))
+    s_ref = np.array([r[1] for r in ref])
+    floor = 20 * 1.1e-16 * max(K, 2 * mu)
+    J = np.abs(np.linalg.det(F)).min()
+    assert np.abs(sig.cpu().numpy() - s_ref).max() <= floor / J + 1e-10 * np.abs(s_ref).max()
+    assert rel(be_t.cpu().numpy(), np.array([r[2] for r in ref])) <= 1e-13 + 1e-10 * strain
+    assert np.abs(eb_t.cpu().numpy() - np.array([r[3] for r in ref])).max() <= 20 * 1.1e-16 + 1e-10 * max(strain, ebar.max())
+    assert rel(T_t.cpu().numpy(), np.array([r[4] for r in ref])) <= 1e-10
+    assert np.array_equal(failed.cpu().numpy().astype(bool), np.array([r[6] for r in ref]))
+
+
+def test_return_map_bad_input_reports_the_same_errors(otm):
+    """Non-finite and inverted input leaves the series form for the eigen decomposition and its codes."""
+    n = 4
+    eye = torch.eye(3, dtype=torch.float64, device="cuda").reshape(1, 9).repeat(n, 1)
+    be0 = torch.tensor([1.0, 1, 1, 0, 0, 0], dtype=torch.float64, device="cuda").repeat(n, 1)
+    z = torch.zeros(n, dtype=torch.float64, device="cuda")
+    for bad, code in ((float("nan"), -5), (-3.0, -5)):
+        be = be0.clone()
+        be[2, 0] = bad
+        _, _, _, st = otm.return_map(scenarios.copper_jc(), 5e-9, eye, eye.clone(), be, z.clone(), z + 300.0)
+        assert st.item() == code
+    F = eye.clone()
+    F[1] = 0.0
+    _, _, _, st = otm.return_map(scenarios.copper_jc(), 5e-9, eye, F, be0.clone() * 1.001, z.clone(), z + 300.0)
+    assert st.item() == -6
