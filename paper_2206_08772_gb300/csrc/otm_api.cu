@@ -693,7 +693,10 @@ extern "C" int otm_state(otm_handle *h, int32_t field, void *host_dst, size_t by
         CK(cudaMemcpy(cnt.data(), h->D.cnt, nm * sizeof(int32_t), cudaMemcpyDeviceToHost));
         if (field == OTM_FIELD_SUPPORT_IDS) {
             int32_t *row = (int32_t *)host_dst;
-            for (size_t p = 0; p < nm; p++) std::sort(row + p * S, row + p * S + cnt[p]);
+            for (size_t p = 0; p < nm; p++) {
+                std::sort(row + p * S, row + p * S + cnt[p]);
+                std::fill(row + p * S + cnt[p], row + (p + 1) * S, 0);   // unused slots: whatever the memory held
+            }
         } else {
             ids.resize(nm * S);
             CK(cudaMemcpy(ids.data(), h->D.ids, nm * S * sizeof(int32_t), cudaMemcpyDeviceToHost));
@@ -712,6 +715,7 @@ extern "C" int otm_state(otm_handle *h, int32_t field, void *host_dst, size_t by
                 tmp.assign(sh + 4 * p * S, sh + 4 * (p * S + n));
                 for (int k = 0; k < n; k++)
                     for (int c = 0; c < 4; c++) sh[4 * (p * S + k) + c] = tmp[4 * perm[k] + c];
+                std::fill(sh + 4 * (p * S + n), sh + 4 * (p + 1) * S, 0.0);
             }
         }
     }
@@ -740,6 +744,7 @@ extern "C" int otm_state_rows(otm_handle *h, int32_t field, const int64_t *rows,
             if (field == OTM_FIELD_SUPPORT_IDS) {
                 int32_t *row = (int32_t *)host_dst + (size_t)r * S;
                 std::sort(row, row + n);
+                std::fill(row + n, row + S, 0);
             } else {
                 CK(cudaMemcpy(ids.data(), h->D.ids + (size_t)rows[r] * S, S * sizeof(int32_t), cudaMemcpyDeviceToHost));
                 double K[6];
@@ -752,6 +757,7 @@ extern "C" int otm_state_rows(otm_handle *h, int32_t field, const int64_t *rows,
                 std::vector<double> tmp(sh, sh + 4 * (size_t)n);
                 for (int k = 0; k < n; k++)
                     for (int c = 0; c < 4; c++) sh[4 * k + c] = tmp[4 * perm[k] + c];
+                std::fill(sh + 4 * (size_t)n, sh + 4 * S, 0.0);
             }
         }
     }
