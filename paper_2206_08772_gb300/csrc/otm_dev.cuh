@@ -304,6 +304,13 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
+__device__ __forceinline__ float warp_max_f(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
 // linked-cell coordinate: floor((x - o) / c) in correctly rounded FP64 (bit-identical to any
 // IEEE implementation of the same expression), optionally clamped to the grid.
 __device__ __forceinline__ int cell_coord(double x, double o, double c, int n, bool clamp)

@@ -113,6 +113,21 @@ OTM_HD i64 fix_from_double(double x, int fb)
     return (b >> 63) ? -(i64)r : (i64)r;
 }
 
+// the same without losing the high words: the value is hi 2^64 + (u64)lo (for points whose distances are
+// not known to fit 64 bits); false for |x| 2^fb of 2^116 or more and for non-finite x
+OTM_HD bool fix_from_double_wide(double x, int fb, i64 &lo, i64 &hi)
+{
+    const u64 b = fx_d_bits(x);
+    const int ef = (int)((b >> 52) & 0x7ff);
+    const u64 m = (b & 0xfffffffffffffULL) | (ef ? 0x10000000000000ULL : 0ULL);
+    const int s = (ef ? ef : 1) - 1075 + fb;
+    const u64 sg = 0ULL - (b >> 63);
+    lo = fix_from_double(x, fb);
+    const u64 h = (s > 11 && s < 64) ? m >> (64 - s) : 0ULL;      // high word of the magnitude
+    hi = (i64)((h ^ sg) + ((sg && lo == 0) ? 1ULL : 0ULL));       // two's complement of (h, |lo|)
+    return s < 64;
+}
+
 // exp: 2^(j/1024) (j = 0..1023) as 64-bit mantissas in [2^63, 2^64) come from a table; the rest
 // s = fraction of the 1024th, 44 bits in [0, 1), goes through exp(s ln2/1024) - 1 by its Taylor
 // polynomial of degree 4 (truncation below 2e-18) in fixed point.

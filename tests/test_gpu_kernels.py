@@ -334,3 +334,33 @@ def test_return_map_bad_input_reports_the_same_errors(otm):
     F[1] = 0.0
     _, _, _, st = otm.return_map(scenarios.copper_jc(), 5e-9, eye, F, be0.clone() * 1.001, z.clone(), z + 300.0)
     assert st.item() == -6
+
+
+@pytest.mark.parametrize("n,far", [(4, 0.0), (31, 0.0), (33, 0.0), (336, 0.0), (337, 0.0), (400, 0.0), (40, 30.0)])
+def test_lme_support_sizes_and_ranges(orc, otm, n, far):
+    """The stand-alone LME at the edges of its fixed-point form: 32-lane passes, 336 shared slots, and one node
+    30 spacings away (outside the fixed-point range), each with a start far from the solution for
+    half of the points. Bound: both solves stop at |r| <= 1e-14 h, 1e-12 on N as in the step's test."""
+    h = 1.3e-3
+    rng = np.random.default_rng(n)
+    g = np.stack(np.meshgrid(*[np.arange(-5, 6)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    g = g[np.argsort((g ** 2).sum(1), kind="stable")]
+    if n == 4:
+        g = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0], [0, 0, 1]])
+    x = (g[:n] + rng.uniform(-0.02, 0.02, (n, 3))) * h + 0.5
+    if far:
+        x[-1] = x[0] + far * h
+    xp = 0.5 + rng.uniform(0.1, 0.3, (12, 3)) * h
+    S, tol, beta = 416, 1e-14 * h, 0.8 / h ** 2
+    ids = np.zeros((12, S), np.int32)
+    ids[:, :n] = rng.permutation(n)
+    lam0 = np.where(np.arange(12)[:, None] % 2, 0.4 / h, 0.0) * np.ones((12, 3))
+    shape, lam, iters, st = otm.lme(dev(x), dev(xp), dev(ids), dev(np.full(12, n, np.int32)), beta, tol,
+                                    lam0=dev(lam0))
+    assert st.item() == 0
+    sh = shape.cpu().numpy()
+    for p in range(12):
+        so, N, dN, _, _ = orc.lme(xp[p] - x[ids[p, :n]], beta, tol)
+        assert so == 0
+        assert rel(sh[p, :n, 0], N) <= 1e-12 and rel(sh[p, :n, 1:], dN) <= 1e-11
+        assert not sh[p, n:].any()
