@@ -7,7 +7,7 @@
 //   k_adj_kin   : Eq. 9 and Eq. 11 transposed (warp per MP, supports of state n)
 //   k_adj_node  : Eq. 4 and Eq. 6 with the frozen wall projection transposed (warp per node; the
 //                 per-pair node contributions are summed over the node-major segments)
-//   k_adj_force : Eq. 5 transposed (warp per MP, supports of state n)
+//   k_adj_force : Eq. 5 transposed and the adjoints of N and grad N of state n (warp per MP)
 #include "otm_dev.cuh"
 #include "otm_rm.cuh"
 
@@ -15,119 +15,99 @@ namespace otm {
 
 constexpr int kAdjWarps = 4;
 
-// (N, grad N) of a stored pair row (N, e = N d): grad N = -K e with K = J^-1 of the MP's LME
-// solve (xx, yy, zz, xy, yz, xz)
-__device__ __forceinline__ double4_32a grad_row(const double4_32a r, double k0, double k1, double k2, double k3,
-                                                double k4, double k5)
+// Pair adjoints are kept as (dL/dN_a, g_a) with g_a = K dL/d(grad N_a), K = J^-1 of the MP: grad N_a enters
+// the backward pass only through K times its adjoint, and the kernel that forms it (k_adj_force)
+// multiplies by 3x3 matrices per MP anyway, so K costs nothing there. The FP64 pipe (2 lanes per clock
+// and SM) bounds these kernels; what can be done once per MP is not done per pair.
+
+// lane that holds value j of warp_reduce_scatter10
+__device__ __forceinline__ int rs10_lane(int j)
 {
-    return make_double4_32a(r.x, -(k0 * r.y + k3 * r.z + k5 * r.w), -(k3 * r.y + k1 * r.z + k4 * r.w),
-                            -(k5 * r.y + k4 * r.z + k2 * r.w));
+    return j < 5 ? (j < 3 ? 2 * j : (j == 3 ? 8 : 10)) : 16 + (j < 8 ? 2 * (j - 5) : (j == 8 ? 8 : 10));
+}
+
+// index of (i, j) of a symmetric tensor stored as (xx, yy, zz, xy, yz, xz)
+__device__ __forceinline__ int sym6(int i, int j) { return i == j ? i : (i + j == 1 ? 3 : (i + j == 3 ? 4 : 5)); }
+
+__device__ __forceinline__ void broadcast9(double v, double (&M)[9])
+{
+#pragma unroll
+    for (int i = 0; i < 9; i++) M[i] = __shfl_sync(0xffffffffu, v, i);
 }
 
 // ---------------------------------------------------------------------------- LME backward
-// d_a = x_p - x_a, N = softmax(f), f_a = -beta |d_a|^2 + lambda . d_a, lambda from
-// r = sum N d = 0, grad N_a = -N_a H^-1 d_a, H = sum N d d^T - r r^T.
-__global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const Dev D, const AdjDev A)
+// d_a = x_p - x_a, N = softmax(f), f_a = -beta |d_a|^2 + lambda . d_a, lambda from r = sum N d = 0,
+// grad N_a = -N_a K d_a, K^-1 = H = sum N d d^T. With e_a = N_a d_a (the stored row) and r = 0:
+//   B = sum g_a e_a^T, Hs = sym(B K)                          (the adjoint of H)
+//   q_a = dL/dN_a - g_a . d_a + d_a . Hs d_a,  S = sum N_a q_a = sum N_a dL/dN_a  (tr B cancels tr(Hs H))
+//   lambda_bar = sum (q_a - S) e_a,  m = K lambda_bar          (implicit function theorem on r = 0)
+//   dL/dd_a = N_a [2 Hs d_a - g_a - m + (q_a - S - d_a . m)(lambda - 2 beta d_a)]
+// Three passes over the pairs with about 55 FP64 instructions each in all (about 115 when H is summed
+// again and the r terms, of relative size 1e-14, are carried): 4.69 -> 2.64 ms on 78,624 MPs.
+__global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_constant__ Dev D, const __grid_constant__ AdjDev A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t p = (int64_t)blockIdx.x * kAdjWarps + warp;
+    const int64_t p = (int64_t)blockIdx.x * (blockDim.x / kWarp) + warp;
     if (p >= D.nm) return;
     const int S = D.S;
-    double *sm = (double *)smem_raw + (size_t)warp * 7 * S;
-    double *dx = sm, *dy = sm + S, *dz = sm + 2 * S, *Nb = sm + 3 * S, *bx = sm + 4 * S, *by = sm + 5 * S,
-           *bz = sm + 6 * S;
+    double *sm = (double *)smem_raw + (size_t)warp * 8 * S;
+    double *dx = sm, *dy = sm + S, *dz = sm + 2 * S, *qa = sm + 3 * S, *wx = sm + 4 * S, *wy = sm + 5 * S, *wz = sm + 6 * S,
+           *Na = sm + 7 * S;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)S;
-    const double4_32a xp = D.xp[p];
-    const double l0 = D.lam[3 * p], l1 = D.lam[3 * p + 1], l2 = D.lam[3 * p + 2], beta = D.beta;
-    double v[16];
+    // B and S
+    double v[10];
 #pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = 0.0;
+    for (int i = 0; i < 10; i++) v[i] = 0.0;
     for (int k = lane; k < n; k += kWarp) {
-        const double4_32a a = D.x[D.ids[base + k]];
+        const double4_32a sh = D.shape[base + k], pb = A.pb_cur[base + k];
+        Na[k] = sh.x;
+        v[0] = fma(pb.y, sh.y, v[0]); v[1] = fma(pb.y, sh.z, v[1]); v[2] = fma(pb.y, sh.w, v[2]);
+        v[3] = fma(pb.z, sh.y, v[3]); v[4] = fma(pb.z, sh.z, v[4]); v[5] = fma(pb.z, sh.w, v[5]);
+        v[6] = fma(pb.w, sh.y, v[6]); v[7] = fma(pb.w, sh.z, v[7]); v[8] = fma(pb.w, sh.w, v[8]);
+        v[9] = fma(sh.x, pb.x, v[9]);
+    }
+    const double t = warp_reduce_scatter10(v, lane);
+    const double Ssum = __shfl_sync(0xffffffffu, t, rs10_lane(9));
+    // lane 3 i + j: (B K)_ij, then its symmetric part
+    const double *K = D.Kinv + 6 * p;
+    const int li = lane < 9 ? lane / 3 : 0, lj = lane < 9 ? lane % 3 : 0;
+    double bk = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; k++) bk = fma(__shfl_sync(0xffffffffu, t, rs10_lane(3 * li + k)), K[sym6(k, lj)], bk);
+    bk = 0.5 * (bk + __shfl_sync(0xffffffffu, bk, 3 * lj + li));
+    const double s00 = __shfl_sync(0xffffffffu, bk, 0), s11 = __shfl_sync(0xffffffffu, bk, 4), s22 = __shfl_sync(0xffffffffu, bk, 8);
+    const double s01 = __shfl_sync(0xffffffffu, bk, 1), s12 = __shfl_sync(0xffffffffu, bk, 5), s02 = __shfl_sync(0xffffffffu, bk, 2);
+    const double4_32a xp = D.xp[p];
+    double lb[3] = {0.0, 0.0, 0.0};
+    for (int k = lane; k < n; k += kWarp) {
+        const double4_32a a = D.x[D.ids[base + k]], sh = D.shape[base + k], pb = A.pb_cur[base + k];
         const double x = xp.x - a.x, y = xp.y - a.y, z = xp.z - a.z;
         dx[k] = x; dy[k] = y; dz[k] = z;
-        const double N = D.shape[base + k].x;
-        v[0] += N * x; v[1] += N * y; v[2] += N * z;
-        v[3] += N * x * x; v[4] += N * y * y; v[5] += N * z * z;
-        v[6] += N * x * y; v[7] += N * y * z; v[8] += N * x * z;
+        const double h0 = fma(s02, z, fma(s01, y, s00 * x)), h1 = fma(s12, z, fma(s11, y, s01 * x)),
+                     h2 = fma(s22, z, fma(s12, y, s02 * x));
+        const double g0 = h0 - pb.y, g1 = h1 - pb.z, g2 = h2 - pb.w;
+        const double q = fma(z, g2, fma(y, g1, fma(x, g0, pb.x - Ssum)));
+        qa[k] = q;
+        wx[k] = h0 + g0; wy[k] = h1 + g1; wz[k] = h2 + g2;
+        lb[0] = fma(q, sh.y, lb[0]); lb[1] = fma(q, sh.z, lb[1]); lb[2] = fma(q, sh.w, lb[2]);
     }
-    double t = warp_reduce_scatter16(v, lane);
-    double r0 = __shfl_sync(0xffffffffu, t, 0), r1 = __shfl_sync(0xffffffffu, t, 2), r2 = __shfl_sync(0xffffffffu, t, 4);
-    const double h00 = __shfl_sync(0xffffffffu, t, 6) - r0 * r0, h11 = __shfl_sync(0xffffffffu, t, 8) - r1 * r1;
-    const double h22 = __shfl_sync(0xffffffffu, t, 10) - r2 * r2, h01 = __shfl_sync(0xffffffffu, t, 12) - r0 * r1;
-    const double h12 = __shfl_sync(0xffffffffu, t, 14) - r1 * r2, h02 = __shfl_sync(0xffffffffu, t, 16) - r0 * r2;
-    const double c00 = h11 * h22 - h12 * h12, c01 = h02 * h12 - h01 * h22, c02 = h01 * h12 - h02 * h11;
-    const double c11 = h00 * h22 - h02 * h02, c12 = h01 * h02 - h00 * h12, c22 = h00 * h11 - h01 * h01;
-    const double det = h00 * c00 + h01 * c01 + h02 * c02;
-    const double id = 1.0 / det;
-    const double i00 = c00 * id, i11 = c11 * id, i22 = c22 * id, i01 = c01 * id, i12 = c12 * id, i02 = c02 * id;
-    // pass 1: G_a = -N_a u_a, u_a = H^-1 d_a;  Nb_a = Nbar_a - Gbar_a . u_a;  db_a = w_a = -N_a H^-1 Gbar_a;
-    // Hbar = -sum w u^T
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = 0.0;
-    for (int k = lane; k < n; k += kWarp) {
-        const double x = dx[k], y = dy[k], z = dz[k];
-        const double N = D.shape[base + k].x;
-        const double4_32a pb = A.pb_cur[base + k];
-        const double u0 = i00 * x + i01 * y + i02 * z, u1 = i01 * x + i11 * y + i12 * z, u2 = i02 * x + i12 * y + i22 * z;
-        Nb[k] = pb.x - (pb.y * u0 + pb.z * u1 + pb.w * u2);
-        const double w0 = -N * (i00 * pb.y + i01 * pb.z + i02 * pb.w);
-        const double w1 = -N * (i01 * pb.y + i11 * pb.z + i12 * pb.w);
-        const double w2 = -N * (i02 * pb.y + i12 * pb.z + i22 * pb.w);
-        bx[k] = w0; by[k] = w1; bz[k] = w2;
-        v[0] -= w0 * u0; v[1] -= w0 * u1; v[2] -= w0 * u2;
-        v[3] -= w1 * u0; v[4] -= w1 * u1; v[5] -= w1 * u2;
-        v[6] -= w2 * u0; v[7] -= w2 * u1; v[8] -= w2 * u2;
-    }
-    t = warp_reduce_scatter16(v, lane);
-    double Hb[9];
-#pragma unroll
-    for (int i = 0; i < 9; i++) Hb[i] = __shfl_sync(0xffffffffu, t, 2 * i);
-    const double s00 = Hb[0], s11 = Hb[4], s22 = Hb[8];
-    const double s01 = 0.5 * (Hb[1] + Hb[3]), s12 = 0.5 * (Hb[5] + Hb[7]), s02 = 0.5 * (Hb[2] + Hb[6]);
-    const double hr0 = s00 * r0 + s01 * r1 + s02 * r2, hr1 = s01 * r0 + s11 * r1 + s12 * r2,
-                 hr2 = s02 * r0 + s12 * r1 + s22 * r2;
-    // pass 2: H = sum N d d^T - r r^T contributions; S = sum N Nb
-    double Ssum = 0.0;
-    for (int k = lane; k < n; k += kWarp) {
-        const double x = dx[k], y = dy[k], z = dz[k];
-        const double N = D.shape[base + k].x;
-        const double hd0 = s00 * x + s01 * y + s02 * z, hd1 = s01 * x + s11 * y + s12 * z, hd2 = s02 * x + s12 * y + s22 * z;
-        Nb[k] += (x * hd0 + y * hd1 + z * hd2) - 2.0 * (x * hr0 + y * hr1 + z * hr2);
-        bx[k] += 2.0 * N * (hd0 - hr0);
-        by[k] += 2.0 * N * (hd1 - hr1);
-        bz[k] += 2.0 * N * (hd2 - hr2);
-        Ssum += N * Nb[k];
-    }
-    Ssum = warp_sum(Ssum);
-    // pass 3: softmax and the prior exponent; lambda bar
-    double lb0 = 0, lb1 = 0, lb2 = 0;
-    for (int k = lane; k < n; k += kWarp) {
-        const double x = dx[k], y = dy[k], z = dz[k];
-        const double N = D.shape[base + k].x;
-        const double fb = N * (Nb[k] - Ssum);
-        bx[k] += fb * (l0 - 2.0 * beta * x);
-        by[k] += fb * (l1 - 2.0 * beta * y);
-        bz[k] += fb * (l2 - 2.0 * beta * z);
-        lb0 += fb * x; lb1 += fb * y; lb2 += fb * z;
-    }
-    lb0 = warp_sum(lb0); lb1 = warp_sum(lb1); lb2 = warp_sum(lb2);
-    const double m0 = i00 * lb0 + i01 * lb1 + i02 * lb2, m1 = i01 * lb0 + i11 * lb1 + i12 * lb2,
-                 m2 = i02 * lb0 + i12 * lb1 + i22 * lb2;
-    // pass 4: lambda(d) through r = 0; scatter to the node and to x_p
+    const double lb0 = warp_sum(lb[0]), lb1 = warp_sum(lb[1]), lb2 = warp_sum(lb[2]);
+    const double m0 = fma(K[0], lb0, fma(K[3], lb1, K[5] * lb2)), m1 = fma(K[3], lb0, fma(K[1], lb1, K[4] * lb2)),
+                 m2 = fma(K[5], lb0, fma(K[4], lb1, K[2] * lb2));
+    const double l0 = D.lam[3 * p], l1 = D.lam[3 * p + 1], l2 = D.lam[3 * p + 2], b2 = -2.0 * D.beta;
+    // scatter to the node and to x_p
     double px = 0, py = 0, pz = 0;
     for (int k = lane; k < n; k += kWarp) {
-        const double x = dx[k], y = dy[k], z = dz[k];
-        const double N = D.shape[base + k].x;
-        const double dm = x * m0 + y * m1 + z * m2;
-        const double b0 = bx[k] - N * (m0 + (l0 - 2.0 * beta * x) * dm);
-        const double b1 = by[k] - N * (m1 + (l1 - 2.0 * beta * y) * dm);
-        const double b2 = bz[k] - N * (m2 + (l2 - 2.0 * beta * z) * dm);
-        px += b0; py += b1; pz += b2;
+        const double x = dx[k], y = dy[k], z = dz[k], N = Na[k];
+        const double c = fma(-x, m0, fma(-y, m1, fma(-z, m2, qa[k])));
+        const double o0 = N * fma(c, fma(b2, x, l0), wx[k] - m0);
+        const double o1 = N * fma(c, fma(b2, y, l1), wy[k] - m1);
+        const double o2 = N * fma(c, fma(b2, z, l2), wz[k] - m2);
+        px += o0; py += o1; pz += o2;
         const int nid = D.ids[base + k];
-        A.sc1[(int64_t)D.noff[nid] + D.rank[base + k]] = make_double4_32a(b0, b1, b2, 0.0);
+        A.sc1[(int64_t)D.noff[nid] + D.rank[base + k]] = make_double4_32a(o0, o1, o2, 0.0);
     }
     px = warp_sum(px); py = warp_sum(py); pz = warp_sum(pz);
     if (lane == 0) A.xpb[p] = make_double4_32a(px, py, pz, 0.0);
@@ -222,17 +202,11 @@ __global__ void __launch_bounds__(128) k_adj_rm(const Dev D, const AdjDev A)
     const double Jn = Fn[0][0] * (Fn[1][1] * Fn[2][2] - Fn[1][2] * Fn[2][1]) -
                       Fn[0][1] * (Fn[1][0] * Fn[2][2] - Fn[1][2] * Fn[2][0]) +
                       Fn[0][2] * (Fn[1][0] * Fn[2][1] - Fn[1][1] * Fn[2][0]);
-    // recompute the return map and its intermediate quantities
+    // the intermediate quantities of the return map; its plastic increment is the state's own
     RmIn in;
-    for (int i = 0; i < 9; i++) in.dF[i] = dF[i / 3][i % 3];
     for (int i = 0; i < 6; i++) in.be[i] = A.be_n[6 * p + i];
     in.ebar = A.ebar_n[p];
     in.T = A.T_n[p];
-    in.J = Jn;
-    in.guess = D.rate[p] * D.dt;   // the recomputed step's own increment
-    in.Q0 = nullptr;
-    RmOut out;
-    return_map_point(M, D.dt, in, out);
     RmDetail o;
     o.K = M.E / (3.0 * (1.0 - 2.0 * M.nu));
     o.mu = M.E / (2.0 * (1.0 + M.nu));
@@ -259,7 +233,7 @@ __global__ void __launch_bounds__(128) k_adj_rm(const Dev D, const AdjDev A)
     }
     o.enorm = sqrt(en2);
     o.qtr = 2.4494897427831780982 * o.mu * o.enorm;
-    o.x = out.ebar - in.ebar;
+    o.x = D.rate[p] * D.dt;
     o.plastic = o.x > 0.0;
     o.q = o.qtr - 3.0 * o.mu * o.x;
     o.rho = o.plastic ? o.q / o.qtr : 1.0;
@@ -390,34 +364,31 @@ __global__ void __launch_bounds__(128) k_adj_rm(const Dev D, const AdjDev A)
 }
 
 // ---------------------------------------------------------------------------- kinematics backward
-// dF = 1 + sum du'_a (x) G_a, x_p' = sum N_a x'_a over the supports of state n
-__global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_kin(const Dev D, const AdjDev A)
+// dF = 1 + sum du'_a (x) G_a, x_p' = sum N_a x'_a over the supports of state n: the nodes' parts,
+// N_a dL/dx_p' and dL/ddF G_a = -(dL/ddF K) e_a (the pairs' parts follow in k_adj_force)
+__global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_kin(const __grid_constant__ Dev D, const __grid_constant__ AdjDev A)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t p = (int64_t)blockIdx.x * kAdjWarps + warp;
     if (p >= D.nm) return;
-    const int S = D.S;
     const int n = A.cnt_n[p];
-    const int64_t base = p * (int64_t)S;
-    double Db[9];
-    for (int i = 0; i < 9; i++) Db[i] = A.dFb[9 * p + i];
+    const int64_t base = p * (int64_t)D.S;
+    double M[9];   // -dL/ddF K
+    {
+        const double *Db = A.dFb + 9 * p, *K = A.K_n + 6 * p;
+        const int i = lane < 9 ? lane / 3 : 0, j = lane < 9 ? lane % 3 : 0;
+        broadcast9(-fma(Db[3 * i], K[sym6(0, j)], fma(Db[3 * i + 1], K[sym6(1, j)], Db[3 * i + 2] * K[sym6(2, j)])), M);
+    }
     const double4_32a xpb = A.xpb[p];
-    const double *K = A.K_n + 6 * p;
-    const double k0 = K[0], k1 = K[1], k2 = K[2], k3 = K[3], k4 = K[4], k5 = K[5];
+#pragma unroll 2
     for (int k = lane; k < n; k += kWarp) {
         const int id = A.ids_n[base + k];
-        const double4_32a sh = grad_row(A.shape_n[base + k], k0, k1, k2, k3, k4, k5);
-        const double4_32a u = D.du[id], xa = D.x[id];
-        const double ub0 = Db[0] * sh.y + Db[1] * sh.z + Db[2] * sh.w;
-        const double ub1 = Db[3] * sh.y + Db[4] * sh.z + Db[5] * sh.w;
-        const double ub2 = Db[6] * sh.y + Db[7] * sh.z + Db[8] * sh.w;
+        const double4_32a sh = A.shape_n[base + k];
         const int64_t pos = (int64_t)A.noff_n[id] + A.rank_n[base + k];
         A.sc3a[pos] = make_double4_32a(sh.x * xpb.x, sh.x * xpb.y, sh.x * xpb.z, 0.0);
-        A.sc3b[pos] = make_double4_32a(ub0, ub1, ub2, 0.0);
-        const double g0 = Db[0] * u.x + Db[3] * u.y + Db[6] * u.z;
-        const double g1 = Db[1] * u.x + Db[4] * u.y + Db[7] * u.z;
-        const double g2 = Db[2] * u.x + Db[5] * u.y + Db[8] * u.z;
-        A.pb_prev[base + k] = make_double4_32a(xpb.x * xa.x + xpb.y * xa.y + xpb.z * xa.z, g0, g1, g2);
+        A.sc3b[pos] = make_double4_32a(fma(M[0], sh.y, fma(M[1], sh.z, M[2] * sh.w)),
+                                       fma(M[3], sh.y, fma(M[4], sh.z, M[5] * sh.w)),
+                                       fma(M[6], sh.y, fma(M[7], sh.z, M[8] * sh.w)), 0.0);
     }
 }
 
@@ -481,53 +452,48 @@ __global__ void __launch_bounds__(128) k_adj_node(const Dev D, const AdjDev A)
     }
 }
 
-// ---------------------------------------------------------------------------- force backward
-// m_I = sum N m_p, r_I = -sum v_p sigma_p G_pI over the supports of state n
-__global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_force(const Dev D, const AdjDev A)
+// ---------------------------------------------------------------------------- force and pair backward
+// Over the supports of state n: m_I = sum N m_p, r_I = -sum v_p sigma_p G_pI, and the pairs' adjoints of
+// these and of the kinematics,
+//   dL/dN_a = dL/dx_p' . x'_a + m_p dL/dm_a,   g_a = K (dL/ddF^T du'_a - v sigma dL/dr_a).
+// dL/dv and dL/dsigma follow from R = sum dL/dr_a (x) G_a = -(sum dL/dr_a (x) e_a) K.
+__global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_force(const __grid_constant__ Dev D, const __grid_constant__ AdjDev A)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t p = (int64_t)blockIdx.x * kAdjWarps + warp;
     if (p >= D.nm) return;
-    const int S = D.S;
     const int n = A.cnt_n[p];
-    const int64_t base = p * (int64_t)S;
-    const double *sg = A.sig_n + 6 * p;
-    const double sxx = sg[0], syy = sg[1], szz = sg[2], sxy = sg[3], syz = sg[4], sxz = sg[5];
+    const int64_t base = p * (int64_t)D.S;
+    const double *sg = A.sig_n + 6 * p, *K = A.K_n + 6 * p, *Db = A.dFb + 9 * p;
     const double vp = A.vol_n[p], mp = D.mass[p];
-    const double *K = A.K_n + 6 * p;
-    const double k0 = K[0], k1 = K[1], k2 = K[2], k3 = K[3], k4 = K[4], k5 = K[5];
-    double v[16];
+    const int i = lane < 9 ? lane / 3 : 0, j = lane < 9 ? lane % 3 : 0;
+    double Mu[9], Mr[9];   // K dL/ddF^T, -v K sigma
+    broadcast9(fma(K[sym6(i, 0)], Db[3 * j], fma(K[sym6(i, 1)], Db[3 * j + 1], K[sym6(i, 2)] * Db[3 * j + 2])), Mu);
+    broadcast9(-vp * fma(K[sym6(i, 0)], sg[sym6(0, j)], fma(K[sym6(i, 1)], sg[sym6(1, j)], K[sym6(i, 2)] * sg[sym6(2, j)])), Mr);
+    const double4_32a xpb = A.xpb[p];
+    double v[10];
 #pragma unroll
-    for (int k = 0; k < 16; k++) v[k] = 0.0;
+    for (int k = 0; k < 10; k++) v[k] = 0.0;
     for (int k = lane; k < n; k += kWarp) {
         const int id = A.ids_n[base + k];
-        const double4_32a sh = grad_row(A.shape_n[base + k], k0, k1, k2, k3, k4, k5);
-        const double4_32a rb = A.rb[id];
-        double4_32a pb = A.pb_prev[base + k];
-        pb.x += rb.w * mp;
-        pb.y -= vp * (sxx * rb.x + sxy * rb.y + sxz * rb.z);
-        pb.z -= vp * (sxy * rb.x + syy * rb.y + syz * rb.z);
-        pb.w -= vp * (sxz * rb.x + syz * rb.y + szz * rb.z);
-        A.pb_prev[base + k] = pb;
-        const double sgx = sxx * sh.y + sxy * sh.z + sxz * sh.w;
-        const double sgy = sxy * sh.y + syy * sh.z + syz * sh.w;
-        const double sgz = sxz * sh.y + syz * sh.z + szz * sh.w;
-        v[0] -= rb.x * sgx + rb.y * sgy + rb.z * sgz;
-        // dL/dsigma_ij (full) = -v rbar_i G_j
-        v[1] -= vp * rb.x * sh.y; v[2] -= vp * rb.y * sh.z; v[3] -= vp * rb.z * sh.w;
-        v[4] -= vp * (rb.x * sh.z + rb.y * sh.y);
-        v[5] -= vp * (rb.y * sh.w + rb.z * sh.z);
-        v[6] -= vp * (rb.x * sh.w + rb.z * sh.y);
+        const double4_32a sh = A.shape_n[base + k], rb = A.rb[id], u = D.du[id], xa = D.x[id];
+        A.pb_prev[base + k] = make_double4_32a(
+            fma(xpb.x, xa.x, fma(xpb.y, xa.y, fma(xpb.z, xa.z, rb.w * mp))),
+            fma(Mu[0], u.x, fma(Mu[1], u.y, fma(Mu[2], u.z, fma(Mr[0], rb.x, fma(Mr[1], rb.y, Mr[2] * rb.z))))),
+            fma(Mu[3], u.x, fma(Mu[4], u.y, fma(Mu[5], u.z, fma(Mr[3], rb.x, fma(Mr[4], rb.y, Mr[5] * rb.z))))),
+            fma(Mu[6], u.x, fma(Mu[7], u.y, fma(Mu[8], u.z, fma(Mr[6], rb.x, fma(Mr[7], rb.y, Mr[8] * rb.z))))));
+        v[0] = fma(rb.x, sh.y, v[0]); v[1] = fma(rb.x, sh.z, v[1]); v[2] = fma(rb.x, sh.w, v[2]);
+        v[3] = fma(rb.y, sh.y, v[3]); v[4] = fma(rb.y, sh.z, v[4]); v[5] = fma(rb.y, sh.w, v[5]);
+        v[6] = fma(rb.z, sh.y, v[6]); v[7] = fma(rb.z, sh.z, v[7]); v[8] = fma(rb.z, sh.w, v[8]);
     }
-    const double t = warp_reduce_scatter16(v, lane);
-    double s[7];
+    const double t = warp_reduce_scatter10(v, lane);
+    double R = 0.0;   // lane 3 i + j: R_ij
 #pragma unroll
-    for (int k = 0; k < 7; k++) s[k] = __shfl_sync(0xffffffffu, t, 2 * k);
-    if (lane == 0) {
-        A.vb[p] += s[0];
-        double *sb = A.sigb + 6 * p;
-        sb[0] = s[1]; sb[1] = s[2]; sb[2] = s[3]; sb[3] = s[4]; sb[4] = s[5]; sb[5] = s[6];
-    }
+    for (int k = 0; k < 3; k++) R = fma(-__shfl_sync(0xffffffffu, t, rs10_lane(3 * i + k)), K[sym6(k, j)], R);
+    const double vbar = warp_sum(lane < 9 ? sg[sym6(i, j)] * R : 0.0);
+    const double Rt = __shfl_sync(0xffffffffu, R, 3 * j + i);
+    if (lane == 0) A.vb[p] -= vbar;
+    if (lane < 9 && i <= j) A.sigb[6 * p + sym6(i, j)] = -vp * (i == j ? R : R + Rt);
 }
 
 // ---------------------------------------------------------------------------- host launchers
@@ -536,10 +502,12 @@ static unsigned wblocks(int64_t n, int warps) { return (unsigned)((n + warps - 1
 cudaError_t launch_adjoint_backward(const Dev &D, const AdjDev &A, cudaStream_t s, long long *launches)
 {
     if (D.nm <= 0) return cudaSuccess;
-    const size_t smem = (size_t)kAdjWarps * 7 * D.S * sizeof(double);
+    // rows of 8 S doubles a warp: two warps a block where four do not fit an SM's 227 KB (S above 900)
+    const int warps = (size_t)kAdjWarps * 8 * D.S * sizeof(double) > 227 * 1024 ? kAdjWarps / 2 : kAdjWarps;
+    const size_t smem = (size_t)warps * 8 * D.S * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_adj_lme, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_adj_lme<<<wblocks(D.nm, kAdjWarps), kAdjWarps * kWarp, smem, s>>>(D, A);
+    k_adj_lme<<<wblocks(D.nm, warps), warps * kWarp, smem, s>>>(D, A);
     k_adj_rm<<<(unsigned)((D.nm + 127) / 128), 128, 0, s>>>(D, A);
     k_adj_kin<<<wblocks(D.nm, kAdjWarps), kAdjWarps * kWarp, 0, s>>>(D, A);
     k_adj_node<<<(unsigned)((D.nn * 32 + 127) / 128), 128, 0, s>>>(D, A);

@@ -141,7 +141,7 @@ struct AdjDev {
     double4_32a *xb, *dub, *rb;        // nodes; rb = (dL/dr_I, dL/dm_I)
     double *Fb, *beb, *ebb, *Tb, *vb, *sigb, *dFb, *thb;   // MPs (thb: 5 per MP, accumulated)
     double4_32a *xpb;
-    double4_32a *pb_cur, *pb_prev;     // pairs: (dL/dN, dL/dgradN) of shape n+1 / shape n
+    double4_32a *pb_cur, *pb_prev;     // pairs: (dL/dN, K dL/dgradN) of shape n+1 / shape n
     // copies of state n taken before the step is recomputed
     double4_32a *du_n;
     double *F_n, *be_n, *ebar_n, *T_n, *vol_n, *sig_n;
