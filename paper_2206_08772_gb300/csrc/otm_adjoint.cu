@@ -48,12 +48,11 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t p = (int64_t)blockIdx.x * (blockDim.x / kWarp) + warp;
+    const int64_t p = (int64_t)blockIdx.x * kAdjWarps + warp;
     if (p >= D.nm) return;
     const int S = D.S;
-    double *sm = (double *)smem_raw + (size_t)warp * 8 * S;
-    double *dx = sm, *dy = sm + S, *dz = sm + 2 * S, *qa = sm + 3 * S, *wx = sm + 4 * S, *wy = sm + 5 * S, *wz = sm + 6 * S,
-           *Na = sm + 7 * S;
+    double *sm = (double *)smem_raw + (size_t)warp * 4 * S;
+    double *qa = sm, *wx = sm + S, *wy = sm + 2 * S, *wz = sm + 3 * S;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)S;
     // B and S
@@ -62,7 +61,6 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
     for (int i = 0; i < 10; i++) v[i] = 0.0;
     for (int k = lane; k < n; k += kWarp) {
         const double4_32a sh = D.shape[base + k], pb = A.pb_cur[base + k];
-        Na[k] = sh.x;
         v[0] = fma(pb.y, sh.y, v[0]); v[1] = fma(pb.y, sh.z, v[1]); v[2] = fma(pb.y, sh.w, v[2]);
         v[3] = fma(pb.z, sh.y, v[3]); v[4] = fma(pb.z, sh.z, v[4]); v[5] = fma(pb.z, sh.w, v[5]);
         v[6] = fma(pb.w, sh.y, v[6]); v[7] = fma(pb.w, sh.z, v[7]); v[8] = fma(pb.w, sh.w, v[8]);
@@ -84,7 +82,6 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
     for (int k = lane; k < n; k += kWarp) {
         const double4_32a a = D.x[D.ids[base + k]], sh = D.shape[base + k], pb = A.pb_cur[base + k];
         const double x = xp.x - a.x, y = xp.y - a.y, z = xp.z - a.z;
-        dx[k] = x; dy[k] = y; dz[k] = z;
         const double h0 = fma(s02, z, fma(s01, y, s00 * x)), h1 = fma(s12, z, fma(s11, y, s01 * x)),
                      h2 = fma(s22, z, fma(s12, y, s02 * x));
         const double g0 = h0 - pb.y, g1 = h1 - pb.z, g2 = h2 - pb.w;
@@ -100,13 +97,14 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
     // scatter to the node and to x_p
     double px = 0, py = 0, pz = 0;
     for (int k = lane; k < n; k += kWarp) {
-        const double x = dx[k], y = dy[k], z = dz[k], N = Na[k];
+        const int nid = D.ids[base + k];
+        const double4_32a a = D.x[nid];
+        const double x = xp.x - a.x, y = xp.y - a.y, z = xp.z - a.z, N = D.shape[base + k].x;
         const double c = fma(-x, m0, fma(-y, m1, fma(-z, m2, qa[k])));
         const double o0 = N * fma(c, fma(b2, x, l0), wx[k] - m0);
         const double o1 = N * fma(c, fma(b2, y, l1), wy[k] - m1);
         const double o2 = N * fma(c, fma(b2, z, l2), wz[k] - m2);
         px += o0; py += o1; pz += o2;
-        const int nid = D.ids[base + k];
         A.sc1[(int64_t)D.noff[nid] + D.rank[base + k]] = make_double4_32a(o0, o1, o2, 0.0);
     }
     px = warp_sum(px); py = warp_sum(py); pz = warp_sum(pz);
@@ -502,12 +500,10 @@ static unsigned wblocks(int64_t n, int warps) { return (unsigned)((n + warps - 1
 cudaError_t launch_adjoint_backward(const Dev &D, const AdjDev &A, cudaStream_t s, long long *launches)
 {
     if (D.nm <= 0) return cudaSuccess;
-    // rows of 8 S doubles a warp: two warps a block where four do not fit an SM's 227 KB (S above 900)
-    const int warps = (size_t)kAdjWarps * 8 * D.S * sizeof(double) > 227 * 1024 ? kAdjWarps / 2 : kAdjWarps;
-    const size_t smem = (size_t)warps * 8 * D.S * sizeof(double);
+    const size_t smem = (size_t)kAdjWarps * 4 * D.S * sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_adj_lme, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_adj_lme<<<wblocks(D.nm, warps), warps * kWarp, smem, s>>>(D, A);
+    k_adj_lme<<<wblocks(D.nm, kAdjWarps), kAdjWarps * kWarp, smem, s>>>(D, A);
     k_adj_rm<<<(unsigned)((D.nm + 127) / 128), 128, 0, s>>>(D, A);
     k_adj_kin<<<wblocks(D.nm, kAdjWarps), kAdjWarps * kWarp, 0, s>>>(D, A);
     k_adj_node<<<(unsigned)((D.nn * 32 + 127) / 128), 128, 0, s>>>(D, A);

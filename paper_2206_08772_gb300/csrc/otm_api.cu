@@ -1165,8 +1165,10 @@ extern "C" int otm_adjoint_begin(otm_handle *h, void *adj_ws, size_t bytes, cons
     h->adj_swap = false;
     h->adj_shape_swap = false;
     h->adj_shape_step = -1;
-    CK(cudaMemsetAsync(adj_ws, 0, need, h->stream));
+    // the adjoint state up to the pair adjoints of the final state starts at zero; what follows is written
+    // by every backward step before it is read
     A = adj_view(h);
+    CK(cudaMemsetAsync(adj_ws, 0, (size_t)((char *)A.pb_prev - (char *)adj_ws), h->stream));
     const int rc = rows_h2d(h, xbar_host, 32, 24, (size_t)h->D.nn, A.xb);
     if (rc != OTM_OK) return rc;
     CK(cudaStreamSynchronize(h->stream));
