@@ -277,6 +277,16 @@ OTM_HD i64 fix_a_about(i64 a, i64 ri, i64 rdj, i64 vi, i64 vj)
     return a + (i64)(((__int128)vi * rdj + (__int128)ri * vj) >> 60);
 }
 
+// floor(v 2^f) for normal or zero v with |v| 2^f < 2^63 (the kinematics gather's row values); whole numbers
+// below zero come out one lower
+OTM_HD i64 fix_floor(double v, int f)
+{
+    const u64 b = fx_d_bits(v);
+    const int s = 1085 - f - (int)((b >> 52) & 0x7ff);       // right shift of the significand 2^10, >= 0
+    const u64 m = ((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 10;
+    return (i64)(m >> (s < 63 ? s : 63)) ^ ((i64)b >> 63);
+}
+
 // N D 2^-fb as FP64 for N > 0 given by its significand nm (in [2^63, 2^64)) and biased exponent en,
 // and 2^32 <= |D| < 2^63: the leading 64 bits of the product (rounded: half a unit is at most one unit
 // of D), normalised and rounded to nearest
@@ -315,5 +325,53 @@ OTM_HD float fix_to_float(i64 D, int fb)
 #endif
     return f;
 }
+
+// ------------------------------------------------------------------ kinematics gather (Eq. 9, 11)
+// The products of a pair's row (N, e) with its node's increment du, summed over the support:
+// sum N du (3) and G = sum du (x) e (9). Limbs: du = uh 2^28 + ul (|du| < 2^57 units; uh 29 bits, ul signed 28
+// bits, kept as 8 ul) and row = rh 2^31 + rl (61 bits; rh 30 bits, rl signed 31 bits), so that both cross
+// products share the unit 2^28. hh += uh rh (2^59), hl += uh rl + ul rh, and ul rl, at most 2^-60 of the largest
+// product, in FP32. With sum N = 1 and |e| <= N r_s the sums of uh rh and ul rh are those of one pair with
+// N = 1; uh rl reaches 12 2^59 in a lane of up to 12 pairs.
+constexpr int kKinDuBits = 57;
+struct KinFixSums {
+    i64 hh[12], hl[12];
+    float ll[12];
+};
+
+// an increment's limbs (uh, 8 ul)
+OTM_HD void kin_fix_split(i64 du, int &uh, int &ul8)
+{
+    uh = (int)((du + (1LL << 27)) >> 28);
+    ul8 = (int)((du - ((i64)uh << 28)) * 8);
+}
+
+// row values in half units: N by fix_floor(N, 62), e by fix_floor(e, fe); rounded here
+OTM_HD void kin_fix_pair(i64 N, i64 e0, i64 e1, i64 e2, const int (&uh)[3], const int (&ul)[3], KinFixSums &s)
+{
+    const i64 r[4] = {N + 1, e0 + 1, e1 + 1, e2 + 1};
+    const float uf[3] = {(float)ul[0], (float)ul[1], (float)ul[2]};
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        const int rh = (int)((r[c] + 0x80000000LL) >> 32), rl = (int)r[c] >> 1;
+        const float rf = (float)rl;
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const int j = c == 0 ? i : 3 + 3 * i + (c - 1);   // 0-2: sum N du_i, 3-11: G row-major
+            s.hh[j] = fx_madw(uh[i], rh, s.hh[j]);
+            s.hl[j] = fx_madw(uh[i], rl, fx_madw(ul[i], rh, s.hl[j]));
+            s.ll[j] += uf[i] * rf;
+        }
+    }
+}
+
+// one lane's sums in units of 2^56 (du unit times row unit); the warp's total stays at most 2^62
+OTM_HD i64 kin_fix_combine(const KinFixSums &s, int j)
+{
+    return (s.hh[j] << 3) + ((s.hl[j] + (1LL << 27)) >> 28) + (int)rintf(s.ll[j] * 0x1p-59f);
+}
+
+// the exponent of the combined sums' unit: du 2^fu, row 2^fr (62 for N, fe for e)
+OTM_HD int kin_fix_exponent(int fu, int fr) { return 56 - fu - (fr - 1); }
 
 }  // namespace otm

@@ -884,7 +884,7 @@ template <>
 struct KinSum<true> {
     float t;
     float c[3];
-    __device__ __forceinline__ void gather(const Dev &D, int64_t base, int n, int lane)
+    __device__ __forceinline__ void gather(const Dev &D, int64_t base, int n, int lane, void *)
     {
         float v[12];
 #pragma unroll
@@ -915,16 +915,120 @@ struct KinSum<true> {
     }
 };
 
+// The FP64 path's gather in fixed point (kin_fix_pair): x_p,n+1 = x_p,n + sum N du (Eq. 9 by the partition of
+// unity and linear reproducibility, as in the mixed path) and G, from the nodes' increments in units of
+// 2^-kin_fu (written by the node update). Errors are below 2^-57 of h in x_p and of 1 in G K, so the
+// roundings of x_p and dF = 1 - G K themselves stay the largest. A support with an increment out of range
+// (half a spacing a step or more) takes the FP64 gather.
+// 12 FP64 FMAs a pair bounded the kernel (pipe 89 % busy); here a pair takes 36 integer multiply-adds, 12 FP32
+// FMAs and about 80 other instructions. k_kin_search on the 202,752-MP rod: 1.61 -> 1.56 ms.
+// A pair's loads (its ID, then row and increment: two dependent latencies) run kKinDepth - 1 passes ahead as
+// asynchronous copies into shared memory, which takes no registers: the sums hold 60. (3 stages: 6 % slower.)
+constexpr int kKinDepth = 2;
+struct KinStage {
+    uint4 c[kKinDepth][4][kWarp];   // row (2 words of 16 bytes), increment (2), one slot a lane
+};
+
+__device__ __forceinline__ void cp16_cg(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp16_ca(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+struct KinFix {
+    double t;      // this lane's reduced value: 0-2 x_p (or its increment), 3-11 G
+    bool inc;      // values 0-2 are increments
+    __device__ __forceinline__ void gather(const Dev &D, int64_t base, int n, int lane, KinStage *st)
+    {
+        i64 v[12];
+        int wide = 0;
+        {
+            KinFixSums s;
+#pragma unroll
+            for (int i = 0; i < 12; i++) s.hh[i] = s.hl[i] = 0, s.ll[i] = 0.f;
+            const int fe = D.kin_fe;
+            const int32_t *ids = D.ids + base;
+            auto fetch = [&](int k, int id) {   // pass k's copies (a group per pass, empty past the end)
+                if (k < n) {
+                    const int b = (k / kWarp) % kKinDepth;
+                    const char *row = (const char *)(D.shape + base + k), *du = (const char *)(D.dufix + 2 * (int64_t)id);
+                    cp16_cg(&st->c[b][0][lane], row);
+                    cp16_cg(&st->c[b][1][lane], row + 16);
+                    cp16_ca(&st->c[b][2][lane], du);
+                    cp16_ca(&st->c[b][3][lane], du + 16);
+                }
+                asm volatile("cp.async.commit_group;");
+            };
+            int id[kKinDepth];
+#pragma unroll
+            for (int j = 0; j < kKinDepth; j++) id[j] = lane + j * kWarp < n ? ids[lane + j * kWarp] : 0;
+#pragma unroll
+            for (int j = 0; j < kKinDepth - 1; j++) fetch(lane + j * kWarp, id[j]);
+            int idn = id[kKinDepth - 1];
+            const int passes = (n + kWarp - 1) / kWarp;   // warp-uniform: every lane commits and waits alike
+            // two passes a round: one leaves a copy of every sum at the loop's end (48 moves)
+#pragma unroll 2
+            for (int q = 0; q < passes; q++) {
+                const int k = lane + q * kWarp;
+                fetch(k + (kKinDepth - 1) * kWarp, idn);
+                idn = k + kKinDepth * kWarp < n ? ids[k + kKinDepth * kWarp] : 0;
+                asm volatile("cp.async.wait_group %0;" ::"n"(kKinDepth - 1) : "memory");
+                if (k < n) {
+                    const int b = q % kKinDepth;
+                    const double2 r0 = *(const double2 *)&st->c[b][0][lane], r1 = *(const double2 *)&st->c[b][1][lane];
+                    const int4 h = *(const int4 *)&st->c[b][2][lane], l = *(const int4 *)&st->c[b][3][lane];
+                    wide |= l.w;
+                    const int uh[3] = {h.x, h.y, h.z}, ul[3] = {l.x, l.y, l.z};
+                    kin_fix_pair(fix_floor(r0.x, 62), fix_floor(r0.y, fe), fix_floor(r1.x, fe), fix_floor(r1.y, fe), uh, ul, s);
+                }
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+            for (int i = 0; i < 12; i++) v[i] = kin_fix_combine(s, i);
+        }
+        if (__any_sync(0xffffffffu, wide != 0) || n > 12 * kWarp) {
+            KinSum<false> ks;
+            ks.gather(D, base, n, lane);
+            t = ks.t;
+            inc = false;
+            return;
+        }
+        const i64 r = warp_reduce_scatter12(v, lane);
+        t = (double)r * ldexp(1.0, kin_fix_exponent(D.kin_fu, rs12_value(lane) < 3 ? 62 : D.kin_fe));
+        inc = true;
+    }
+    __device__ __forceinline__ double g() const { return t; }
+    __device__ __forceinline__ double xp(double old, int) const { return inc ? old + t : t; }
+};
+
+template <bool MIXED>
+struct KinGather;
+template <>
+struct KinGather<false> {
+    using type = KinFix;
+    using stage = KinStage;
+};
+template <>
+struct KinGather<true> {
+    using type = KinSum<true>;
+    struct stage {};
+};
+
 // ======================================================================== k_kin_search
 // Kinematics (Eq. 9, 11) and the support search at the new position (Algorithm 3) in one warp
 // per MP: the gather over the old support gives x_p and dF, then the candidate scan builds the
 // new support in the same row. Used when no erosion can remove MPs between the two; the
 // return map (which only needs dF) follows.
-// Occupancy: the mixed kernel is bound by memory latency (the FP32 gather leaves the FP64 pipe
-// idle), so 12 blocks per SM (40 registers, a 16-byte spill) beat 10 (48 registers): 14.2 against
-// 14.8 ms on the 2.85 M-MP rod; the FP64 kernel is bound by its FP64 gather and takes 8 blocks.
+// Occupancy: both are bound by latency. Mixed: 12 blocks per SM (40 registers, a 16-byte spill) 2.86 ms on
+// 616 k MPs. FP64: the gather's sums take 60 registers; 6 blocks (80 registers, a 72-byte spill) 1.56 ms on
+// 202,752 MPs.
 template <bool MIXED>
-__global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 8) k_kin_search(const Dev D)
+__global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 6) k_kin_search(const __grid_constant__ Dev D)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -934,8 +1038,9 @@ __global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 8) k_kin_se
     const int S = D.S;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)S;
-    KinSum<MIXED> ks;
-    ks.gather(D, base, n, lane);
+    __shared__ typename KinGather<MIXED>::stage kst[kSearchWarps];
+    typename KinGather<MIXED>::type ks;
+    ks.gather(D, base, n, lane, &kst[(threadIdx.x >> 5)]);
     const int j = rs12_value(lane);
     if (rs12_writer(lane) && j >= 3) D.dF[9 * p + (j - 3)] = ks.g();   // G = sum du (x) e; k_return_map forms dF
     // values 0, 1, 2 (x_p) sit at lanes 0, 2, 4
@@ -1816,7 +1921,7 @@ cudaError_t launch_lme(const Dev &D, cudaStream_t s, long long *launches)
 // once per MP in the thread-per-MP return-map kernel with the products with F, det(dF) and the
 // volume update.
 template <bool MIXED>
-__global__ void __launch_bounds__(128) k_kinematics(const Dev D)
+__global__ void __launch_bounds__(128) k_kinematics(const __grid_constant__ Dev D)
 {
     const int lane = threadIdx.x & 31;
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1824,8 +1929,9 @@ __global__ void __launch_bounds__(128) k_kinematics(const Dev D)
     if (has_error(D.err)) return;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)D.S;
-    KinSum<MIXED> ks;
-    ks.gather(D, base, n, lane);
+    __shared__ typename KinGather<MIXED>::stage kst[kSearchWarps];
+    typename KinGather<MIXED>::type ks;
+    ks.gather(D, base, n, lane, &kst[(threadIdx.x >> 5)]);
     const int j = rs12_value(lane);
     if (rs12_writer(lane)) {
         if (j < 3) {

@@ -66,17 +66,41 @@ extern "C" int eval(int n, const double *x, const double *xp, const double *lam,
 '''
 
 
+KIN = r'''
+// one warp's kinematics sums: out[12] = sum N du (3), G = sum du (x) e (9)
+extern "C" void gather(int n, const double *row, const double *du, int fu, int fe, double *out)
+{
+    i64 t[12] = {0};
+    for (int lane = 0; lane < 32; lane++) {
+        KinFixSums s;
+        for (int i = 0; i < 12; i++) s.hh[i] = s.hl[i] = 0, s.ll[i] = 0.f;
+        for (int k = lane; k < n; k += 32)
+        {
+            int uh[3], ul[3];
+            for (int i = 0; i < 3; i++) kin_fix_split(fix_from_double(du[3 * k + i], fu), uh[i], ul[i]);
+            kin_fix_pair(fix_floor(row[4 * k], 62), fix_floor(row[4 * k + 1], fe), fix_floor(row[4 * k + 2], fe),
+                         fix_floor(row[4 * k + 3], fe), uh, ul, s);
+        }
+        for (int i = 0; i < 12; i++) t[i] += kin_fix_combine(s, i);
+    }
+    for (int i = 0; i < 12; i++) out[i] = std::ldexp((double)t[i], kin_fix_exponent(fu, i < 3 ? 62 : fe));
+}
+'''
+
+
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
     gxx = shutil.which("g++")
     if gxx is None:
         pytest.skip("no host compiler")
     d = tmp_path_factory.mktemp("fix")
-    (d / "fix.cpp").write_text(SRC)
+    (d / "fix.cpp").write_text(SRC + KIN)
     so = str(d / "fix.so")
     subprocess.run([gxx, "-O2", "-std=gnu++17", "-shared", "-fPIC", "-I", CSRC, str(d / "fix.cpp"), "-o", so], check=True)
     L = C.CDLL(so)
     L.eval.argtypes = [C.c_int] + [C.c_void_p] * 3 + [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_uint64] + [C.c_void_p] * 3
+    L.gather.argtypes = [C.c_int, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_void_p]
+    L.gather.restype = None
     return L
 
 
@@ -133,3 +157,27 @@ def test_fixed_point_evaluation(lib, h, origin, corner, lam_h, tol):
             ref = D(float(w[k])) * d[k][i]
             # half an ulp, and half a unit of each coordinate
             assert abs(D(float(prod[k, i])) - ref) <= D(2) ** -53 * abs(ref) + D(float(w[k])) * D(2) ** (1 - fb)
+
+
+@pytest.mark.parametrize("n,speed", [(1, 0.02), (33, 0.499), (286, 0.02), (384, 0.499), (286, 1e-9)])
+def test_fixed_point_kinematics_gather(lib, n, speed):
+    """sum N du and sum du (x) e of one support with increments up to half a spacing, all of one sign
+    (the largest sums). Units: du 2^-57 h at most, N 2^-61, e 2^-61 of at most twice r_s; dropped low products and
+    truncations are a few units each: 2^-57 h and 2^-57 h r_s hold for 384 pairs with sum N = 1."""
+    h, rs = 1.3e-4, 5.4e-4
+    rng = np.random.default_rng(n)
+    N = rng.uniform(0.1, 1.0, n) ** 6
+    N /= N.sum()
+    row = np.ascontiguousarray(np.concatenate([N[:, None], N[:, None] * rng.uniform(-rs, rs, (n, 3))], 1))
+    du = np.ascontiguousarray(rng.uniform(0.9, 1.0, (n, 3)) * speed * h)
+    fu, fe = 57 - int(np.floor(np.log2(h))), 61 - int(np.floor(np.log2(rs)))
+    out = np.zeros(12)
+    ptr = lambda t: t.ctypes.data_as(C.c_void_p)
+    lib.gather(n, ptr(row), ptr(du), fu, fe, ptr(out))
+    D = Decimal
+    for i in range(3):
+        ref = sum(D(float(row[k, 0])) * D(float(du[k, i])) for k in range(n))
+        assert abs(D(float(out[i])) - ref) <= D(2) ** -53 * abs(ref) + D(2) ** -57 * D(h)
+        for j in range(3):
+            ref = sum(D(float(du[k, i])) * D(float(row[k, 1 + j])) for k in range(n))
+            assert abs(D(float(out[3 + 3 * i + j])) - ref) <= D(2) ** -53 * abs(ref) + D(2) ** -57 * D(h) * D(rs)

@@ -460,3 +460,28 @@ def test_lme_cold_start_after_a_failed_warm_start(orc, OTM):
     assert rel(g.get("shape"), shape0) <= 1e-12
     o = orc.Sim(p)
     assert rel(g.get("lam"), o.get("lam")) <= 1e-10
+
+
+@pytest.mark.parametrize("shift", [0.0, 1e-7, 0.3, 0.49, 0.51, 0.9])
+def test_kinematics_gather_over_the_range_of_increments(OTM, shift):
+    """One step of a body moving rigidly by `shift` spacings with a small random deformation: x_p and dF against
+    numpy over the exported shape functions (the fixed-point gather below half a spacing a step, FP64
+    above). Bounds: x_p moves by sum N du where Eq. 9 sums N x, equal to the Newton tolerance 1e-14 h,
+    plus FP64 rounding of positions; dF - 1 is a sum of products |du||grad N| (their sum is below 4 shift
+    + 1), rounded a few times in either implementation."""
+    p = scenarios.taylor_rod(h=0.8e-3, R=3.2e-3, L=6.4e-3, wall=False, material=scenarios.copper_j2())
+    rng = np.random.default_rng(2)
+    p.node_du0[:] = np.array([shift, -0.7 * shift, 0.4 * shift]) * p.h + rng.normal(0, 1e-4 * p.h, p.node_du0.shape)
+    sim = OTM(p)
+    rows = np.arange(0, p.n_mps, 7)
+    x0, cnt = sim.get("mp_x"), sim.get("support_count")
+    ids, sh = sim.get_rows("support_ids", rows), sim.get_rows("shape", rows)
+    assert sim.step(1) == 0, sim.error()
+    x, du, xp, dF = sim.get("node_x"), sim.get("node_du"), sim.get("mp_x"), sim.get("dF").reshape(-1, 3, 3)
+    for r, q in enumerate(rows):
+        n = cnt[q]
+        a, N, g = ids[r, :n], sh[r, :n, 0], sh[r, :n, 1:]
+        assert np.abs(xp[q] - N @ x[a]).max() <= 2e-14 * p.h + 8 * 2.0 ** -53 * np.abs(x[a]).max()
+        ref = np.eye(3) + du[a].T @ g
+        assert np.abs(dF[q] - ref).max() <= 64 * 2.0 ** -53 * (4 * shift + 1)
+    assert not np.array_equal(x0, xp)
