@@ -334,28 +334,6 @@ __device__ __forceinline__ double dist2_exact(double ax, double ay, double az, d
     return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-// bitonic sort (ascending) of a[0..n2) in shared memory by one warp; n2 a power of two
-template <typename T>
-__device__ __forceinline__ void warp_bitonic_sort(T *a, int n2, int lane)
-{
-    for (int k = 2; k <= n2; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < n2; i += kWarp) {
-                int ixj = i ^ j;
-                if (ixj > i) {
-                    T ai = a[i], aj = a[ixj];
-                    bool up = ((i & k) == 0);
-                    if ((ai > aj) == up) {
-                        a[i] = aj;
-                        a[ixj] = ai;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
 __host__ __device__ __forceinline__ int next_pow2(int v)
 {
     int p = 1;

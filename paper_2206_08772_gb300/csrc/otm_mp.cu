@@ -436,69 +436,92 @@ __device__ int warp_support_search(const SearchGrid &G, const SearchConst &C, do
     const float X = (float)(px - g->origin[0]), Y = (float)(py - g->origin[1]), Z = (float)(pz - g->origin[2]);
     const float cf = C.cf;
     const float rs = C.rs;
-    // cell ranges covering [x - r_s, x + r_s] with a 1e-4 relative margin (which covers the FP32
-    // rounding of X and of the quotient; nodes are binned by the exact FP64 floor)
-    const float rsm = rs * 1.0001f;
-    const int x0 = max((int)fmaxf(floorf((X - rsm) / cf), -1.f), 0);
-    const int x1 = min((int)fminf(floorf((X + rsm) / cf), (float)nx), nx - 1);
-    const int y0 = max((int)fmaxf(floorf((Y - rsm) / cf), -1.f), 0);
-    const int y1 = min((int)fminf(floorf((Y + rsm) / cf), (float)ny), ny - 1);
-    const int z0 = max((int)fmaxf(floorf((Z - rsm) / cf), -1.f), 0);
-    const int z1 = min((int)fminf(floorf((Z + rsm) / cf), (float)nz), nz - 1);
-    int cnt = 0;
-    if (x0 > x1 || y0 > y1 || z0 > z1) return 0;
     const float ext = fmaxf(fmaxf((float)nx, (float)ny), (float)nz) * cf;
     const float U = fmaxf(fmaxf(fmaxf(fabsf(X), fabsf(Y)), fabsf(Z)), ext);
     const float u = 0x1p-24f;
     const float e = 1.001f * u * (2.f * U + 1.5f * rs);
     const float band = 1.5f * (1.25f * (e * (9.f * rs + 3.f * e) + 3.1f * u * rs * rs) + 1e-15f * rs * rs);
     const float lo = __fsub_rd(C.rs2_rd, band), hi = __fadd_ru(C.rs2_ru, band);
-    // the test of one candidate slot s of a row ending at s1 (its FP32 record already loaded)
-    auto test = [&](int s, int s1, const float4 &a, int &id) -> bool {
-        if (s >= s1) return false;
+    // Cells that a ball of radius r_s (1 + 1e-4) + 2 e about the point meets (the margin covers the FP32
+    // rounding of the point, the quotients and the distances; nodes are binned by the exact FP64
+    // floor): the rows along x whose (y, z) square it meets, and of each row the cells it reaches. 84
+    // cells on average instead of the 125 of the bounding box. With the branch-free tests and the next row's
+    // loads ahead: k_kin_search 1.56 -> 1.41 ms (202,752 MPs, FP64), 2.86 -> 2.64 ms (616 k, mixed).
+    const float rsm = rs * 1.0001f + 2.f * e;
+    const int y0 = max((int)fmaxf(floorf((Y - rsm) / cf), -1.f), 0);
+    const int y1 = min((int)fminf(floorf((Y + rsm) / cf), (float)ny), ny - 1);
+    const int z0 = max((int)fmaxf(floorf((Z - rsm) / cf), -1.f), 0);
+    const int z1 = min((int)fminf(floorf((Z + rsm) / cf), (float)nz), nz - 1);
+    int cnt = 0;
+    if (y0 > y1 || z0 > z1) return 0;
+    const unsigned below = (1u << lane) - 1u;
+    // the tests of 32 candidates from slot s on (their FP32 records loaded; lanes past the row's end hold a
+    // point at infinity), the accepted IDs appended
+    auto scan = [&](int s, const float4 &a) {
         const float dx = X - a.x, dy = Y - a.y, dz = Z - a.z;
         const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        id = __float_as_int(a.w);
-        if (d2 <= lo) return true;
-        if (d2 > hi) return false;
-        const double4_32a q = G.spos[s];   // ambiguity band: exact FP64 test
-        return dist2_exact(px, py, pz, q.x, q.y, q.z) <= rs2;
-    };
-    auto append = [&](bool acc, int id) {
-        const unsigned m = __ballot_sync(0xffffffffu, acc);
-        if (acc) {
-            const int pos = cnt + __popc(m & ((1u << lane) - 1u));
-            if (pos < S) list[pos] = id;
+        bool acc = d2 <= lo;
+        const bool near = !acc && d2 <= hi;
+        if (__any_sync(0xffffffffu, near)) {   // ambiguity band: exact FP64 test
+            if (near) {
+                const double4_32a q = G.spos[s + lane];
+                acc = dist2_exact(px, py, pz, q.x, q.y, q.z) <= rs2;
+            }
+            __syncwarp();
         }
+        const unsigned m = __ballot_sync(0xffffffffu, acc);
+        const int pos = cnt + __popc(m & below);
+        if (acc && pos < S) list[pos] = __float_as_int(a.w);
         cnt += __popc(m);
     };
-    // Rows in (z, y) order, r = (kz - z0) ny' + (ky - y0). The candidate ranges of up to 32 rows
-    // are loaded at once, one row per lane, and each row is scanned 64 slots per pass with both
-    // chunks' loads in flight; the accepted IDs keep the order of a plain scan (rows, cells,
+    // Rows in (z, y) order, r = (kz - z0) ny' + (ky - y0), up to 32 at once, one a lane for their ranges of
+    // slots; then row by row, 64 slots a pass with both chunks' loads in flight and the next row's
+    // first pass ahead of this row's tests. The accepted IDs keep the order of a plain scan (rows, cells,
     // slots).
     const int nyr = y1 - y0 + 1, nrows = nyr * (z1 - z0 + 1);
+    const float4 none = make_float4(INFINITY, 0.f, 0.f, 0.f);
+    const float4 *sp = G.spos32 + lane;
     for (int g0 = 0; g0 < nrows; g0 += kWarp) {
-        int r0 = 0, r1 = 0;
+        int r0 = 0, len = 0;
         if (g0 + lane < nrows) {
-            const int r = g0 + lane;
-            const int rowc = ((z0 + r / nyr) * ny + (y0 + r % nyr)) * nx;
-            r0 = G.cell_start[rowc + x0];
-            r1 = G.cell_start[rowc + x1 + 1];
-        }
-        const int ng = min(kWarp, nrows - g0);
-        for (int r = 0; r < ng; r++) {
-            const int s0 = __shfl_sync(0xffffffffu, r0, r), s1 = __shfl_sync(0xffffffffu, r1, r);
-            for (int b = s0; b < s1; b += 2 * kWarp) {
-                const int sa = b + lane, sb = b + kWarp + lane;
-                float4 qa = make_float4(0.f, 0.f, 0.f, 0.f), qb = qa;
-                if (sa < s1) qa = G.spos32[sa];
-                if (sb < s1) qb = G.spos32[sb];
-                int ida = 0, idb = 0;
-                const bool acca = test(sa, s1, qa, ida);
-                const bool accb = test(sb, s1, qb, idb);
-                append(acca, ida);
-                if (b + kWarp < s1) append(accb, idb);
+            const int r = g0 + lane, kz = z0 + r / nyr, ky = y0 + r % nyr;
+            // distance of the point from the row's square, less 2 e (the FP32 rounding of both)
+            const float dy = fmaxf(fmaxf((float)ky * cf - Y, Y - (float)(ky + 1) * cf) - 2.f * e, 0.f);
+            const float dz = fmaxf(fmaxf((float)kz * cf - Z, Z - (float)(kz + 1) * cf) - 2.f * e, 0.f);
+            const float h2 = fmaf(-dz, dz, fmaf(-dy, dy, rsm * rsm));
+            if (h2 >= 0.f) {
+                const float half = sqrtf(h2) + 1e-4f * rs + 2.f * e;
+                const int x0 = max((int)fmaxf(floorf((X - half) / cf), -1.f), 0);
+                const int x1 = min((int)fminf(floorf((X + half) / cf), (float)nx), nx - 1);
+                if (x0 <= x1) {
+                    const int rowc = (kz * ny + ky) * nx;
+                    r0 = G.cell_start[rowc + x0];
+                    len = G.cell_start[rowc + x1 + 1] - r0;
+                }
             }
+        }
+        unsigned live = __ballot_sync(0xffffffffu, len > 0);
+        if (!live) continue;
+        int s0, n, r = __ffs(live) - 1;
+        s0 = __shfl_sync(0xffffffffu, r0, r);
+        n = __shfl_sync(0xffffffffu, len, r);
+        float4 qa = lane < n ? sp[s0] : none, qb = lane + kWarp < n ? sp[s0 + kWarp] : none;
+        for (;;) {
+            live &= live - 1;
+            int s1 = 0, n1 = 0;
+            float4 na = none, nb = none;
+            if (live) {
+                r = __ffs(live) - 1;
+                s1 = __shfl_sync(0xffffffffu, r0, r);
+                n1 = __shfl_sync(0xffffffffu, len, r);
+                if (lane < n1) na = sp[s1];
+                if (lane + kWarp < n1) nb = sp[s1 + kWarp];
+            }
+            scan(s0, qa);
+            if (n > kWarp) scan(s0 + kWarp, qb);
+            for (int b = 2 * kWarp; b < n; b += kWarp) scan(s0 + b, b + lane < n ? sp[s0 + b] : none);
+            if (!live) break;
+            s0 = s1; n = n1; qa = na; qb = nb;
         }
     }
     return cnt;
@@ -1024,9 +1047,9 @@ struct KinGather<true> {
 // per MP: the gather over the old support gives x_p and dF, then the candidate scan builds the
 // new support in the same row. Used when no erosion can remove MPs between the two; the
 // return map (which only needs dF) follows.
-// Occupancy: both are bound by latency. Mixed: 12 blocks per SM (40 registers, a 16-byte spill) 2.86 ms on
-// 616 k MPs. FP64: the gather's sums take 60 registers; 6 blocks (80 registers, a 72-byte spill) 1.56 ms on
-// 202,752 MPs.
+// Occupancy: both are bound by latency. Mixed: 12 blocks per SM (40 registers, a 24-byte spill) 2.64 ms, 10
+// blocks 2.84 ms on 616 k MPs. FP64: the gather's sums take 60 registers; 6 blocks (80 registers, a 116-byte
+// spill) 1.41 ms, 5 blocks 1.47 ms on 202,752 MPs, and the two as separate kernels 1.5 ms.
 template <bool MIXED>
 __global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 6) k_kin_search(const __grid_constant__ Dev D)
 {
@@ -2284,7 +2307,71 @@ cudaError_t launch_return_map(const Dev &D, cudaStream_t s, long long *launches)
 }
 
 // ======================================================================== stand-alone kernels
-__global__ void __launch_bounds__(kSearchWarps * kWarp)
+// Ascending bitonic sort of 32 R integers by one warp in registers (in shared memory it took 7,200 of a
+// point's 9,200 instructions at 250 nodes a support; 600,007 points: 5.80 -> 2.19 ms), lane l holding the sorted elements
+// [l R, (l + 1) R) afterwards (in any order before). Steps over fewer than R elements stay in the lane as plain
+// minima and maxima, the others exchange with a lane of the same direction; lanes of a descending
+// subsequence hold the complements instead.
+template <int R>
+__device__ __forceinline__ void warp_sort(int (&v)[R], int lane)
+{
+    int dir = 0;   // -1: complements
+#pragma unroll
+    for (int k = 2; k <= kWarp * R; k *= 2) {
+        if (k >= R) {
+            const int d = (lane * R & k) ? -1 : 0, f = d ^ dir;
+#pragma unroll
+            for (int r = 0; r < R; r++) v[r] ^= f;
+            dir = d;
+        }
+#pragma unroll
+        for (int j = k / 2; j > 0; j /= 2) {
+            if (j >= R) {
+                const bool lower = !(lane & (j / R));
+#pragma unroll
+                for (int r = 0; r < R; r++) {
+                    const int o = __shfl_xor_sync(0xffffffffu, v[r], j / R);
+                    v[r] = lower ? min(v[r], o) : max(v[r], o);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; r++)
+                    if (!(r & j)) {
+                        const int a = v[r], b = v[r + j];
+                        const bool up = k >= R || !(r & k);
+                        v[r] = up ? min(a, b) : max(a, b);
+                        v[r + j] = up ? max(a, b) : min(a, b);
+                    }
+            }
+        }
+    }
+}
+
+// list[0..n) (n <= 32 R, room for 33 R) in ascending order
+template <int R>
+__device__ void warp_sort_list(int32_t *list, int n, int lane)
+{
+    int v[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) v[r] = lane + kWarp * r < n ? list[lane + kWarp * r] : 0x7fffffff;
+    __syncwarp();
+    warp_sort<R>(v, lane);
+#pragma unroll
+    for (int r = 0; r < R; r++) {   // through a row of 33 words a warp's worth: no bank conflicts
+        const int k = lane * R + r;
+        list[k + k / kWarp] = v[r];
+    }
+    __syncwarp();
+}
+
+// shared-memory words of a warp's list of up to S IDs
+__host__ __device__ __forceinline__ int search_list_words(int S)
+{
+    const int P2 = next_pow2(S < kWarp ? kWarp : S);
+    return P2 + P2 / kWarp;
+}
+
+__global__ void __launch_bounds__(kSearchWarps * kWarp, 8)   // 64 registers; 48 the same, 40 (spills) 19 % slower
     k_search_only(const GridDev *g, const int32_t *cell_start, const float4 *spos32, const double4_32a *spos,
                   const SearchConst C, const double *mp_x, int64_t nm, int S, int32_t *ids, int32_t *counts,
                   int32_t *status, const unsigned long long *grid_err)
@@ -2293,8 +2380,7 @@ __global__ void __launch_bounds__(kSearchWarps * kWarp)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t p = (int64_t)blockIdx.x * kSearchWarps + warp;
     if (p >= nm) return;
-    const int P2 = next_pow2(S);
-    int32_t *list = (int32_t *)smem_raw + (size_t)warp * P2;
+    int32_t *list = (int32_t *)smem_raw + (size_t)warp * search_list_words(S);
     if (*grid_err != ~0ULL) {
         if (lane == 0) {
             atomicCAS(status, 0, (int)(-(int)(*grid_err & 0xff)));
@@ -2306,11 +2392,14 @@ __global__ void __launch_bounds__(kSearchWarps * kWarp)
     SearchGrid G{g, cell_start, spos32, spos};
     const int cnt = warp_support_search(G, C, px, py, pz, list, S, lane);
     const int n = min(cnt, S);
-    const int Q2 = next_pow2(max(n, 1));
-    for (int k = n + lane; k < Q2; k += kWarp) list[k] = 0x7fffffff;
     __syncwarp();
-    warp_bitonic_sort(list, Q2, lane);
-    for (int k = lane; k < n; k += kWarp) ids[p * (int64_t)S + k] = list[k];
+    if (n <= kWarp) warp_sort_list<1>(list, n, lane);
+    else if (n <= 2 * kWarp) warp_sort_list<2>(list, n, lane);
+    else if (n <= 4 * kWarp) warp_sort_list<4>(list, n, lane);
+    else if (n <= 8 * kWarp) warp_sort_list<8>(list, n, lane);
+    else if (n <= 16 * kWarp) warp_sort_list<16>(list, n, lane);
+    else warp_sort_list<kMaxS / kWarp>(list, n, lane);
+    for (int k = lane; k < n; k += kWarp) ids[p * (int64_t)S + k] = list[k + k / kWarp];
     if (lane == 0) {
         counts[p] = cnt;
         if (cnt > S) atomicCAS(status, 0, OTM_ERR_CAPACITY);
@@ -2325,7 +2414,7 @@ cudaError_t launch_search_only(const double *node_x, int64_t nn, const double *m
     if (!carve_search_scratch(scratch, scratch_bytes, nn, &V)) return cudaErrorInvalidValue;
     cudaError_t e = build_search_grid(node_x, nn, cell, &V, grid_out, s);
     if (e != cudaSuccess) return e;
-    const size_t smem = (size_t)kSearchWarps * next_pow2(S) * sizeof(int32_t);
+    const size_t smem = (size_t)kSearchWarps * search_list_words(S) * sizeof(int32_t);
     const unsigned blocks = (unsigned)((nm + kSearchWarps - 1) / kSearchWarps);
     if (blocks == 0) return cudaSuccess;
     k_search_only<<<blocks, kSearchWarps * kWarp, smem, s>>>(V.g, V.cell_start, V.spos32, V.spos,

@@ -55,6 +55,37 @@ def test_search_bit_exact(orc, otm, seed, nn, nm, r, S):
     assert np.array_equal(g[:3], origin) and np.array_equal(g[3:].astype(np.int64), dims)
 
 
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 65, 127, 129, 256, 257, 511, 513, 1024])
+def test_search_list_lengths(otm, n):
+    """Supports of every sort length: all n nodes in one point's ball; a second point with no node; the rows
+    hold exactly the IDs, ascending, and a truncated row still ascends."""
+    node_x, _ = scenarios.random_cloud(n, 1, n)
+    mp_x = np.array([[0.5, 0.5, 0.5], [9.0, 9.0, 9.0]])
+    ids, counts, _, status = otm.support_search(dev(node_x), dev(mp_x), 4.0, 1.0, n)
+    assert counts.cpu().tolist() == [n, 0] and int(status) == 0
+    assert np.array_equal(ids.cpu().numpy()[0], np.arange(n))
+    S = max(1, n // 2)
+    ids, counts, _, status = otm.support_search(dev(node_x), dev(mp_x), 4.0, 1.0, S)
+    assert counts.cpu().tolist() == [n, 0]
+    row = ids.cpu().numpy()[0]
+    assert (np.diff(row) > 0).all() and 0 <= row[0] and row[-1] < n
+
+
+@pytest.mark.parametrize("cell,scale,shift", [(0.50001, 1.0, 0.0), (0.6, 1.0, 40.0), (0.51, 1e-4, -7.0), (0.9, 1e3, 300.0),
+                                              (1.7, 1.0, 0.0), (12.0, 1.0, 5.0)])
+def test_search_cells_of_the_ball(orc, otm, cell, scale, shift):
+    """The cells a ball meets, for cells from half the radius to beyond the body, away from the origin;
+    bit-equal to the oracle's full box."""
+    node_x, mp_x = scenarios.random_cloud(3000, 400, 11)
+    node_x, mp_x, r = (node_x + shift) * scale, (1.2 * mp_x - 0.1 + shift) * scale, 0.17 * scale
+    ids, counts, _, _ = otm.support_search(dev(node_x), dev(mp_x), r * r, cell * r, 256)
+    off, ref = orc.search(node_x, mp_x, r * r, cell * r)
+    counts, ids = counts.cpu().numpy(), ids.cpu().numpy()
+    assert np.array_equal(counts, np.diff(off)) and counts.max() <= 256
+    for p in range(len(counts)):
+        assert np.array_equal(ids[p, :counts[p]], ref[off[p]:off[p + 1]])
+
+
 def test_search_ties_exact(orc, otm):
     r = 0.25
     rs2 = r * r
