@@ -313,6 +313,19 @@ __device__ __forceinline__ float warp_max_f(float v)
     return v;
 }
 
+// FP64 -> FP32, rounded to nearest (ties away from zero), with integer operations on the bits: a
+// conversion instruction takes an FP64-pipe slot on this GPU, integer operations do not. Values
+// below the normal FP32 range give a signed zero; |v| < 2^127 is assumed (shape-function values,
+// their products with separations, and force contributions).
+__device__ __forceinline__ float f32_round_bits(double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
+    const unsigned sgn = hi & 0x80000000u;
+    const unsigned mag = ((unsigned)(e + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    return __uint_as_float(e < -126 ? sgn : (sgn | (mag + ((lo >> 28) & 1u))));
+}
+
 // linked-cell coordinate: floor((x - o) / c) in correctly rounded FP64 (bit-identical to any
 // IEEE implementation of the same expression), optionally clamped to the grid.
 __device__ __forceinline__ int cell_coord(double x, double o, double c, int n, bool clamp)

@@ -852,19 +852,6 @@ __global__ void __launch_bounds__(kSearchWarps * kWarp) k_search(const Dev D)
 }
 
 // ======================================================================== kinematics gathers
-// FP64 -> FP32, rounded to nearest (ties away from zero), with integer operations on the bits: a
-// conversion instruction takes an FP64-pipe slot on this GPU, integer operations do not. Values
-// below the normal FP32 range give a signed zero; |v| < 2^127 is assumed (shape-function values,
-// their products with separations, and force contributions).
-__device__ __forceinline__ float f32_round_bits(double v)
-{
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
-    const unsigned sgn = hi & 0x80000000u;
-    const unsigned mag = ((unsigned)(e + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
-    return __uint_as_float(e < -126 ? sgn : (sgn | (mag + ((lo >> 28) & 1u))));
-}
-
 // The 12 sums of the kinematics over MP p's old support (n pairs at row base), reduce-scattered
 // (value rs12_value(lane) at each lane): 0-2 the x_p sums, 3-11 G = sum du_a (x) e_a row-major.
 //  FP64 path: x_p = sum N_a x_a of the updated node positions (Eq. 9), G from the FP64 increments.

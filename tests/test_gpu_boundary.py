@@ -175,6 +175,35 @@ def test_grid_cell_order_matches_the_oracle(orc, OTM):
     assert np.array_equal(srt, o_srt)
 
 
+@pytest.mark.parametrize("h,L,n_range", [(1.6e-3, 3.2e-3, (1, 512)), (0.8e-3, 9.6e-3, (513, 16384)),
+                                         (0.4e-3, 20e-3, (513, 16384)), (0.35e-3, 25.4e-3, (16385, 40000))])
+@pytest.mark.parametrize("kind", ["boundaries", "one cell", "sparse"])
+def test_grid_of_awkward_positions(orc, OTM, h, L, n_range, kind):
+    """Each size of build, exactly the oracle's cells: coordinates on cell boundaries and an ulp beside them,
+    nearly all nodes in one cell, and far fewer nodes than cells."""
+    p = scenarios.taylor_rod(h=h, R=3.2e-3, L=L, material=scenarios.copper_j2(), v0=100.0)
+    g = OTM(p)
+    n = g.counts()["n_nodes"]
+    assert n_range[0] <= n <= n_range[1]
+    rng = np.random.default_rng(n)
+    c = p.cell_size
+    if kind == "boundaries":
+        x = rng.integers(0, 25, (n, 3)) * c
+        x = np.where(rng.uniform(size=x.shape) < 0.3, np.nextafter(x, rng.choice([-1.0, 1.0], x.shape)), x)
+        x[0] = 0.0
+        x = np.maximum(x, 0.0)
+    elif kind == "one cell":
+        x = rng.uniform(0.0, 0.9 * c, (n, 3))
+        x[-3:] = rng.uniform(0.0, 3.0 * c, (3, 3))
+    else:
+        x = rng.uniform(-18.0 * c, 20.0 * c, (n, 3))
+    g.set("node_x", x)
+    origin, dims, cs, srt = g.grid_cells()
+    o_origin, o_dims, o_cs, o_srt = orc.grid(g.get("node_x"), c)
+    assert np.array_equal(origin, o_origin) and np.array_equal(dims.astype(np.int64), o_dims)
+    assert np.array_equal(cs.astype(np.int64), o_cs) and np.array_equal(srt, o_srt)
+
+
 def test_device_support_record_replays_the_run_bit_for_bit(OTM):
     p = scenarios.taylor_rod(h=0.8e-3, R=3.2e-3, L=9.6e-3, material=scenarios.copper_jc(), v0=400.0)
     base = OTM(p)
