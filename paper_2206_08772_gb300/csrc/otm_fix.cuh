@@ -52,6 +52,20 @@ __device__ __forceinline__ int fx_log2(uint32_t v) { return (int)(__float_as_uin
 __device__ __forceinline__ int fx_rint(float v) { return __float2int_rn(v); }
 __device__ __forceinline__ double fx_bits_d(u64 b) { return __longlong_as_double((i64)b); }
 __device__ __forceinline__ u64 fx_d_bits(double v) { return (u64)__double_as_longlong(v); }
+__device__ __forceinline__ uint32_t fx_f_bits(float v) { return __float_as_uint(v); }
+// shifts by any amount: 64 and more (as unsigned) give 0
+__device__ __forceinline__ u64 fx_shr(u64 v, unsigned n)
+{
+    u64 r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+__device__ __forceinline__ u64 fx_shl(u64 v, unsigned n)
+{
+    u64 r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
 #else
 #ifdef __CUDACC__
 #define OTM_HD __host__ __device__ inline
@@ -82,6 +96,14 @@ OTM_HD u64 fx_d_bits(double v)
     memcpy(&b, &v, 8);
     return b;
 }
+OTM_HD uint32_t fx_f_bits(float v)
+{
+    uint32_t b;
+    memcpy(&b, &v, 4);
+    return b;
+}
+OTM_HD u64 fx_shr(u64 v, unsigned n) { return n < 64 ? v >> n : 0; }
+OTM_HD u64 fx_shl(u64 v, unsigned n) { return n < 64 ? v << n : 0; }
 #endif
 
 // constants of a problem (host-derived, see make_fix_const)
@@ -373,5 +395,44 @@ OTM_HD i64 kin_fix_combine(const KinFixSums &s, int j)
 
 // the exponent of the combined sums' unit: du 2^fu, row 2^fr (62 for N, fe for e)
 OTM_HD int kin_fix_exponent(int fu, int fr) { return 56 - fu - (fr - 1); }
+
+// ------------------------------------------------------------------ node sums (Eq. 5)
+// Signed fixed-point sums. A term enters as the magnitude's bits, complemented if it is negative; each
+// negative term is short of its two's complement by one unit, which `neg` counts.
+using u128 = unsigned __int128;
+template <typename U>
+struct FixedSum {
+    U v;
+    int neg;
+};
+using Sum128 = FixedSum<u128>;
+using Sum64 = FixedSum<u64>;
+
+// adds v / 2^(emax - 110), truncated toward zero. Branch-free: the significand, left-aligned in 128 bits, moves
+// right by 17 + emax - e; zero, subnormal (negligible) and non-finite values (caught elsewhere) move out.
+OTM_HD void add_fixed(Sum128 &a, double v, int emax)
+{
+    const u64 b = fx_d_bits(v);
+    const u64 m = (b | 0x0010000000000000ULL) << 11;
+    const unsigned ef = (unsigned)(b >> 52) & 0x7ffu;
+    const unsigned r = ef - 1u >= 0x7feu ? 128u : (unsigned)(emax + 1023 + 17) - ef;
+    const u64 sg = (u64)((long long)b >> 63);
+    const u64 h = fx_shr(m, r) ^ sg;
+    const u64 l = (fx_shl(m, 64u - r) | fx_shr(m, r - 64u)) ^ sg;
+    a.v += ((u128)h << 64) | l;
+    a.neg -= (int)sg;
+}
+
+// adds v / 2^(emax - 46), truncated toward zero
+OTM_HD void add_fixed(Sum64 &a, float v, int emax)
+{
+    const uint32_t b = fx_f_bits(v);
+    const u64 m = (u64)((b | 0x00800000u) << 8) << 32;
+    const unsigned ef = (b >> 23) & 0xffu;
+    const unsigned r = ef - 1u >= 0xfeu ? 64u : (unsigned)(emax + 127 + 17) - ef;
+    const int sg = (int)b >> 31;
+    a.v += fx_shr(m, r) ^ (u64)(long long)sg;
+    a.neg -= sg;
+}
 
 }  // namespace otm

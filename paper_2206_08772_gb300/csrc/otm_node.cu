@@ -14,83 +14,33 @@
 // stays below 2^127 resp. 2^63 and fits the signed accumulator whatever the signs.
 #include "otm_dev.cuh"
 
+#include <type_traits>
+
 namespace otm {
 
-struct I128 {
-    unsigned long long lo;
-    long long hi;
-};
-
-__device__ __forceinline__ void add128(I128 &a, const I128 &b)
+__device__ __forceinline__ u64 shfl_xor_any(u64 v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ u128 shfl_xor_any(u128 v, int o)
 {
-    const unsigned long long lo = a.lo + b.lo;
-    a.hi = a.hi + b.hi + (lo < a.lo ? 1 : 0);
-    a.lo = lo;
+    return ((u128)shfl_xor_any((u64)(v >> 64), o) << 64) | shfl_xor_any((u64)v, o);
 }
 
-// v / 2^(emax - 110) truncated toward zero, as a signed 128-bit integer
-__device__ __forceinline__ I128 to_fixed128(double v, int emax)
+// the warp's sum in every lane
+template <typename U>
+__device__ __forceinline__ U warp_total(const FixedSum<U> &a)
 {
-    I128 r = {0ULL, 0LL};
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int ef = (int)((b >> 52) & 0x7ff);
-    if (ef == 0 || ef == 0x7ff) return r;   // zero / subnormal (negligible); non-finite caught elsewhere
-    const unsigned long long m = (b & 0x000FFFFFFFFFFFFFULL) | 0x0010000000000000ULL;
-    const int sh = (ef - 1023) - emax + 58;  // value = m * 2^(e - 52); lsb = 2^(emax - 110)
-    if (sh < -52) return r;
-    if (sh < 0) {
-        r.lo = m >> (-sh);
-    } else if (sh < 64) {
-        r.lo = m << sh;
-        r.hi = (sh == 0) ? 0 : (long long)(m >> (64 - sh));
-    } else {
-        r.hi = (long long)(m << (sh - 64));
-    }
-    if (b >> 63) {   // two's complement negation
-        r.lo = ~r.lo + 1ULL;
-        r.hi = ~r.hi + (r.lo == 0ULL ? 1 : 0);
-    }
-    return r;
-}
-
-__device__ __forceinline__ double from_fixed128(const I128 &a, int emax)
-{
-    // value = (hi * 2^64 + lo) * 2^(emax - 110)
-    const double v = (double)a.hi * 18446744073709551616.0 + (double)a.lo;
-    return ldexp(v, emax - 110);
-}
-
-__device__ __forceinline__ I128 warp_sum128(I128 a)
-{
+    U v = a.v + (U)(u64)a.neg;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        I128 b;
-        b.lo = __shfl_xor_sync(0xffffffffu, a.lo, o);
-        b.hi = __shfl_xor_sync(0xffffffffu, a.hi, o);
-        add128(a, b);
-    }
-    return a;
-}
-
-__device__ __forceinline__ long long to_fixed64(float v, int emax)
-{
-    const unsigned int b = __float_as_uint(v);
-    const int ef = (int)((b >> 23) & 0xff);
-    if (ef == 0 || ef == 0xff) return 0;
-    const long long m = (long long)((b & 0x007FFFFFu) | 0x00800000u);
-    const int sh = (ef - 127) - emax + 23;   // value = m * 2^(e - 23); lsb = 2^(emax - 46)
-    long long r;
-    if (sh < -23) return 0;
-    r = (sh < 0) ? (m >> (-sh)) : (m << sh);
-    return (b >> 31) ? -r : r;
-}
-
-__device__ __forceinline__ long long warp_sum64(long long v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) v += shfl_xor_any(v, o);
     return v;
 }
+
+__device__ __forceinline__ double sum_value(u128 a, int emax)
+{
+    // (hi * 2^64 + lo) * 2^(emax - 110)
+    const double v = (double)(long long)(u64)(a >> 64) * 18446744073709551616.0 + (double)(u64)a;
+    return ldexp(v, emax - 110);
+}
+__device__ __forceinline__ double sum_value(u64 a, int emax) { return ldexp((double)(long long)a, emax - 46); }
 
 // ---------------------------------------------------------------------------- contact
 // rigid frictionless wall: project a penetrating node onto the plane
@@ -133,45 +83,54 @@ __device__ __forceinline__ void tool_project(const Dev &D, double t_next, double
 }
 
 // ---------------------------------------------------------------------------- node kernel
-template <bool MIXED>
-__global__ void __launch_bounds__(kNodeWarps * kWarp) k_node_update(const Dev D, double t_next)
+// W warps a node. Bound by the integer pipes (about 30 instructions a term; the FP64 sums of 38 k nodes with
+// 1,420 terms each, 1.7 GB: 0.50 ms with three-way branches on the shift, 0.35 ms without).
+template <bool MIXED, int W>
+__global__ void __launch_bounds__(kNodeWarps * kWarp) k_node_update(const __grid_constant__ Dev D, double t_next)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= D.nn) return;
-    if (has_error(D.err)) return;
+    using U = typename std::conditional<MIXED, u64, u128>::type;
+    __shared__ U part[W > 1 ? kNodeWarps : 1][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * (kNodeWarps / W) + warp / W;
+    if (W == 1 && (i >= D.nn || has_error(D.err))) return;
+    if (W > 1 && __syncthreads_or(has_error(D.err))) return;   // one node a block
     const int b = D.noff[i], L = D.noff[i + 1] - b;
     const int em = D.emax[0], ef = D.emax[1];
-    double m, rx, ry, rz;
-    if (MIXED) {
-        long long sm = 0, sx = 0, sy = 0, sz = 0;
-        for (int k = lane; k < L; k += kWarp) {
-            const float4 c = D.contrib32[b + k];
-            sm += to_fixed64(c.x, em);
-            sx += to_fixed64(c.y, ef);
-            sy += to_fixed64(c.z, ef);
-            sz += to_fixed64(c.w, ef);
-        }
-        sm = warp_sum64(sm); sx = warp_sum64(sx); sy = warp_sum64(sy); sz = warp_sum64(sz);
-        m = ldexp((double)sm, em - 46);
-        rx = ldexp((double)sx, ef - 46);
-        ry = ldexp((double)sy, ef - 46);
-        rz = ldexp((double)sz, ef - 46);
-    } else {
-        I128 sm = {0, 0}, sx = {0, 0}, sy = {0, 0}, sz = {0, 0};
-        for (int k = lane; k < L; k += kWarp) {
-            const double4_32a c = D.contrib64[b + k];
-            add128(sm, to_fixed128(c.x, em));
-            add128(sx, to_fixed128(c.y, ef));
-            add128(sy, to_fixed128(c.z, ef));
-            add128(sz, to_fixed128(c.w, ef));
-        }
-        sm = warp_sum128(sm); sx = warp_sum128(sx); sy = warp_sum128(sy); sz = warp_sum128(sz);
-        m = from_fixed128(sm, em);
-        rx = from_fixed128(sx, ef);
-        ry = from_fixed128(sy, ef);
-        rz = from_fixed128(sz, ef);
+    FixedSum<U> t[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) t[j].v = 0, t[j].neg = 0;
+    // a lane's terms W warps apart, the next one loading while this one is added
+    using T = typename std::conditional<MIXED, float4, double4_32a>::type;
+    const T *src = (MIXED ? (const T *)D.contrib32 : (const T *)D.contrib64) + b;
+    constexpr int step = W * kWarp;
+    int k = (warp % W) * kWarp + lane;
+    T c;
+    if (k < L) c = src[k];
+    for (; k < L; k += step) {
+        T n = c;
+        if (k + step < L) n = src[k + step];
+        add_fixed(t[0], c.x, em);
+        add_fixed(t[1], c.y, ef);
+        add_fixed(t[2], c.z, ef);
+        add_fixed(t[3], c.w, ef);
+        c = n;
     }
+    U v[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) v[j] = warp_total(t[j]);
+    if (W > 1) {
+        if (lane == 0) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) part[warp][j] = v[j];
+        }
+        __syncthreads();
+        if (warp != 0) return;
+#pragma unroll
+        for (int w = 1; w < W; w++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) v[j] += part[w][j];
+    }
+    const double m = sum_value(v[0], em), rx = sum_value(v[1], ef), ry = sum_value(v[2], ef), rz = sum_value(v[3], ef);
     if (lane != 0) return;
     D.mr[i] = make_double4_32a(m, rx, ry, rz);
     const double4_32a xo = D.x[i];
@@ -226,14 +185,20 @@ __global__ void __launch_bounds__(kNodeWarps * kWarp) k_node_update(const Dev D,
     if (!isfinite(x) || !isfinite(y) || !isfinite(z)) raise_error(D.err, OTM_ERR_NONFINITE, D.ngid[i]);
 }
 
+// A block per node (its list split over the warps) up to kNodeSplitMax nodes, a warp per node beyond: with a
+// warp each, a few thousand nodes leave most of the chip's warps idle. FP64, warp / block per node: 45 / 30 us
+// at 1.6 k nodes, 99 / 86 at 6 k, 157 / 155 at 13 k, 350 / 375 at 38 k.
+constexpr int64_t kNodeSplitMax = 8192;
+
 cudaError_t launch_node_update(const Dev &D, double t_next, cudaStream_t s, long long *launches)
 {
-    const unsigned blocks = (unsigned)((D.nn * 32 + kNodeWarps * 32 - 1) / (kNodeWarps * 32));
-    if (blocks == 0) return cudaSuccess;
-    if (D.precision == OTM_PRECISION_MIXED)
-        k_node_update<true><<<blocks, kNodeWarps * 32, 0, s>>>(D, t_next);
-    else
-        k_node_update<false><<<blocks, kNodeWarps * 32, 0, s>>>(D, t_next);
+    if (D.nn <= 0) return cudaSuccess;
+    const bool split = D.nn <= kNodeSplitMax;
+    const unsigned blocks = (unsigned)(split ? D.nn : (D.nn + kNodeWarps - 1) / kNodeWarps);
+    const bool mixed = D.precision == OTM_PRECISION_MIXED;
+    auto *k = mixed ? (split ? k_node_update<true, kNodeWarps> : k_node_update<true, 1>)
+                    : (split ? k_node_update<false, kNodeWarps> : k_node_update<false, 1>);
+    k<<<blocks, kNodeWarps * kWarp, 0, s>>>(D, t_next);
     if (launches) *launches += 1;
     return cudaGetLastError();
 }

@@ -88,19 +88,40 @@ extern "C" void gather(int n, const double *row, const double *du, int fu, int f
 '''
 
 
+SUMS = r'''
+// node sums of n terms: the two's complement 128-bit total
+extern "C" void sum128(int n, const double *v, int emax, u64 *out)
+{
+    Sum128 a = {0, 0};
+    for (int i = 0; i < n; i++) add_fixed(a, v[i], emax);
+    const u128 t = a.v + (u128)(u64)a.neg;
+    out[0] = (u64)t;
+    out[1] = (u64)(t >> 64);
+}
+extern "C" void sum64(int n, const float *v, int emax, u64 *out)
+{
+    Sum64 a = {0, 0};
+    for (int i = 0; i < n; i++) add_fixed(a, v[i], emax);
+    out[0] = a.v + (u64)a.neg;
+    out[1] = (u64)((i64)out[0] >> 63);
+}
+'''
+
+
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
     gxx = shutil.which("g++")
     if gxx is None:
         pytest.skip("no host compiler")
     d = tmp_path_factory.mktemp("fix")
-    (d / "fix.cpp").write_text(SRC + KIN)
+    (d / "fix.cpp").write_text(SRC + KIN + SUMS)
     so = str(d / "fix.so")
     subprocess.run([gxx, "-O2", "-std=gnu++17", "-shared", "-fPIC", "-I", CSRC, str(d / "fix.cpp"), "-o", so], check=True)
     L = C.CDLL(so)
     L.eval.argtypes = [C.c_int] + [C.c_void_p] * 3 + [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_uint64] + [C.c_void_p] * 3
     L.gather.argtypes = [C.c_int, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_void_p]
-    L.gather.restype = None
+    L.gather.restype = L.sum128.restype = L.sum64.restype = None
+    L.sum128.argtypes = L.sum64.argtypes = [C.c_int, C.c_void_p, C.c_int, C.c_void_p]
     return L
 
 
@@ -181,3 +202,33 @@ def test_fixed_point_kinematics_gather(lib, n, speed):
         for j in range(3):
             ref = sum(D(float(du[k, i])) * D(float(row[k, 1 + j])) for k in range(n))
             assert abs(D(float(out[3 + 3 * i + j])) - ref) <= D(2) ** -53 * abs(ref) + D(2) ** -57 * D(h) * D(rs)
+
+
+@pytest.mark.parametrize("emax", [1023, 3, -40, -900])
+def test_node_sum_terms(lib, emax):
+    """Node sums: each term is exactly trunc(v 2^(110 - emax)) (FP64) or trunc(v 2^(46 - emax)) (FP32) for exponents
+    from emax down past the last unit; zero, subnormal and non-finite terms count nothing."""
+    rng = np.random.default_rng(emax + 1000)
+    for bits, lsb, lo, fn in ((52, 110, -1022, lib.sum128), (23, 46, -126, lib.sum64)):
+        e = emax if bits == 52 else max(min(emax, 127), -60)
+        ex = np.concatenate([np.arange(e - 150, e + 1), [e, e, e - 63, e - 64, e - 47, e - 46]])
+        ex = np.repeat(ex[ex >= lo], 3)
+        m = rng.integers(0, 1 << bits, ex.size)
+        m[::7] = 0
+        m[1::7] = (1 << bits) - 1
+        sg = np.where(rng.uniform(size=ex.size) < 0.5, -1.0, 1.0)
+        v = np.ldexp(1.0 + m * 2.0 ** -bits, ex) * sg
+        tiny = np.ldexp(1.0, lo - 3)
+        v = np.concatenate([v, [0.0, -0.0, tiny, -tiny, np.inf, -np.inf, np.nan]])
+        v = np.ascontiguousarray(v, np.float64 if bits == 52 else np.float32)
+        out = np.zeros(2, np.uint64)
+        fn(v.size, v.ctypes.data_as(C.c_void_p), e, out.ctypes.data_as(C.c_void_p))
+        got = int(out[0]) | int(out[1]) << 64
+        got -= (1 << 128) if got >> 127 else 0
+        # whole numbers by shifting the significand, so that nothing is rounded
+        ref = 0
+        for mk, ek, sk in zip(m, ex, sg):
+            s = int(ek) - bits + lsb - e
+            t = (1 << bits) | int(mk)
+            ref += int(sk) * (t << s if s >= 0 else t >> -s)
+        assert got == ref
