@@ -249,6 +249,17 @@ def test_stabilised_residual_matches_oracle(orc, OTM):
     assert np.abs(plain.get("node_x") - sim_o.get("node_x")).max() > 1e-9
 
 
+@pytest.mark.parametrize("eps,v0", [(1e-4, 50.0), (1e-2, 400.0), (1e-1, 190.0)])
+def test_stabilised_steps_over_the_weights(orc, OTM, eps, v0):
+    """The penalty term over its range of weights, against the oracle."""
+    p = scenarios.taylor_rod(h=0.8e-3, R=3.2e-3, L=6.4e-3, v0=v0, material=scenarios.copper_jc())
+    p.eps_stab = eps * p.materials[0].E * p.h ** 2
+    sim_o, sim_g = orc.Sim(p), OTM(p)
+    assert sim_o.step(6) == 0 and sim_g.step(6) == 0, sim_g.error()
+    errs, bad = compare(sim_g, sim_o, {"default": 1e-10, "node_x": 1e-10, "mp_x": 1e-10})
+    assert not bad, (errs, bad)
+
+
 def insertion_rod(max_insert=200):
     p = scenarios.taylor_rod(h=0.8e-3, R=3.2e-3, L=6.4e-3, v0=2000.0, material=scenarios.copper_jc())
     p.max_insert = max_insert
