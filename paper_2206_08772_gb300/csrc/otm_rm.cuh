@@ -165,10 +165,10 @@ __device__ inline int return_map_point(const otm_material &M, double dt, const R
             double x = (in.guess > 0.0 && in.guess < hi) ? in.guess : 0.5 * hi;
             const double tol = 1e-12 * q_tr;
             bool ok = false;
+            double sy, dsy, g;
             for (int it = 0; it < 300; it++) {
-                double sy, dsy;
                 jc_sigma_y(M, in.ebar, x, dt, therm, sy, dsy);
-                const double g = q_tr - 3.0 * mu * x - sy;
+                g = q_tr - 3.0 * mu * x - sy;
                 if (fabs(g) <= tol) { ok = true; break; }
                 if (g > 0.0) lo = x; else hi = x;
                 if (hi - lo <= 4e-16 * hi) { ok = true; break; }
@@ -177,11 +177,8 @@ __device__ inline int return_map_point(const otm_material &M, double dt, const R
                 x = xn;
             }
             if (!ok) return OTM_ERR_RETURNMAP_NOCONV;
-            {   // one more Newton step: the accepted iterate is fixed only to the tolerance, the
-                // step fixes it to rounding, whatever the start (warm or the bracket's midpoint)
-                double sy, dsy;
-                jc_sigma_y(M, in.ebar, x, dt, therm, sy, dsy);
-                const double g = q_tr - 3.0 * mu * x - sy;
+            {   // one more Newton step from the accepted iterate's values: the iterate is fixed only to the
+                // tolerance, the step fixes it to rounding, whatever the start (warm or the bracket's midpoint)
                 const double xn = x - g / (-3.0 * mu - dsy);
                 if (xn > lo && xn < hi) x = xn;
             }
