@@ -1124,11 +1124,11 @@ __device__ __forceinline__ void lme_record(const Dev &D, int64_t p, double l0, d
     D.lam[3 * p + 2] = l2;
 }
 
-// Shared-memory rows per MP in k_lme and k_lme_fix. With 336 slots a block of 4 MPs takes 55 KB and 4 blocks
-// fit an SM (3 with full 384-slot rows), which hides more of the FP64 pipe's dependency and
+// Shared-memory rows per MP in k_lme and k_lme_fix. With 336 slots a block of 4 MPs takes 43 KB of rows: 5 blocks
+// of k_lme fit an SM, and 4 of k_lme_fix with its table, which hides more of the dependency and
 // barrier stalls; the supports of the benchmark rods stay below (at most 316 slots mid-run on the
-// 2.85 M-MP rod). MPs with larger supports are deferred to k_lme_wide, which runs the same block
-// code with rows of the full capacity S, so either launch gives the same bits.
+// 2.85 M-MP rod). MPs with larger supports are deferred to k_lme_wide, which runs k_lme's block
+// code with rows of the full capacity S.
 constexpr int kLmeRows = 336;
 
 __host__ __device__ __forceinline__ int lme_rows(int S) { return S < kLmeRows ? S : kLmeRows; }
@@ -1276,16 +1276,23 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
     const double *__restrict__ T = g_exp2_table;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = D.S;
-    MpNewton *NS = (MpNewton *)(smem_raw + (size_t)kLmeWarps * 5 * (size_t)rows * sizeof(double));
+    MpNewton *NS = (MpNewton *)(smem_raw + (size_t)kLmeWarps * 4 * (size_t)rows * sizeof(double));
     // every warp reaches the block barriers below; idle warps skip the work
-    WarpSmem W = warp_smem(smem_raw, rows, warp);
+    WarpSmem W;
+    W.dx = (double *)smem_raw + (size_t)warp * 4 * (size_t)rows;
+    W.dy = W.dx + rows;
+    W.dz = W.dy + rows;
+    W.q = W.dz + rows;
     const int64_t base = p * (int64_t)S;
     MpNewton &M = NS[warp];
-    int cnt = 0;
+    const int cnt = active ? D.cnt[p] : 0;
+    // the weights, packed at the end of the MP's pair rows in memory: without their 8 bytes a slot in shared
+    // memory a fifth block fits the SM (mixed, 616 k MPs: 14.89 -> 14.51 ms, the FP64 pipe 86 % busy). Row k
+    // reaches w_j only for k >= j, so the output loop below may overwrite them pass by pass.
+    W.w = (double *)(D.shape + base + S) - cnt;
     double shift0 = 0;
     if (active) {
         const double4_32a xp = D.xp[p];
-        cnt = D.cnt[p];
         // d_a = x_p - x_a and the prior exponent -beta |d_a|^2, minus the Newton solve's shift,
         // in units of ln2/1024
         const double beta_s = D.beta * kExpScale;
@@ -1332,8 +1339,11 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
     const float mpf = MIXED ? (float)mp : 0.f;
     LmeStab<STAB> stab;
     stab.load(D, p);
-    for (int k = lane; k < cnt; k += kWarp) {
-        const double wk = W.w[k];
+    for (int k0 = 0; k0 < cnt; k0 += kWarp) {
+        const int k = k0 + lane;
+        const double wk = k < cnt ? W.w[k] : 0.0;
+        __syncwarp();
+        if (k >= cnt) continue;
         const double N = wk * iZ;
         const double x = W.dx[k], y = W.dy[k], z = W.dz[k];
         double ex, ey, ez;
@@ -1391,7 +1401,7 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
 }
 
 template <bool MIXED, bool STAB>
-__global__ void __launch_bounds__(kLmeWarps * kWarp) k_lme(const Dev D)
+__global__ void __launch_bounds__(kLmeWarps * kWarp, 5) k_lme(const Dev D)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31;
@@ -1718,14 +1728,25 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4) k_lme_fix(const __grid_c
         active = false;
     }
     const int64_t base = p * (int64_t)S;
+    constexpr int G = 6;   // passes of dependent gathers in flight (4: 2.97 instead of 2.86 ms on 202,752 MPs)
     int cnt = 0;
     double shift0 = 0;
     if (active) {
         cnt = D.cnt[p];
         shift0 = D.logz[p];
-        for (int k = lane; k < cnt; k += kWarp) {
-            const longlong4_32a a = D.xfix[D.ids[base + k]];
-            F.x0[k] = a.x; F.x1[k] = a.y; F.x2[k] = a.z;
+        for (int k0 = lane; k0 < cnt; k0 += G * kWarp) {
+            int id[G];
+            longlong4_32a a[G];
+#pragma unroll
+            for (int j = 0; j < G; j++) id[j] = k0 + j * kWarp < cnt ? D.ids[base + k0 + j * kWarp] : -1;
+#pragma unroll
+            for (int j = 0; j < G; j++)
+                if (id[j] >= 0) a[j] = D.xfix[id[j]];
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                const int k = k0 + j * kWarp;
+                if (id[j] >= 0) { F.x0[k] = a[j].x; F.x1[k] = a[j].y; F.x2[k] = a[j].z; }
+            }
         }
         if (lane < 11) {   // the start formed by k_lme_prep
             const i64 v = ((const i64 *)&D.fstart[p])[lane];
@@ -1755,22 +1776,22 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4) k_lme_fix(const __grid_c
     }
     if (!active) return;
     if (!lme_finish(D, p, cnt, M, shift0, lane)) return;
-    // the pairs' node-major positions hang on two dependent loads: gathered ahead of the output loop, four
+    // the pairs' node-major positions hang on two dependent loads: gathered ahead of the output loop, G
     // passes in flight, into this warp's share of the exp table (every warp of the block is past its
     // last evaluation)
     int32_t *pos = (int32_t *)B.table + warp * (2 * kExpTable / kLmeWarps);
-    for (int k0 = lane; k0 < cnt; k0 += 4 * kWarp) {
-        int id[4], r[4];
+    for (int k0 = lane; k0 < cnt; k0 += G * kWarp) {
+        int id[G], r[G];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
+        for (int j = 0; j < G; j++) {
             const int k = k0 + j * kWarp;
             id[j] = k < cnt ? D.ids[base + k] : 0;
             r[j] = k < cnt ? D.rank[base + k] : 0;
         }
 #pragma unroll
-        for (int j = 0; j < 4; j++) r[j] += D.noff[id[j]];
+        for (int j = 0; j < G; j++) r[j] += D.noff[id[j]];
 #pragma unroll
-        for (int j = 0; j < 4; j++)
+        for (int j = 0; j < G; j++)
             if (k0 + j * kWarp < cnt) pos[k0 + j * kWarp] = r[j];
     }
     const double iZ = M.iZ, mp = D.mass[p];
@@ -1914,7 +1935,7 @@ FixConst make_fix_const(double beta, double rs2)
 
 static size_t lme_block_smem(int rows)
 {
-    return (size_t)kLmeWarps * 5 * (size_t)rows * sizeof(double) + (size_t)kLmeWarps * sizeof(MpNewton);
+    return (size_t)kLmeWarps * 4 * (size_t)rows * sizeof(double) + (size_t)kLmeWarps * sizeof(MpNewton);
 }
 
 // Which kernel (D.lme_fix, set by the step driver): the fixed-point one for the FP64 path's solves where
