@@ -1290,6 +1290,7 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
     // memory a fifth block fits the SM (mixed, 616 k MPs: 14.89 -> 14.51 ms, the FP64 pipe 86 % busy). Row k
     // reaches w_j only for k >= j, so the output loop below may overwrite them pass by pass.
     W.w = (double *)(D.shape + base + S) - cnt;
+    constexpr int G = 5;   // passes of dependent gathers in flight (3: 14.24 instead of 14.19 ms, mixed, 616 k MPs; 1: 14.54)
     double shift0 = 0;
     if (active) {
         const double4_32a xp = D.xp[p];
@@ -1298,11 +1299,22 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
         const double beta_s = D.beta * kExpScale;
         shift0 = D.logz[p];
         const double shift_s = shift0 * kExpScale;
-        for (int k = lane; k < cnt; k += kWarp) {
-            const double4_32a a = D.x[D.ids[base + k]];
-            const double x = xp.x - a.x, y = xp.y - a.y, z = xp.z - a.z;
-            W.dx[k] = x; W.dy[k] = y; W.dz[k] = z;
-            W.q[k] = fma(-beta_s, fma(z, z, fma(y, y, x * x)), -shift_s);
+        for (int k0 = lane; k0 < cnt; k0 += G * kWarp) {
+            int id[G];
+            double4_32a a[G];
+#pragma unroll
+            for (int j = 0; j < G; j++) id[j] = k0 + j * kWarp < cnt ? D.ids[base + k0 + j * kWarp] : -1;
+#pragma unroll
+            for (int j = 0; j < G; j++)
+                if (id[j] >= 0) a[j] = D.x[id[j]];
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+                if (id[j] < 0) continue;
+                const int k = k0 + j * kWarp;
+                const double x = xp.x - a[j].x, y = xp.y - a[j].y, z = xp.z - a[j].z;
+                W.dx[k] = x; W.dy[k] = y; W.dz[k] = z;
+                W.q[k] = fma(-beta_s, fma(z, z, fma(y, y, x * x)), -shift_s);
+            }
         }
         if (lane == 0) {
             lme_start(D, p, M, shift0);
@@ -1329,6 +1341,23 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
     if (!active) return;
     if (!lme_finish(D, p, cnt, M, shift0, lane)) return;
 
+    // the pairs' node-major positions hang on two dependent loads: gathered ahead of the output loop into the
+    // exponents' row
+    int32_t *pos = (int32_t *)W.q;
+    for (int k0 = lane; k0 < cnt; k0 += G * kWarp) {
+        int id[G], rk[G];
+#pragma unroll
+        for (int j = 0; j < G; j++) {
+            const int k = k0 + j * kWarp;
+            id[j] = k < cnt ? D.ids[base + k] : 0;
+            rk[j] = k < cnt ? D.rank[base + k] : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < G; j++) rk[j] += D.noff[id[j]];
+#pragma unroll
+        for (int j = 0; j < G; j++)
+            if (k0 + j * kWarp < cnt) pos[k0 + j * kWarp] = rk[j];
+    }
     const double iZ = M.iZ, mp = D.mass[p];
     double Q[9];
     lme_force_matrix(D, p, M, lane, Q);
@@ -1360,10 +1389,8 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
             ex = N * x; ey = N * y; ez = N * z;
         }
         D.shape[base + k] = make_double4_32a(N, ex, ey, ez);
-        const int id = D.ids[base + k];
-        const int64_t pos = (int64_t)D.noff[id] + D.rank[base + k];
         double sx = 0.0, sy = 0.0, sz = 0.0;
-        stab.term(D, id, N, x, y, z, sx, sy, sz);
+        if (STAB) stab.term(D, D.ids[base + k], N, x, y, z, sx, sy, sz);
         if (MIXED) {
             const float c0 = mpf * fN;
             float c1 = fmaf(Qf[2], fez, fmaf(Qf[1], fey, Qf[0] * fex));
@@ -1374,7 +1401,7 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
                 c2 += f32_round_bits(sy);
                 c3 += f32_round_bits(sz);
             }
-            D.contrib32[pos] = make_float4(c0, c1, c2, c3);
+            D.contrib32[pos[k]] = make_float4(c0, c1, c2, c3);
             em = max(em, fexp32(c0));
             ef = max(ef, max(fexp32(c1), max(fexp32(c2), fexp32(c3))));
         } else {
@@ -1387,7 +1414,7 @@ __device__ __forceinline__ void lme_block(const Dev &D, int64_t p, bool active, 
                 fy += sy;
                 fz += sz;
             }
-            D.contrib64[pos] = make_double4_32a(cm, fx, fy, fz);
+            D.contrib64[pos[k]] = make_double4_32a(cm, fx, fy, fz);
             em = max(em, fexp64(cm));
             ef = max(ef, max(fexp64(fx), max(fexp64(fy), fexp64(fz))));
         }
@@ -2568,9 +2595,20 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
         const float bf = (float)beta, lf0 = (float)l0, lf1 = (float)l1, lf2 = (float)l2, u32 = (float)(C.r_unit * 0x1p32);
         i64 far = 0;                // largest |D| of any component
         float mx = -INFINITY, sum = 0.f;   // running log-sum of the exponents at the start
-        for (int k = lane; k < n; k += kWarp) {
-            double a[3];
-            nx.get(ids[base + k], a[0], a[1], a[2]);
+        constexpr int G = 4;        // passes of dependent gathers in flight (150 k points: 1 3.56, 2 3.47, 4 3.45 ms)
+        for (int k0 = lane; k0 < n; k0 += G * kWarp) {
+            int id[G];
+            double ag[G][3];
+#pragma unroll
+            for (int j = 0; j < G; j++) id[j] = k0 + j * kWarp < n ? ids[base + k0 + j * kWarp] : -1;
+#pragma unroll
+            for (int j = 0; j < G; j++)
+                if (k0 + j * kWarp < n) nx.get(id[j], ag[j][0], ag[j][1], ag[j][2]);
+#pragma unroll
+            for (int j = 0; j < G; j++) {
+            const int k = k0 + j * kWarp;
+            if (k >= n) continue;
+            const double (&a)[3] = ag[j];
             float d[3];
 #pragma unroll
             for (int i = 0; i < 3; i++) {
@@ -2586,6 +2624,7 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
             const float m2 = fmaxf(mx, f);
             sum = sum * __expf(mx - m2) + __expf(f - m2);
             mx = m2;
+            }
         }
         const float wm = warp_max_f(mx);
         const float ws = warp_sumf(sum > 0.f ? sum * __expf(mx - wm) : 0.f);
@@ -2638,6 +2677,7 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
     double K[6];
 #pragma unroll
     for (int i = 0; i < 6; i++) K[i] = -M.inv[i] * Z;
+    const bool wide = ((uintptr_t)shape & 31) == 0;
 #pragma unroll 1
     for (int k = lane; k < n; k += kWarp) {
         const double N = w[k * ws] * iZ;
@@ -2650,10 +2690,13 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
             ex = N * (px - ax); ey = N * (py - ay); ez = N * (pz - az);
         }
         double *o = shape + 4 * (base + k);
-        o[0] = N;
-        o[1] = fma(K[0], ex, fma(K[3], ey, K[5] * ez));
-        o[2] = fma(K[3], ex, fma(K[1], ey, K[4] * ez));
-        o[3] = fma(K[5], ex, fma(K[4], ey, K[2] * ez));
+        const double4_32a row = make_double4_32a(N, fma(K[0], ex, fma(K[3], ey, K[5] * ez)), fma(K[3], ex, fma(K[1], ey, K[4] * ez)),
+                                                 fma(K[5], ex, fma(K[4], ey, K[2] * ez)));
+        if (wide) {
+            *(double4_32a *)o = row;
+        } else {
+            o[0] = row.x; o[1] = row.y; o[2] = row.z; o[3] = row.w;
+        }
     }
 }
 
