@@ -63,20 +63,19 @@ MIXED_DTYPE = ("f32 scatter/node update/kinematics gather/row N d, double-float 
 #  algorithmic, the method's own work (the exp not counted as flops): per evaluation 25 (exponent
 #  lambda . d + prior: 6; Z, r, J = sum w d d^T: 1 + 6 + 12), once 15 (d_a and the prior term,
 #  N, grad N) and 17 (mass and force contributions): (1 + k) 25 + 32.
-#  executed in FP64 by this kernel: setup 10 (d, prior exponent), per evaluation 29 (exponent 6,
-#  the table exp's two FMAs 4 (its range reduction in integer operations, its polynomial in
-#  double-float on the FP32 pipe), w d 3, Z 1, r 3, J 12), final 20 (N 1, e = N d 3, mass 1,
-#  force Q e 15): 30 + 29 (1 + k).
+#  executed in FP64 by the FP64 path's kernel: 17 once (N 1, mass 1, force Q e 15). Its evaluations
+#  (exponent, exp, Z, r, J) and e = N d run in fixed point on the integer pipes, so the algorithmic
+#  rate may exceed the FP64 peak.
 LME_ALG_PER_EVAL, LME_ALG_ONCE = 25, 32
-LME_EXEC_PER_EVAL, LME_EXEC_ONCE = 29, 30
+LME_EXEC_PER_EVAL, LME_EXEC_ONCE = 0, 17
 #  k_search (FP32): 8 flops per candidate (3 sub, 1 mul, 2 fma); candidates ~ 3.73 x support.
-#  k_kinematics (FP64): 24 flops per pair (x_p: 3 fma, G = sum du (x) e: 9 fma).
+#  k_kinematics: 24 flops per pair (x_p: 3 fma, G = sum du (x) e: 9 fma; the FP64 path's in fixed point).
 SEARCH_PER_CAND, CAND_PER_PAIR = 8, 3.73
 KIN_PER_PAIR = 24
-# DRAM bytes per pair of one k_lme launch, from the ncu capture of the h 0.29 mm rod at step 302
-# (dram__bytes_read.sum + dram__bytes_write.sum = 3.959 GB over 54.11 M pairs); the traffic of
+# DRAM bytes per pair of one k_lme_fix launch, from the ncu capture of the h 0.4 mm rod
+# (dram__bytes_read.sum + dram__bytes_write.sum = 1.440 GB over 20.17 M pairs); the traffic of
 # a launch scales with its pairs (shape and contribution writes, ID and rank reads)
-LME_DRAM_BYTES_PER_PAIR = (0.395994e9 + 3.563405e9) / (202752 * 266.871)
+LME_DRAM_BYTES_PER_PAIR = (0.150299e9 + 1.289973e9) / (78624 * 256.6)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12   # 2 FP64 FMA lanes / SM / clock at 2070 MHz
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 
@@ -694,7 +693,7 @@ def main():
                       "frac": tf / (ms_k / 1e3) / peak}
     dom = max(kernels, key=lambda k: kernels[k]["ms"])
     kd = kernels[dom]
-    roofline = {"kernel": f"k_{dom}", "bound": "alu", "achieved": kd["achieved_tflops"], "peak": kd["peak"],
+    roofline = {"kernel": "k_lme_fix" if dom == "lme" and args.precision == "fp64" else f"k_{dom}", "bound": "alu", "achieved": kd["achieved_tflops"], "peak": kd["peak"],
                 "unit": "TFLOP/s", "frac": kd["frac"],
                 # the executed-flop count and the captured DRAM bytes are those of the FP64 path's kernel
                 "frac_executed": ((lme_exec / (kd["ms"] / 1e3) / kd["peak"])
@@ -703,7 +702,7 @@ def main():
                                    "executed": (LME_EXEC_PER_EVAL * (1 + k_bar) + LME_EXEC_ONCE
                                                 if args.precision == "fp64" else None)},
                 "traffic": LME_DRAM_BYTES_PER_PAIR * pairs if dom == "lme" and args.precision == "fp64" else None,
-                "traffic_note": ("bytes per launch: DRAM bytes per pair of the ncu capture on the 202,752-MP rod "
+                "traffic_note": ("bytes per launch: DRAM bytes per pair of the ncu capture on the 78,624-MP rod "
                                  "(profiles/) x this launch's pairs"),
                 "peak_source": ("derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2070 MHz (no FP64 entry in the "
                                 "measured peaks)" if kd["kind"] == "fp64"

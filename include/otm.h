@@ -54,7 +54,7 @@ extern "C" {
 #define OTM_ERR_RETURNMAP_NOCONV (-7) /* Johnson-Cook consistency iteration failed */
 #define OTM_ERR_CAPACITY (-8)         /* support / influence / cell capacity exceeded */
 
-#define OTM_PRECISION_FP64 0          /* every step in FP64 */
+#define OTM_PRECISION_FP64 0          /* FP64 accuracy throughout (pair sums in 59- to 64-bit fixed point) */
 #define OTM_PRECISION_MIXED 1         /* FP32 force scatter, node update, pair rows' e = N d and
                                        * kinematics gather (x_p increment and G = sum du (x) N d);
                                        * the LME Newton's Hessian sums in double-float (FP32 pairs,
@@ -270,7 +270,8 @@ int otm_snapshot_bytes(otm_handle *h, size_t *bytes);
 /* Copy the complete state into / from a snapshot. Loading regenerates the shape functions and
  * node-major lists from the stored state, reproducing them exactly. A snapshot loads into any
  * handle made with the same problem sizes, max_support and max_insert, of either precision
- * (otherwise OTM_ERR_ARG); the FP32 increments are rebuilt from the FP64 ones. */
+ * (otherwise OTM_ERR_ARG); the FP32 increments are rebuilt from the FP64 ones, and the shape functions
+ * by the kind of evaluation (fixed point or FP64) that produced the stored state. */
 int otm_snapshot_save(otm_handle *h, void *dst);
 int otm_snapshot_load(otm_handle *h, const void *src);
 

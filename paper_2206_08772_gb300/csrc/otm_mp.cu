@@ -5,7 +5,8 @@
 //                  Ascending-ID sort, influence counting (integer atomics -> rank).
 //   k_lme        : Eq. 14, warp per MP: damped Newton for lambda (warm start, exponent shift from
 //                  the previous log Z), N and grad N = -N J^-1 d, per-pair contributions
-//                  (m_p N, -v sigma grad N) written straight into node-major order.
+//                  (m_p N, -v sigma grad N) written straight into node-major order. k_lme_fix: the same
+//                  with the pair sums in fixed point (the FP64 path; k_lme is the mixed path's).
 //   k_kinematics : Eq. 9-13, warp per MP: x_p = sum N x_I, dF = 1 + sum du_I (x) grad N_I,
 //                  F <- dF F, v <- det(dF) v
 //   k_return_map : Sec. 4.1 / 4.2, thread per MP: Hencky exponential-map radial return (J2
@@ -1476,11 +1477,11 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp) k_lme_wide(const Dev D)
 // only sees the scalars and the force contributions.
 //
 // Bound: k_lme keeps the FP64 pipe 89 % busy (19 FP64 instructions a pair and evaluation). Here it is
-// 47 % busy (11 a pair for the force contributions and N, plus the rounds' scalars), and the integer
+// 43 % busy (11 a pair for the force contributions and N, plus the rounds' scalars), and the integer
 // instructions (about 200 a pair and evaluation, two to four cycles of an SM quarter each) and their
 // latency at 16 warps an SM (128 registers; four blocks of 54 KB) bound the kernel.
 // Measured on the 202,752-MP rod (267 pairs an MP, 1.19 Newton iterations): k_lme 7.78 ms, this kernel
-// 2.96 ms (with k_lme_prep). Five blocks an SM (96 registers, the exp table in L1) take 3.40 ms: spills.
+// 2.87 ms (with k_lme_prep). Five blocks an SM (96 registers, the exp table in L1) take 15 % longer: spills.
 struct MpFix {
     i64 xp[3];         // X of the material point
     i64 v[3];          // centre offset of the pending trial, lambda / (2 beta) in LSB
