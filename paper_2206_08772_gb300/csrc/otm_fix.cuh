@@ -348,6 +348,52 @@ OTM_HD float fix_to_float(i64 D, int fb)
     return f;
 }
 
+// ------------------------------------------------------------------ force contributions (Eq. 5)
+// f = N Q D 2^-fb of fixed-point separations D (|D| < 2^62) and an FP64 matrix Q per material point. Rows of Q
+// as 60-bit integers of the row's own exponent, in limbs q = qh 2^32 + ql; what is dropped (ql dl and the
+// rounding of Q) stays below 5 units of F: 2^-56 of the row's largest entry times 2^62.
+struct FixRows {
+    int qh[9], ql[9], fb[3];   // fb: the exponent of F in fix_mul_double
+    bool ok;                   // false if a row is zero, not finite or far out of range: FP64 then
+};
+
+OTM_HD void fix_rows(const double (&Q)[9], int fb, FixRows &R)
+{
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        int e = 0;
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const int ej = (int)(fx_d_bits(Q[3 * i + j]) >> 52) & 0x7ff;
+            e = e > ej ? e : ej;
+        }
+        ok = ok && e > 600 && e < 1450;
+        const int s = 60 - (e - 1022);                        // |Q_ij| < 2^(e - 1022)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const i64 q = fix_from_double(Q[3 * i + j], s);
+            R.qh[3 * i + j] = (int)((q + 0x80000000LL) >> 32);
+            R.ql[3 * i + j] = (int)q;
+        }
+        R.fb[i] = fb + s - 62;
+    }
+    R.ok = ok;
+}
+
+// row i: F = sum_j q_ij D_j in units of 2^62, below 2^62
+OTM_HD i64 fix_row_dot(const FixRows &R, int i, const int (&dh)[3], const int (&dl)[3])
+{
+    i64 hh = 0, hl = 1LL << 29;
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        const int qh = R.qh[3 * i + j];
+        hh = fx_madw(qh, dh[j], hh);
+        hl = fx_madw(qh, dl[j], fx_madw(R.ql[3 * i + j], dh[j], hl));
+    }
+    return (hh << 2) + (hl >> 30);
+}
+
 // ------------------------------------------------------------------ kinematics gather (Eq. 9, 11)
 // The products of a pair's row (N, e) with its node's increment du, summed over the support:
 // sum N du (3) and G = sum du (x) e (9). Limbs: du = uh 2^28 + ul (|du| < 2^57 units; uh 29 bits, ul signed 28

@@ -5,6 +5,7 @@ import os
 import shutil
 import subprocess
 from decimal import Decimal, getcontext
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -88,6 +89,22 @@ extern "C" void gather(int n, const double *row, const double *du, int fu, int f
 '''
 
 
+FORCE = r'''
+// f = N Q D 2^-fb; returns whether the rows are in range
+extern "C" int force(const double *Q, double N, const i64 *D, int fb, double *f)
+{
+    double q[9];
+    for (int i = 0; i < 9; i++) q[i] = Q[i];
+    FixRows R;
+    fix_rows(q, fb, R);
+    const int dh[3] = {(int)((D[0] + 0x80000000LL) >> 32), (int)((D[1] + 0x80000000LL) >> 32), (int)((D[2] + 0x80000000LL) >> 32)};
+    const int dl[3] = {(int)D[0], (int)D[1], (int)D[2]};
+    const u64 nb = fx_d_bits(N), nm = ((nb & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
+    if (R.ok) for (int i = 0; i < 3; i++) f[i] = fix_mul_double(nm, (int)(nb >> 52), fix_row_dot(R, i, dh, dl), R.fb[i]);
+    return R.ok;
+}
+'''
+
 SUMS = r'''
 // node sums of n terms: the two's complement 128-bit total
 extern "C" void sum128(int n, const double *v, int emax, u64 *out)
@@ -114,13 +131,14 @@ def lib(tmp_path_factory):
     if gxx is None:
         pytest.skip("no host compiler")
     d = tmp_path_factory.mktemp("fix")
-    (d / "fix.cpp").write_text(SRC + KIN + SUMS)
+    (d / "fix.cpp").write_text(SRC + KIN + FORCE + SUMS)
     so = str(d / "fix.so")
     subprocess.run([gxx, "-O2", "-std=gnu++17", "-shared", "-fPIC", "-I", CSRC, str(d / "fix.cpp"), "-o", so], check=True)
     L = C.CDLL(so)
     L.eval.argtypes = [C.c_int] + [C.c_void_p] * 3 + [C.c_double, C.c_double, C.c_int, C.c_void_p, C.c_uint64] + [C.c_void_p] * 3
     L.gather.argtypes = [C.c_int, C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_void_p]
     L.gather.restype = L.sum128.restype = L.sum64.restype = None
+    L.force.argtypes = [C.c_void_p, C.c_double, C.c_void_p, C.c_int, C.c_void_p]
     L.sum128.argtypes = L.sum64.argtypes = [C.c_int, C.c_void_p, C.c_int, C.c_void_p]
     return L
 
@@ -232,3 +250,28 @@ def test_node_sum_terms(lib, emax):
             t = (1 << bits) | int(mk)
             ref += int(sk) * (t << s if s >= 0 else t >> -s)
         assert got == ref
+
+
+@pytest.mark.parametrize("scale,spread", [(1.0, 0), (1e-90, 3), (1e60, 12), (3e7, 40)])
+def test_force_rows(lib, scale, spread):
+    """f = N Q d with rows of Q of any scale and entries up to 2^spread apart: half an ulp of f and 2^-56 of the
+    row's largest entry times N and 2^62 units (5 units of F and one of the product); zero and infinite rows are out
+    of range."""
+    rng = np.random.default_rng(spread)
+    fb = 70
+    ptr = lambda t: t.ctypes.data_as(C.c_void_p)
+    f = np.zeros(3)
+    for _ in range(200):
+        Q = np.ascontiguousarray(rng.uniform(-1, 1, 9) * scale * 2.0 ** rng.integers(-spread, 1, 9))
+        d = rng.integers(-(1 << 62) + 1, 1 << 62, 3)
+        N = float(rng.uniform(0.5, 1.0) * 2.0 ** rng.integers(-30, 1))
+        assert lib.force(ptr(Q), N, ptr(d), fb, ptr(f))
+        for i in range(3):
+            q = [Fraction(float(v)) for v in Q[3 * i:3 * i + 3]]
+            ref = sum(a * int(b) for a, b in zip(q, d)) * Fraction(N) / 2 ** fb
+            tol = abs(ref) / 2 ** 53 + max(abs(a) for a in q) * Fraction(N) * Fraction(2 ** 62, 2 ** fb) / 2 ** 56
+            assert abs(Fraction(float(f[i])) - ref) <= tol
+    for bad in (0.0, np.inf, np.nan):
+        Q = np.ones(9)
+        Q[3:6] = bad
+        assert not lib.force(ptr(Q), 0.5, ptr(d), fb, ptr(f))
