@@ -27,9 +27,9 @@
  *  - After an error the state is that of the failing step, partially updated (the oracle
  *    behaves the same way); otm_error_detail names the code and the smallest offending ID.
  *    otm_keep_last_good makes otm_step leave the state at the last good step instead.
- *  - Device reset: the library keeps two pieces of module data per device (the table of its
- *    FP64 exponential and the allocation-free search's scratch address), set up by the first
- *    call on that device. A reset of the device or of its primary context (cudaDeviceReset)
+ *  - Device reset: the library keeps two pieces of module data per device (the tables of its
+ *    FP64 exponential and logarithm, and the allocation-free search's scratch address), set up by
+ *    the first call on that device. A reset of the device or of its primary context (cudaDeviceReset)
  *    discards module data: otm_init checks for that and sets the table up again, so a reset must
  *    be followed by otm_init before the stand-alone kernels are used; the allocation-free search
  *    is not supported after a reset in the same process.
@@ -350,12 +350,13 @@ int otm_lme(const double *node_x, const double *mp_x, int64_t n_mps, const int32
 /* Self-test of the library's internal FP64 exponential (table-driven after Tang, used for the
  * LME weights of Eq. 14). Its argument is scaled: y = f * 1024 / ln 2. Device arrays of n
  * doubles: mine[i] = internal exp of f_i = y[i] ln2/1024; ref[i] = CUDA's exp of the same f_i
- * (carried as a rounded product plus its error, so ref is accurate to about an ulp). The first
- * call on a device uploads the exponential's table (synchronous copy). */
+ * (carried as a rounded product plus its error, so ref is accurate to about an ulp). */
 int otm_exp_selftest(const double *y, int64_t n, double *mine, double *ref, void *stream);
 
 /* Constitutive update (Sec. 4.1 / 4.2) of n_mps points: inputs dF (9), F_new (9, for J),
- * be (6, in/out), ebar, T (in/out); outputs sigma (6), rate, failed (uint8, optional). */
+ * be (6, in/out), ebar, T (in/out); outputs sigma (6), rate, failed (uint8, optional). Like otm_lme
+ * and otm_exp_selftest, the first call on a device uploads the library's tables and waits for that
+ * copy (allowed while a stream is being captured). */
 int otm_return_map(const otm_material *mat, double dt, int64_t n_mps, const double *dF,
                    const double *F_new, double *be, double *ebar, double *T, double *sigma,
                    double *rate, uint8_t *failed, int32_t *status, void *stream);

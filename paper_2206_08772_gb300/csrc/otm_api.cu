@@ -1307,6 +1307,7 @@ extern "C" int otm_return_map(const otm_material *mat, double dt, int64_t n_mps,
 {
     if (!mat || !status || n_mps < 0 || !(dt > 0)) return OTM_ERR_ARG;
     if (n_mps > 0 && (!dF || !F_new || !be || !ebar || !T || !sigma)) return OTM_ERR_ARG;
+    if (n_mps > 0) CK(exp_table_setup());
     CK(launch_return_map_only(mat, dt, n_mps, dF, F_new, be, ebar, T, sigma, rate, failed, status,
                               (cudaStream_t)stream));
     return OTM_OK;

@@ -101,11 +101,33 @@ static __device__ double g_exp2_table[kExpTable];
 static __device__ u64 g_exp2_mant[kExpTable];          // 2^(j/1024) as 64-bit mantissas (fix_exp)
 static __device__ double2 g_log_table[kExpTable];      // (r, -log r), see log_pos
 
-// Fill g_exp2_table on the current device (first call per device; a synchronous copy, so it
-// belongs before any stream capture: otm_init and the stand-alone entries call it). With
+// Upload the three tables to the current device in a stream of its own. A synchronous copy belongs before any
+// stream capture, but the stand-alone entries may be called first under one (this thread's or another's):
+// a non-blocking stream has no part in a capture, and relaxed mode lets this thread use it meanwhile.
+static cudaError_t upload_tables(const double *exp2, const u64 *mant, const double2 *lg)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return e;
+    cudaStream_t s = nullptr;
+    e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e == cudaSuccess) {
+        const cudaMemcpyKind k = cudaMemcpyHostToDevice;
+        e = cudaMemcpyToSymbolAsync(g_exp2_mant, mant, kExpTable * sizeof(u64), 0, k, s);
+        if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(g_log_table, lg, kExpTable * sizeof(double2), 0, k, s);
+        if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(g_exp2_table, exp2, kExpTable * sizeof(double), 0, k, s);
+        const cudaError_t es = cudaStreamSynchronize(s), ed = cudaStreamDestroy(s);
+        if (e == cudaSuccess) e = es != cudaSuccess ? es : ed;
+    }
+    const cudaError_t em = cudaThreadExchangeStreamCaptureMode(&mode);
+    return e != cudaSuccess ? e : em;
+}
+
+// Fill the tables on the current device (first call per device: otm_init and every stand-alone entry whose
+// kernels read them). With
 // `verify`, a device whose table was already filled is checked again (a synchronous 8-byte read
 // of 2^0 = 1): module data is lost when the device or its primary context is reset, and the
-// table is then filled anew. otm_init verifies; the stand-alone entries, which must stay free of
+// tables are then filled anew. otm_init verifies; the stand-alone entries, which must stay free of
 // synchronisation once set up, do not.
 cudaError_t exp_table_setup(bool verify)
 {
@@ -128,8 +150,6 @@ cudaError_t exp_table_setup(bool verify)
     u64 mant[kExpTable];
     for (int j = 0; j < kExpTable; j++)
         mant[j] = (u64)std::floor(std::ldexp(std::exp2((long double)j / (long double)kExpTable), 63) + 0.5L);
-    e = cudaMemcpyToSymbol(g_exp2_mant, mant, sizeof(mant));
-    if (e != cudaSuccess) return e;
     double2 lg[kExpTable];   // (r, -log r), r ~ 1/m at the middle of the interval (1 exactly about m = 1)
     for (int j = 0; j < kExpTable; j++) {
         double m = 1.0 + (j + 0.5) / kExpTable;
@@ -137,9 +157,7 @@ cudaError_t exp_table_setup(bool verify)
         const double r = (j == 0 || j == kExpTable - 1) ? 1.0 : 1.0 / m;
         lg[j] = make_double2(r, (double)-std::log((long double)r));
     }
-    e = cudaMemcpyToSymbol(g_log_table, lg, sizeof(lg));
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyToSymbol(g_exp2_table, host, sizeof(host));
+    e = upload_tables(host, mant, lg);
     if (e == cudaSuccess) done[dev] = true;
     return e;
 }
