@@ -79,6 +79,7 @@ OTM_HD uint32_t fx_umulhi(uint32_t a, uint32_t b) { return (uint32_t)(((u64)a * 
 OTM_HD uint32_t fx_shf_r(uint32_t lo, uint32_t hi, int s) { return (uint32_t)((((u64)hi << 32) | lo) >> (s & 31)); }
 OTM_HD int fx_log2(uint32_t v)
 {
+    if (!v) return -127;   // as the device's
     int l = -1;
     while (v) { v >>= 1; l++; }
     return l;
@@ -309,8 +310,8 @@ OTM_HD i64 fix_floor(double v, int f)
     return (i64)(m >> (s < 63 ? s : 63)) ^ ((i64)b >> 63);
 }
 
-// N D 2^-fb as FP64 for N > 0 given by its significand nm (in [2^63, 2^64)) and biased exponent en,
-// and 2^32 <= |D| < 2^63: the leading 64 bits of the product (rounded: half a unit is at most one unit
+// N D 2^-fb as FP64 for N > 0 given by its significand nm (in [2^63, 2^64)) and biased exponent en, inside
+// fix_mul_in_range: the leading 64 bits of the product (rounded: half a unit is at most one unit
 // of D), normalised and rounded to nearest
 OTM_HD double fix_mul_double(u64 nm, int en, i64 D, int fb)
 {
@@ -324,6 +325,36 @@ OTM_HD double fix_mul_double(u64 nm, int en, i64 D, int fb)
     p = ((p << lz) + 512ULL) >> 10;                      // 53 bits, the leading one adds to the exponent
     const uint32_t hi = (uint32_t)(p >> 32) + ((uint32_t)(en + 62 - fb - lz) << 20);
     return fx_bits_d(((u64)(hi | ((uint32_t)sg & 0x80000000u)) << 32) | (uint32_t)p);
+}
+
+// Whether N, of biased exponent en, times each of a, b, c is in fix_mul_double's range: 2^33 <= |D| < 2^63, so
+// that the high word of the product is not zero (it is normalised by that word), and N large enough
+// for a normal result with any fb in [-60, 540]. By the high words, floors: 3 and above, -3 and below.
+OTM_HD bool fix_mul_in_range(int en, i64 a, i64 b, i64 c)
+{
+    const int ah = (int)(a >> 32), bh = (int)(b >> 32), ch = (int)(c >> 32);
+    const int am = ah < 0 ? -ah : ah, bm = bh < 0 ? -bh : bh, cm = ch < 0 ? -ch : ch;
+    const int m = am < bm ? am : bm;
+    return (m < cm ? m : cm) > 2 && en > 600;
+}
+
+// the significand of a normal v > 0 in [2^63, 2^64)
+OTM_HD u64 fix_significand(double v) { return ((fx_d_bits(v) & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11; }
+
+// e = N d from the fixed-point separation; in FP64 where a component is within 2^-30 of the range or N is tiny
+OTM_HD void fix_nd(double N, i64 d0, i64 d1, i64 d2, int fb, double unit, double &ex, double &ey, double &ez)
+{
+    const u64 nm = fix_significand(N);
+    const int en = (int)(fx_d_bits(N) >> 52);
+    if (fix_mul_in_range(en, d0, d1, d2)) {
+        ex = fix_mul_double(nm, en, d0, fb);
+        ey = fix_mul_double(nm, en, d1, fb);
+        ez = fix_mul_double(nm, en, d2, fb);
+    } else {
+        ex = N * ((double)d0 * unit);
+        ey = N * ((double)d1 * unit);
+        ez = N * ((double)d2 * unit);
+    }
 }
 
 // D 2^-fb rounded to FP32 (nearest, ties away from zero; |D| < 2^63)
@@ -392,6 +423,21 @@ OTM_HD i64 fix_row_dot(const FixRows &R, int i, const int (&dh)[3], const int (&
         hl = fx_madw(qh, dl[j], fx_madw(R.ql[3 * i + j], dh[j], hl));
     }
     return (hh << 2) + (hl >> 30);
+}
+
+// f = Q e from the fixed-point separation; false: out of range, FP64 then
+OTM_HD bool force_fix(const FixRows &R, double N, i64 d0, i64 d1, i64 d2, double &fx, double &fy, double &fz)
+{
+    const int dh[3] = {(int)((d0 + 0x80000000LL) >> 32), (int)((d1 + 0x80000000LL) >> 32), (int)((d2 + 0x80000000LL) >> 32)};
+    const int dl[3] = {(int)d0, (int)d1, (int)d2};
+    const i64 F0 = fix_row_dot(R, 0, dh, dl), F1 = fix_row_dot(R, 1, dh, dl), F2 = fix_row_dot(R, 2, dh, dl);
+    const u64 nm = fix_significand(N);
+    const int en = (int)(fx_d_bits(N) >> 52);
+    if (!R.ok || !fix_mul_in_range(en, F0, F1, F2)) return false;
+    fx = fix_mul_double(nm, en, F0, R.fb[0]);
+    fy = fix_mul_double(nm, en, F1, R.fb[1]);
+    fz = fix_mul_double(nm, en, F2, R.fb[2]);
+    return true;
 }
 
 // ------------------------------------------------------------------ kinematics gather (Eq. 9, 11)

@@ -1740,41 +1740,6 @@ __device__ __noinline__ void lme_eval64(X x, const int32_t *ids, double px, doub
     if (lane == 0) m.E[10] = sh;
 }
 
-// e = N d from the fixed-point separation
-__device__ __forceinline__ void fix_nd(double N, i64 d0, i64 d1, i64 d2, int fb, double unit, double &ex, double &ey,
-                                       double &ez)
-{
-    const u64 nb = fx_d_bits(N);
-    const u64 nm = ((nb & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
-    const int en = (int)(nb >> 52);
-    // a component within 2^-31 of the range (the last 32 bits of D), or N subnormal: FP64
-    const int least = min(min(abs((int)(d0 >> 32)), abs((int)(d1 >> 32))), abs((int)(d2 >> 32)));
-    if (least > 1 && en > 0) {
-        ex = fix_mul_double(nm, en, d0, fb);
-        ey = fix_mul_double(nm, en, d1, fb);
-        ez = fix_mul_double(nm, en, d2, fb);
-    } else {
-        const double Nu = N * unit;
-        ex = Nu * (double)d0; ey = Nu * (double)d1; ez = Nu * (double)d2;
-    }
-}
-
-// f = Q e from the fixed-point separation; false: out of range, FP64 then
-__device__ __forceinline__ bool force_fix(const FixRows &R, double N, i64 d0, i64 d1, i64 d2, double &fx, double &fy, double &fz)
-{
-    const int dh[3] = {(int)((d0 + 0x80000000LL) >> 32), (int)((d1 + 0x80000000LL) >> 32), (int)((d2 + 0x80000000LL) >> 32)};
-    const int dl[3] = {(int)d0, (int)d1, (int)d2};
-    const i64 F0 = fix_row_dot(R, 0, dh, dl), F1 = fix_row_dot(R, 1, dh, dl), F2 = fix_row_dot(R, 2, dh, dl);
-    const u64 nb = fx_d_bits(N), nm = ((nb & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
-    const int en = (int)(nb >> 52);
-    const int least = min(min(abs((int)(F0 >> 32)), abs((int)(F1 >> 32))), abs((int)(F2 >> 32)));
-    if (!R.ok || least <= 1 || en <= 500) return false;
-    fx = fix_mul_double(nm, en, F0, R.fb[0]);
-    fy = fix_mul_double(nm, en, F1, R.fb[1]);
-    fz = fix_mul_double(nm, en, F2, R.fb[2]);
-    return true;
-}
-
 // shared memory of one block: the exp table, the warps' rows (a compile-time stride, so that a slot's four
 // words share one address register) and the solves' states
 struct FixBlock {
