@@ -52,7 +52,8 @@ struct SearchConst {
 // the start of one MP's fixed-point LME solve (k_lme_prep -> k_lme_fix, copied word by word)
 struct FixStart {
     double trial[3];
-    i64 xp[3], v[3], cst, ok, pad;
+    i64 xp[3], v[3], cst, ok;
+    double vmax;
 };
 
 // a material's derived constants (return_map_small)

@@ -1505,19 +1505,20 @@ struct MpFix {
     i64 v[3];          // centre offset of the pending trial, lambda / (2 beta) in LSB
     i64 cst;           // the trial's exponent constant, 46 fraction bits
     i64 ok;            // the trial is inside the fixed-point range
+    double vmax;       // largest centre offset per axis for this MP's separations, in LSB
 };
 static_assert(2 * kExpTable / kLmeWarps >= kLmeRows, "the exp table holds the warps' pair positions");
-static_assert(sizeof(FixStart) == 3 * sizeof(double) + sizeof(MpFix) + 8, "k_lme_fix copies FixStart word by word");
+static_assert(sizeof(FixStart) == 3 * sizeof(double) + sizeof(MpFix), "k_lme_fix copies FixStart word by word");
 
 // centre offset and constant of a trial with a shift; false out of range (or not finite): FP64 evaluation
-__device__ __forceinline__ bool fix_trial(const FixConst &C, const double *trial, double sh, i64 *v, i64 &cst)
+__device__ __forceinline__ bool fix_trial(const FixConst &C, double vmax, const double *trial, double sh, i64 *v, i64 &cst)
 {
     bool ok = true;
     double l2 = 0.0;
     for (int i = 0; i < 3; i++) {
         const double x = trial[i] * C.i2b;
         l2 = fma(trial[i], trial[i], l2);
-        ok = ok && fabs(x) < C.vmax;
+        ok = ok && fabs(x) < vmax;
         v[i] = __double2ll_rn(x);
     }
     const double c = fma(l2, C.cy, -sh * kFixYScale);
@@ -1583,7 +1584,7 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
     const double t0 = from(trial, 0), t1 = from(trial, 1), t2 = from(trial, 2);
     const double l2 = fma(t2, t2, fma(t1, t1, t0 * t0)), v = trial * C.i2b;
     const double sh = m.E[10], c = fma(l2, C.cy, -sh * kFixYScale);
-    const unsigned inside = __ballot_sync(0xffffffffu, q >= 3 || fabs(v) < C.vmax);
+    const unsigned inside = __ballot_sync(0xffffffffu, q >= 3 || fabs(v) < f.vmax);
     __syncwarp();
     const bool finish = conv && regular, next = newton && regular;
     if (accept) {
@@ -1630,7 +1631,7 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
             for (int i = 0; i < 3; i++) m.trial[i] = fma(m.t, m.dir[i], m.lam[i]);
             newton_set_trial(m);
         }
-        if (m.state == kNewtonEval) f.ok = fix_trial(C, m.trial, m.sh, f.v, f.cst) ? 1 : 0;
+        if (m.state == kNewtonEval) f.ok = fix_trial(C, f.vmax, m.trial, m.sh, f.v, f.cst) ? 1 : 0;
     }
     __syncwarp();
     return m.state == kNewtonEval;
@@ -1789,7 +1790,7 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4) k_lme_fix(const __grid_c
                 if (id[j] >= 0) { F.x0[k] = a[j].x; F.x1[k] = a[j].y; F.x2[k] = a[j].z; }
             }
         }
-        if (lane < 11) {   // the start formed by k_lme_prep
+        if (lane < 12) {   // the start formed by k_lme_prep
             const i64 v = ((const i64 *)&D.fstart[p])[lane];
             if (lane < 3) M.trial[lane] = M.ws[lane] = fx_bits_d((u64)v);
             else ((i64 *)&X)[lane - 3] = v;
@@ -1961,8 +1962,8 @@ __global__ void __launch_bounds__(256) k_lme_prep(const __grid_constant__ Dev D)
         s.xp[0] = fix_from_double(x.x, C.fb);
         s.xp[1] = fix_from_double(x.y, C.fb);
         s.xp[2] = fix_from_double(x.z, C.fb);
-        s.ok = fix_trial(C, s.trial, D.logz[p], s.v, s.cst) ? 1 : 0;
-        s.pad = 0;
+        s.vmax = C.vmax;
+        s.ok = fix_trial(C, s.vmax, s.trial, D.logz[p], s.v, s.cst) ? 1 : 0;
         D.fstart[p] = s;
     }
 }
@@ -2662,8 +2663,9 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) far = max(far, (i64)__shfl_xor_sync(0xffffffffu, far, o));
         fixed = __all_sync(0xffffffffu, ok) && (double)far < kFixT;
-        FixConst Cp = C;
-        Cp.vmax = kFixT - (double)far;
+        // what the farthest node leaves of the range bounds every trial of this point (caller's supports may reach
+        // well past the default radius that C.vmax is for)
+        const double vmax = kFixT - (double)far;
         // log Z at the start, plus ln 2.8: Z begins near 0.35 (in FP64 evaluations any shift near log Z does)
         const float sh0 = wm + __logf(ws) + 1.04f;
         const double shift0 = isfinite(sh0) ? (double)sh0 : 0.0;
@@ -2677,7 +2679,8 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
             M.retried = 1;          // no second start here
             M.shift0 = M.sh = shift0;
             M.state = kNewtonEval;
-            X.ok = fix_trial(Cp, M.trial, shift0, X.v, X.cst) ? 1 : 0;
+            X.vmax = vmax;
+            X.ok = fix_trial(C, vmax, M.trial, shift0, X.v, X.cst) ? 1 : 0;
         }
     } else if (lane == 0) {
         M.state = kNewtonIdle;

@@ -39,3 +39,29 @@ def test_gradient_of_a_node_beside_the_point(orc, otm, units, sign):
     got = shape.cpu().numpy()[0]
     assert abs(got[62, 0] - N[62]) <= 1e-11 * N[62]
     assert np.abs(got[62, 1:] - dN[62]).max() <= 1e-9 * np.abs(dN[62]).max()
+
+
+@pytest.mark.parametrize("far", [0.45, 0.55, 0.62, 0.64, 0.655, 0.665, 0.9, 1.1])
+def test_caller_supports_wider_than_the_default(orc, otm, far):
+    """A node `far` of the fixed-point range from the point on every axis (0.23 is the default support radius), and
+    points close to the corner of the body, whose lambda moves the centre of the weights by as much as a radius away
+    from that node. J is near-singular there (its condition is (distance / h)^-1, 1e4 at most), so N is good to
+    1e4 times the 1e-14 of the Newton tolerance: 1e-9 with margin."""
+    rho = np.sqrt(13.815510557964274 / 0.8)
+    h = 2.0 ** -7 * 1.002 / (2.2 * rho)
+    beta, span = 0.8 / h ** 2, 2.0 ** -6
+    x = np.stack(np.meshgrid(*[np.arange(4)] * 3, indexing="ij"), -1).reshape(-1, 3) * h
+    x = np.vstack([x, np.full((1, 3), far * span)])
+    xp = np.array([[d, d, d] for d in (0.4, 0.1, 1e-2, 3e-3, 1e-3, 3e-4)]) * h
+    n, m = len(x), len(xp)
+    ids = np.tile(np.arange(n, dtype=np.int32), (m, 1))
+    tol = 1e-14 * h
+    shape, lam, _, st = otm.lme(dev(x), dev(xp), dev(ids), dev(np.full(m, n, np.int32)), beta, tol)
+    assert st.item() == 0
+    got = shape.cpu().numpy()
+    for p in range(m):
+        so, N, dN, _, _ = orc.lme(xp[p] - x, beta, tol)
+        assert so == 0
+        assert np.abs(got[p, :, 0] - N).max() <= 1e-9
+        assert np.abs(got[p, :, 1:] - dN).max() <= 1e-8 * np.abs(dN).max()
+        assert got[p, -1, 0] <= 1e-15
