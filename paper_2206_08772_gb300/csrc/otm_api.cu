@@ -32,7 +32,9 @@ struct otm_handle {
     bool adj_swap;
     bool adj_shape_swap;           // the two state-shape buffers of the adjoint workspace trade roles
     int64_t adj_shape_step;        // state whose shape functions the spare buffer holds (-1: none)
-    bool state_fix;                // the state's shape functions come from fixed-point evaluations
+    // which evaluations the state's shape functions come from: 0 FP64; fixed point, of supports 1 just
+    // searched, 2 given, frozen or moved by the caller (their separations are checked)
+    int state_fix;
     bool contrib_stale;            // node-major contributions not regenerated by the last load
     void *keep_buf;                // otm_keep_last_good: snapshot of the state before the running step
     // phase timing
@@ -251,13 +253,15 @@ static int read_error(otm_handle *h, int32_t *code, int64_t *id)
 
 // The LME solve of the current positions and supports. A solve that only regenerates the shape functions
 // of the state (kLmeKeep) evaluates them as the solve that led to the state did, whichever path that
-// was, and so repeats them bit for bit; any other solve evaluates as this handle's path does.
-static int solve_lme(otm_handle *h, int lme_mode)
+// was, and so repeats them bit for bit; any other solve evaluates as this handle's path does. `searched`: the
+// supports come from a search at the current positions, so that no separation exceeds r_s.
+static int solve_lme(otm_handle *h, int lme_mode, bool searched)
 {
     Dev &D = h->D;
     D.lme_mode = lme_mode;
-    if (lme_mode != kLmeKeep) h->state_fix = D.precision == OTM_PRECISION_FP64 && D.fix.on;
+    if (lme_mode != kLmeKeep) h->state_fix = D.precision == OTM_PRECISION_FP64 && D.fix.on ? (searched ? 1 : 2) : 0;
     D.lme_fix = h->state_fix && D.fix.on;
+    D.lme_far = h->state_fix == 2;
     CK(launch_lme(D, h->stream, &h->launches));
     return OTM_OK;
 }
@@ -285,7 +289,7 @@ static int rebuild_supports(otm_handle *h, bool insert, int lme_mode)
     }
     {
         PhaseScope ps(h, OTM_PHASE_LME);
-        const int rc = solve_lme(h, lme_mode);
+        const int rc = solve_lme(h, lme_mode, true);
         if (rc != OTM_OK) return rc;
     }
     D.insert_mode = 0;
@@ -400,7 +404,7 @@ static int regenerate_contributions(otm_handle *h)
     if (!h->contrib_stale) return OTM_OK;
     Dev &D = h->D;
     CK(cudaMemsetAsync(D.emax, 0x80, 2 * sizeof(int), h->stream));
-    const int rc = solve_lme(h, kLmeKeep);
+    const int rc = solve_lme(h, kLmeKeep, false);
     if (rc != OTM_OK) return rc;
     h->contrib_stale = false;
     return OTM_OK;
@@ -433,7 +437,7 @@ static int enqueue_step(otm_handle *h)
         CK(cudaMemsetAsync(D.emax, 0x80, 2 * sizeof(int), s));
         {
             PhaseScope ps(h, OTM_PHASE_LME);
-            const int rc = solve_lme(h, kLmeStep);
+            const int rc = solve_lme(h, kLmeStep, false);
             if (rc != OTM_OK) return rc;
         }
         h->step++;
@@ -463,7 +467,7 @@ static int enqueue_step(otm_handle *h)
         {
             PhaseScope ps(h, OTM_PHASE_LME);
             D.insert_mode = h->P.max_insert > 0 ? 1 : 0;
-            const int rc = solve_lme(h, kLmeStep);
+            const int rc = solve_lme(h, kLmeStep, true);
             if (rc != OTM_OK) return rc;
             D.insert_mode = 0;
         }
@@ -786,6 +790,8 @@ extern "C" int otm_set_state(otm_handle *h, int32_t field, const void *host_src,
         const int rc = rows_h2d(h, host_src, v.pitch, v.width, v.rows, (void *)v.src);
         if (rc != OTM_OK) return rc;
     }
+    // positions moved away from the supports' search: a solve that regenerates this state checks them
+    if ((field == OTM_FIELD_NODE_X || field == OTM_FIELD_MP_X) && h->state_fix) h->state_fix = 2;
     if (field == OTM_FIELD_NODE_DU)   // keep the FP32 copy of the increments in step
         CK(launch_du_to_f32(h->D, h->stream, &h->launches));
     CK(cudaStreamSynchronize(h->stream));
@@ -848,7 +854,7 @@ static int replay_step(otm_handle *h, Place place)
     }
     {
         PhaseScope ps(h, OTM_PHASE_LME);
-        const int rc = solve_lme(h, kLmeStep);
+        const int rc = solve_lme(h, kLmeStep, false);
         if (rc != OTM_OK) return rc;
     }
     h->step++;
@@ -985,7 +991,7 @@ extern "C" void otm_destroy(otm_handle *h)
 struct SnapHeader {
     int64_t nn, nm, step, magic, n_inserted;
     int64_t nn_cap, nm_cap, S;     // the layout the snapshot was written with
-    int64_t state_fix;             // its shape functions come from fixed-point evaluations
+    int64_t state_fix;             // its shape functions' evaluations (otm_handle)
 };
 struct SnapField {
     void *p;
@@ -1032,7 +1038,7 @@ extern "C" int otm_snapshot_save(otm_handle *h, void *dst)
     SnapField f[32];
     const int n = snap_fields(h, f);
     SnapHeader hd = {h->D.nn, h->D.nm, h->step, 0x4f544d53, h->n_inserted, h->nn_cap, h->nm0, h->D.S,
-                     h->state_fix ? 1 : 0};
+                     h->state_fix};
     CK(cudaMemcpyAsync(dst, &hd, sizeof(hd), cudaMemcpyDefault, h->stream));
     char *o = (char *)dst + 256;
     for (int i = 0; i < n; i++) {
@@ -1061,7 +1067,7 @@ static int snapshot_load_impl(otm_handle *h, const void *src, const double4_32a 
     h->D.nm = hd.nm;
     h->step = hd.step;
     h->n_inserted = hd.n_inserted;
-    h->state_fix = hd.state_fix != 0;
+    h->state_fix = hd.state_fix == 2 ? 2 : (hd.state_fix ? 1 : 0);
     SnapField f[32];
     const int n = snap_fields(h, f);
     const char *o = (const char *)src + 256;
@@ -1088,7 +1094,7 @@ static int snapshot_load_impl(otm_handle *h, const void *src, const double4_32a 
         CK(cudaMemcpyAsync(D.Kinv, K, (size_t)D.nm * 48, cudaMemcpyDeviceToDevice, h->stream));
         h->contrib_stale = true;
     } else {
-        const int rc = solve_lme(h, kLmeKeep);
+        const int rc = solve_lme(h, kLmeKeep, false);
         if (rc != OTM_OK) return rc;
         h->contrib_stale = false;
     }

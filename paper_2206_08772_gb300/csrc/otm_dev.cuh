@@ -77,6 +77,7 @@ struct Dev {
     FixConst fix;                    // fixed-point LME evaluation
     int kin_fu, kin_fe;              // units of the kinematics gather: du 2^kin_fu, e 2^kin_fe
     int lme_fix;                     // 1: this LME launch evaluates in fixed point (see launch_lme)
+    int lme_far;                     // 1: its supports were not searched at these positions (see k_lme_far)
     double logz0;                    // exponent shift of the first solve
     int max_newton;
     int wall, tool, allow_erode;
@@ -111,7 +112,7 @@ struct Dev {
     uint8_t *lme_fail;               // LME failures of the step (node insertion)
     int32_t *n_fail;                 // their count
     FixStart *fstart;                // starts of the fixed-point LME solves
-    int32_t *lme_defer;              // MPs whose support exceeds k_lme's shared-memory rows
+    int32_t *lme_defer;              // MPs whose support exceeds the LME's shared-memory rows or fixed-point range
     int32_t *n_defer;                // their count (k_lme_wide solves them)
     int32_t *flag;                   // one int of scratch for host-read checks (argument validation)
     int64_t *mgid;

@@ -111,6 +111,7 @@ OTM_HD u64 fx_shl(u64 v, unsigned n) { return n < 64 ? v << n : 0; }
 struct FixConst {
     int on;            // 1: the fixed-point evaluation covers this problem's support radius
     int fb;            // X = round(x 2^fb)
+    uint32_t near;     // high word of r_s (1 + 1e-9)
     u64 bq;            // beta 256/ln2 a^2 2^46 2^63, a = 2^(32 - fb): y units per unit of a^2, halved
     double i2b;        // 2^fb / (2 beta): lambda to the centre offset in LSB
     double cy;         // 256 / (4 beta ln 2): |lambda|^2 to the exponent's constant

@@ -1765,7 +1765,7 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4) k_lme_fix(const __grid_c
     MpNewton &M = B.newton[warp];
     MpFix &X = B.fix[warp];
     bool active = (p < D.nm) && !has_error(D.err);
-    if (active && D.cnt[p] > rows) {   // solved by k_lme_wide
+    if (active && (D.cnt[p] > rows || (D.lme_far && D.fstart[p].vmax < 0.0))) {   // solved by k_lme_wide
         if (lane == 0) D.lme_defer[atomicAdd(D.n_defer, 1)] = (int32_t)p;
         active = false;
     }
@@ -1968,6 +1968,40 @@ __global__ void __launch_bounds__(256) k_lme_prep(const __grid_constant__ Dev D)
     }
 }
 
+// Between k_lme_prep and k_lme_fix when the supports were not searched at the current positions (given or frozen
+// supports, or positions set by the caller): separations may then exceed r_s by any factor, and k_lme_fix keeps
+// coordinates modulo 2^64 (4.4 to 8.8 r_s). Warp per MP: the largest separation of any axis leaves the solve the
+// rest of the range for its centre; from 2^62 units on (1.1 to 2.2 r_s, what the force products take) the MP is
+// left to lme_block (k_lme_wide). Bound by the FP64 pipe (three subtractions a pair; the comparisons
+// go by high words): 0.43 ms beside the solve's 2.48 on 202,752 MPs.
+__global__ void __launch_bounds__(128) k_lme_far(const __grid_constant__ Dev D)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (p >= D.nm) return;
+    const FixConst &C = D.fix;
+    const int n = D.cnt[p];
+    if (n > lme_rows(D.S)) return;   // goes to lme_block as it is
+    const int64_t base = p * (int64_t)D.S;
+    const double4_32a xp = D.xp[p];
+    // magnitudes by their high words (non-finite ones are the largest)
+    unsigned top = 0;
+    for (int k = lane; k < n; k += kWarp) {
+        const double4_32a a = D.x[D.ids[base + k]];
+        const unsigned dx = (unsigned)__double2hiint(xp.x - a.x) & 0x7fffffffu, dy = (unsigned)__double2hiint(xp.y - a.y) & 0x7fffffffu,
+                       dz = (unsigned)__double2hiint(xp.z - a.z) & 0x7fffffffu;
+        top = max(max(top, dx), max(dy, dz));
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane != 0) return;
+    FixStart &s = D.fstart[p];
+    // within r_s (to 2^-20): as after a search, so that supports recorded from a run replay its solves bit for bit
+    if (top <= C.near) return;
+    const double far = __hiloint2double((int)(min(top, 0x7fefffffu) + 1u), 0) / C.r_unit;   // rounded up, in LSB
+    s.vmax = far <= 0x1p62 ? fmin(C.vmax, kFixT - far) : -1.0;
+    s.ok = fix_trial(C, s.vmax, s.trial, D.logz[p], s.v, s.cst) ? 1 : 0;
+}
+
 // The fixed-point evaluation's constants: fb so that the support radius lies between 2^63/4.4 and
 // 2^63/2.2 LSB (a trial's centre may then move by 0.45 support radii or more per axis before it leaves
 // the range). Off where the exponent scale does not fit 64 bits (support tolerances below about
@@ -1987,6 +2021,7 @@ FixConst make_fix_const(double beta, double rs2)
     c.i2b = std::ldexp(1.0, c.fb) / (2.0 * beta);
     c.cy = 64.0 / (beta * std::log(2.0));
     c.vmax = kFixT - std::ldexp(rs, c.fb) * (1.0 + 1e-9);
+    c.near = (uint32_t)(fx_d_bits(rs * (1.0 + 1e-9)) >> 32);
     c.r_unit = std::ldexp(1.0, -c.fb);
     c.a_unit = a * a / 16.0;
     return c;
@@ -2013,6 +2048,10 @@ static cudaError_t launch_lme_t(const Dev &D, cudaStream_t s, unsigned blocks, l
         int64_t pb = ((D.nn > D.nm ? D.nn : D.nm) + 255) / 256;
         if (pb > 152 * 8) pb = 152 * 8;
         k_lme_prep<<<(unsigned)pb, 256, 0, s>>>(D);
+        if (D.lme_far) {
+            k_lme_far<<<(unsigned)((D.nm * kWarp + 127) / 128), 128, 0, s>>>(D);
+            if (launches) *launches += 1;
+        }
         k_lme_fix<MIXED, STAB><<<blocks, kLmeWarps * kWarp, smem, s>>>(D);
         if (launches) *launches += 2;
     } else {
@@ -2024,7 +2063,7 @@ static cudaError_t launch_lme_t(const Dev &D, cudaStream_t s, unsigned blocks, l
         k_lme<MIXED, STAB><<<blocks, kLmeWarps * kWarp, smem, s>>>(D);
         if (launches) *launches += 1;
     }
-    if (D.S > kLmeRows) {
+    if (D.S > kLmeRows || (D.lme_fix && D.lme_far)) {
         // one persistent round of blocks over the deferred MPs (none on most steps: the launch then
         // returns at once)
         const size_t smem = lme_block_smem(D.S);

@@ -65,3 +65,68 @@ def test_caller_supports_wider_than_the_default(orc, otm, far):
         assert np.abs(got[p, :, 0] - N).max() <= 1e-9
         assert np.abs(got[p, :, 1:] - dN).max() <= 1e-8 * np.abs(dN).max()
         assert got[p, -1, 0] <= 1e-15
+
+
+def check_shapes(orc, sim, p, rows, bound=1e-12):
+    x, xp, cnt = sim.get("node_x"), sim.get("mp_x"), sim.get("support_count")
+    ids, sh = sim.get_rows("support_ids", rows), sim.get_rows("shape", rows)
+    for r, q in enumerate(rows):
+        n = cnt[q]
+        st, N, dN, _, _ = orc.lme(xp[q] - x[ids[r, :n]], p.beta, p.newton_tol * p.h)
+        assert st == 0
+        assert np.abs(sh[r, :n, 0] - N).max() <= bound * N.max()
+        assert np.abs(sh[r, :n, 1:] - dN).max() <= 10 * bound * np.abs(dN).max()
+
+
+@pytest.mark.parametrize("how", ["padded", "csr", "moved"])
+@pytest.mark.parametrize("precision,eps", [("fp64", 0.0), ("fp64", 1e-2), ("mixed", 0.0)])
+def test_supports_beyond_the_search(orc, how, precision, eps):
+    """Supports that no search gave: nodes 1.05 to 6 support radii away added to some points' own (4.4 to 8.8 radii are
+    2^64 units of the fixed-point grid), replayed, then kept by frozen steps, each state restored from a snapshot;
+    and positions moved by the caller before a snapshot. Bound as of searched steps: 1e-12 on N (1e-6 and FP32
+    rounding of the gradients in the mixed path)."""
+    import scenarios
+    from paper_2206_08772_gb300.otm import OTM
+    h = 0.8e-3
+    p = scenarios.taylor_rod(h=h, R=3.2e-3, L=26 * h, material=scenarios.copper_jc(), v0=50.0)
+    p.eps_stab = eps * p.materials[0].E * h ** 2
+    bound = 1e-12 if precision == "fp64" else 1e-6
+    base, sim = OTM(p, precision=precision), OTM(p, precision=precision)
+    assert base.step(1) == 0
+    cnt, ids = base.get("support_count"), base.get("support_ids")
+    x, xp = base.get("node_x"), base.get("mp_x")
+    rs = np.sqrt(p.rs2)
+    rows = np.linspace(0, p.n_mps - 1, 40).astype(int)
+    for k, q in enumerate(rows):
+        d = np.sqrt(((xp[q] - x) ** 2).sum(1)) / rs
+        want = [1.05, 1.2, 1.45, 2.2, 2.9, 3.6, 4.6, 4.7, 5.0, 6.0][: 1 + k % 10]
+        add = sorted({int(np.argmin(np.abs(d - w))) for w in want} - set(ids[q, :cnt[q]].tolist()))
+        add = add[: 384 - cnt[q]]
+        ids[q, cnt[q]:cnt[q] + len(add)] = add
+        cnt[q] += len(add)
+    if how == "padded":
+        assert sim.step_with_supports(cnt, ids) == 0, sim.error()
+    elif how == "csr":
+        off = np.concatenate([[0], np.cumsum(cnt)]).astype(np.int32)
+        flat = np.concatenate([ids[q, :cnt[q]] for q in range(p.n_mps)]).astype(np.int32)
+        assert sim.step_with_supports_csr(dev(off), dev(flat)) == 0, sim.error()
+    else:
+        assert sim.step(1) == 0, sim.error()
+        far = np.linspace(0, p.n_nodes - 1, 12).astype(int)
+        x = sim.get("node_x")
+        x[far, 2] += 19.53125 * h * np.linspace(0.3, 1.0, 12)
+        sim.set("node_x", x)
+        sim.restore(sim.snapshot())
+    assert how == "moved" or np.array_equal(sim.get("support_count"), cnt)
+
+    def check():
+        check_shapes(orc, sim, p, rows, bound)
+        before = sim.get("shape")
+        sim.restore(sim.snapshot())
+        assert np.array_equal(before, sim.get("shape"))
+
+    check()
+    if how != "moved":
+        sim.freeze_topology()
+        assert sim.step(2) == 0, sim.error()
+        check()
