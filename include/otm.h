@@ -54,7 +54,7 @@ extern "C" {
 #define OTM_ERR_RETURNMAP_NOCONV (-7) /* Johnson-Cook consistency iteration failed */
 #define OTM_ERR_CAPACITY (-8)         /* support / influence / cell capacity exceeded */
 
-#define OTM_PRECISION_FP64 0          /* FP64 accuracy throughout (pair sums in 59- to 64-bit fixed point) */
+#define OTM_PRECISION_FP64 0          /* FP64 accuracy throughout (the LME solve's pair sums in 64-bit fixed point) */
 #define OTM_PRECISION_MIXED 1         /* FP32 force scatter, node update, pair rows' e = N d and
                                        * kinematics gather (x_p increment and G = sum du (x) N d);
                                        * the LME Newton's Hessian sums in double-float (FP32 pairs,

@@ -102,7 +102,6 @@ static size_t layout(int64_t nn, int64_t nn_cap, int64_t nm, int S, int precisio
     TAKE(d.spos, double4_32a, nn_cap);
     TAKE(d.spos32, float4, nn_cap);
     TAKE(d.du32, float4, nn_cap);
-    if (precision == OTM_PRECISION_FP64) TAKE(d.dufix, int4, 2 * nn_cap);
     TAKE(d.xfix, longlong4_32a, nn_cap);
     TAKE(d.nflags, uint8_t, nn_cap);
     TAKE(d.ngid, int64_t, nn_cap);
@@ -206,9 +205,6 @@ static void fill_params(Dev &D, const otm_params *P)
     D.cell = P->cell_size;
     D.sc = make_search_const(P->cell_size, P->rs2);
     D.fix = make_fix_const(P->beta, P->rs2);
-    // |du| < 2^57 units is at least half a spacing a step; |e| = |N d| <= r_s is below 2^62 half units
-    D.kin_fu = kKinDuBits - ilogb(P->h);
-    D.kin_fe = 61 - ilogb(sqrt(P->rs2) * (1.0 + 1e-9));
     // FP64 path: log of the weights' sum of a regular cloud of spacing h, plus ln 2.8: the first sums
     // start near 0.35, inside the fixed-point evaluation's window
     D.logz0 = P->precision == OTM_PRECISION_FP64 ? 1.5 * log(3.141592653589793 / (P->beta * P->h * P->h)) + 1.04 : 0.0;

@@ -75,7 +75,6 @@ struct Dev {
     double h, beta, rs2, cell, dt, tol_abs, eps_stab;
     SearchConst sc;
     FixConst fix;                    // fixed-point LME evaluation
-    int kin_fu, kin_fe;              // units of the kinematics gather: du 2^kin_fu, e 2^kin_fe
     int lme_fix;                     // 1: this LME launch evaluates in fixed point (see launch_lme)
     int lme_far;                     // 1: its supports were not searched at these positions (see k_lme_far)
     double logz0;                    // exponent shift of the first solve
@@ -91,7 +90,6 @@ struct Dev {
     // nodes
     double4_32a *x, *x_prev, *du, *mr;   // mr = (mass, force xyz) of the last node update
     float4 *du32;
-    int4 *dufix;                     // increments as limbs, two int4 a node: (uh, -) and (8 ul, 1 if out of range)
     longlong4_32a *xfix;             // fixed-point node positions of the running LME solve (otm_fix.cuh)
     uint8_t *nflags;
     int64_t *ngid;

@@ -442,6 +442,8 @@ OTM_HD bool force_fix(const FixRows &R, double N, i64 d0, i64 d1, i64 d2, double
 }
 
 // ------------------------------------------------------------------ kinematics gather (Eq. 9, 11)
+// Not on a step's path: the step gathers in FP64 (k_kin_search), because the units here are fixed by the node
+// spacing and the sums' error does not shrink with the increments. Used by the host tests alone.
 // The products of a pair's row (N, e) with its node's increment du, summed over the support:
 // sum N du (3) and G = sum du (x) e (9). Limbs: du = uh 2^28 + ul (|du| < 2^57 units; uh 29 bits, ul signed 28
 // bits, kept as 8 ul) and row = rh 2^31 + rl (61 bits; rh 30 bits, rl signed 31 bits), so that both cross

@@ -465,7 +465,7 @@ __device__ int warp_support_search(const SearchGrid &G, const SearchConst &C, do
     // rounding of the point, the quotients and the distances; nodes are binned by the exact FP64
     // floor): the rows along x whose (y, z) square it meets, and of each row the cells it reaches. 84
     // cells on average instead of the 125 of the bounding box. With the branch-free tests and the next row's
-    // loads ahead: k_kin_search 1.56 -> 1.41 ms (202,752 MPs, FP64), 2.86 -> 2.64 ms (616 k, mixed).
+    // loads ahead: k_kin_search 2.86 -> 2.64 ms (616 k MPs, mixed).
     const float rsm = rs * 1.0001f + 2.f * e;
     const int y0 = max((int)fmaxf(floorf((Y - rsm) / cf), -1.f), 0);
     const int y1 = min((int)fminf(floorf((Y + rsm) / cf), (float)ny), ny - 1);
@@ -936,7 +936,7 @@ template <>
 struct KinSum<true> {
     float t;
     float c[3];
-    __device__ __forceinline__ void gather(const Dev &D, int64_t base, int n, int lane, void *)
+    __device__ __forceinline__ void gather(const Dev &D, int64_t base, int n, int lane)
     {
         float v[12];
 #pragma unroll
@@ -967,120 +967,18 @@ struct KinSum<true> {
     }
 };
 
-// The FP64 path's gather in fixed point (kin_fix_pair): x_p,n+1 = x_p,n + sum N du (Eq. 9 by the partition of
-// unity and linear reproducibility, as in the mixed path) and G, from the nodes' increments in units of
-// 2^-kin_fu (written by the node update). Errors are below 2^-57 of h in x_p and of 1 in G K, so the
-// roundings of x_p and dF = 1 - G K themselves stay the largest. A support with an increment out of range
-// (half a spacing a step or more) takes the FP64 gather.
-// 12 FP64 FMAs a pair bounded the kernel (pipe 89 % busy); here a pair takes 36 integer multiply-adds, 12 FP32
-// FMAs and about 80 other instructions. k_kin_search on the 202,752-MP rod: 1.61 -> 1.56 ms.
-// A pair's loads (its ID, then row and increment: two dependent latencies) run kKinDepth - 1 passes ahead as
-// asynchronous copies into shared memory, which takes no registers: the sums hold 60. (3 stages: 6 % slower.)
-constexpr int kKinDepth = 2;
-struct KinStage {
-    uint4 c[kKinDepth][4][kWarp];   // row (2 words of 16 bytes), increment (2), one slot a lane
-};
-
-__device__ __forceinline__ void cp16_cg(void *dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp16_ca(void *dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
-struct KinFix {
-    double t;      // this lane's reduced value: 0-2 x_p (or its increment), 3-11 G
-    bool inc;      // values 0-2 are increments
-    __device__ __forceinline__ void gather(const Dev &D, int64_t base, int n, int lane, KinStage *st)
-    {
-        i64 v[12];
-        int wide = 0;
-        {
-            KinFixSums s;
-#pragma unroll
-            for (int i = 0; i < 12; i++) s.hh[i] = s.hl[i] = 0, s.ll[i] = 0.f;
-            const int fe = D.kin_fe;
-            const int32_t *ids = D.ids + base;
-            auto fetch = [&](int k, int id) {   // pass k's copies (a group per pass, empty past the end)
-                if (k < n) {
-                    const int b = (k / kWarp) % kKinDepth;
-                    const char *row = (const char *)(D.shape + base + k), *du = (const char *)(D.dufix + 2 * (int64_t)id);
-                    cp16_cg(&st->c[b][0][lane], row);
-                    cp16_cg(&st->c[b][1][lane], row + 16);
-                    cp16_ca(&st->c[b][2][lane], du);
-                    cp16_ca(&st->c[b][3][lane], du + 16);
-                }
-                asm volatile("cp.async.commit_group;");
-            };
-            int id[kKinDepth];
-#pragma unroll
-            for (int j = 0; j < kKinDepth; j++) id[j] = lane + j * kWarp < n ? ids[lane + j * kWarp] : 0;
-#pragma unroll
-            for (int j = 0; j < kKinDepth - 1; j++) fetch(lane + j * kWarp, id[j]);
-            int idn = id[kKinDepth - 1];
-            const int passes = (n + kWarp - 1) / kWarp;   // warp-uniform: every lane commits and waits alike
-            // two passes a round: one leaves a copy of every sum at the loop's end (48 moves)
-#pragma unroll 2
-            for (int q = 0; q < passes; q++) {
-                const int k = lane + q * kWarp;
-                fetch(k + (kKinDepth - 1) * kWarp, idn);
-                idn = k + kKinDepth * kWarp < n ? ids[k + kKinDepth * kWarp] : 0;
-                asm volatile("cp.async.wait_group %0;" ::"n"(kKinDepth - 1) : "memory");
-                if (k < n) {
-                    const int b = q % kKinDepth;
-                    const double2 r0 = *(const double2 *)&st->c[b][0][lane], r1 = *(const double2 *)&st->c[b][1][lane];
-                    const int4 h = *(const int4 *)&st->c[b][2][lane], l = *(const int4 *)&st->c[b][3][lane];
-                    wide |= l.w;
-                    const int uh[3] = {h.x, h.y, h.z}, ul[3] = {l.x, l.y, l.z};
-                    kin_fix_pair(fix_floor(r0.x, 62), fix_floor(r0.y, fe), fix_floor(r1.x, fe), fix_floor(r1.y, fe), uh, ul, s);
-                }
-            }
-            asm volatile("cp.async.wait_all;" ::: "memory");
-#pragma unroll
-            for (int i = 0; i < 12; i++) v[i] = kin_fix_combine(s, i);
-        }
-        if (__any_sync(0xffffffffu, wide != 0) || n > 12 * kWarp) {
-            KinSum<false> ks;
-            ks.gather(D, base, n, lane);
-            t = ks.t;
-            inc = false;
-            return;
-        }
-        const i64 r = warp_reduce_scatter12(v, lane);
-        t = (double)r * ldexp(1.0, kin_fix_exponent(D.kin_fu, rs12_value(lane) < 3 ? 62 : D.kin_fe));
-        inc = true;
-    }
-    __device__ __forceinline__ double g() const { return t; }
-    __device__ __forceinline__ double xp(double old, int) const { return inc ? old + t : t; }
-};
-
-template <bool MIXED>
-struct KinGather;
-template <>
-struct KinGather<false> {
-    using type = KinFix;
-    using stage = KinStage;
-};
-template <>
-struct KinGather<true> {
-    using type = KinSum<true>;
-    struct stage {};
-};
-
 // ======================================================================== k_kin_search
 // Kinematics (Eq. 9, 11) and the support search at the new position (Algorithm 3) in one warp
 // per MP: the gather over the old support gives x_p and dF, then the candidate scan builds the
 // new support in the same row. Used when no erosion can remove MPs between the two; the
 // return map (which only needs dF) follows.
-// Occupancy: both are bound by latency. Mixed: 12 blocks per SM (40 registers, a 24-byte spill) 2.64 ms, 10
-// blocks 2.84 ms on 616 k MPs. FP64: the gather's sums take 60 registers; 6 blocks (80 registers, a 116-byte
-// spill) 1.41 ms, 5 blocks 1.47 ms on 202,752 MPs, and the two as separate kernels 1.5 ms.
+// Mixed: bound by latency; 12 blocks per SM (40 registers, a 24-byte spill) 2.64 ms, 10 blocks 2.84 ms on 616 k
+// MPs. FP64: bound by the gather's 12 FP64 FMAs a pair (1.1 of 1.60 ms on 202,752 MPs, where 6, 7 and 8 blocks
+// are within 0.3 % and 10 take 1.63); 8 blocks also suit the search's latency on few MPs (9,984: 0.110 ms, 6 blocks
+// 0.116). The sums in fixed point, in units of 2^-57 h, take 1.43 ms, but their error does not shrink with the
+// increments: 13 times the FP64 sums' at 0.013 h a step, 1e6 times at 1e-7 h.
 template <bool MIXED>
-__global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 6) k_kin_search(const __grid_constant__ Dev D)
+__global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 8) k_kin_search(const __grid_constant__ Dev D)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1090,9 +988,8 @@ __global__ void __launch_bounds__(kSearchWarps * kWarp, MIXED ? 12 : 6) k_kin_se
     const int S = D.S;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)S;
-    __shared__ typename KinGather<MIXED>::stage kst[kSearchWarps];
-    typename KinGather<MIXED>::type ks;
-    ks.gather(D, base, n, lane, &kst[(threadIdx.x >> 5)]);
+    KinSum<MIXED> ks;
+    ks.gather(D, base, n, lane);
     const int j = rs12_value(lane);
     if (rs12_writer(lane) && j >= 3) D.dF[9 * p + (j - 3)] = ks.g();   // G = sum du (x) e; k_return_map forms dF
     // values 0, 1, 2 (x_p) sit at lanes 0, 2, 4
@@ -2101,9 +1998,8 @@ __global__ void __launch_bounds__(128) k_kinematics(const __grid_constant__ Dev 
     if (has_error(D.err)) return;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)D.S;
-    __shared__ typename KinGather<MIXED>::stage kst[kSearchWarps];
-    typename KinGather<MIXED>::type ks;
-    ks.gather(D, base, n, lane, &kst[(threadIdx.x >> 5)]);
+    KinSum<MIXED> ks;
+    ks.gather(D, base, n, lane);
     const int j = rs12_value(lane);
     if (rs12_writer(lane)) {
         if (j < 3) {

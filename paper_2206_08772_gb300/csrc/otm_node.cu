@@ -165,20 +165,8 @@ __global__ void __launch_bounds__(kNodeWarps * kWarp) k_node_update(const __grid
         if (D.tool) tool_project(D, t_next, ux, uy, uz, x, y, z);
     }
     ux = x - xo.x; uy = y - xo.y; uz = z - xo.z;
-    if (MIXED) {
+    if (MIXED)
         D.du32[i] = make_float4((float)ux, (float)uy, (float)uz, 0.f);
-    } else {   // the kinematics gather's copy
-        const double top = ldexp(1.0, kKinDuBits - D.kin_fu);
-        const bool in = fabs(ux) < top && fabs(uy) < top && fabs(uz) < top;
-        int4 h = make_int4(0, 0, 0, 0), l = make_int4(0, 0, 0, in ? 0 : 1);
-        if (in) {
-            kin_fix_split(fix_from_double(ux, D.kin_fu), h.x, l.x);
-            kin_fix_split(fix_from_double(uy, D.kin_fu), h.y, l.y);
-            kin_fix_split(fix_from_double(uz, D.kin_fu), h.z, l.z);
-        }
-        D.dufix[2 * i] = h;
-        D.dufix[2 * i + 1] = l;
-    }
     D.du[i] = make_double4_32a(ux, uy, uz, 0.0);
     D.x_prev[i] = xo;
     D.x[i] = make_double4_32a(x, y, z, 0.0);
