@@ -37,13 +37,15 @@ __device__ __forceinline__ void broadcast9(double v, double (&M)[9])
 
 // ---------------------------------------------------------------------------- LME backward
 // d_a = x_p - x_a, N = softmax(f), f_a = -beta |d_a|^2 + lambda . d_a, lambda from r = sum N d = 0,
-// grad N_a = -N_a K d_a, K^-1 = H = sum N d d^T. With e_a = N_a d_a (the stored row) and r = 0:
+// grad N_a = -N_a K d_a, K^-1 = H = sum N d d^T - r r^T. With e_a = N_a d_a (the stored row), r = sum e_a (zero to
+// the caller's Newton tolerance) and c = 2 Hs r:
 //   B = sum g_a e_a^T, Hs = sym(B K)                          (the adjoint of H)
-//   q_a = dL/dN_a - g_a . d_a + d_a . Hs d_a,  S = sum N_a q_a = sum N_a dL/dN_a  (tr B cancels tr(Hs H))
+//   q_a = dL/dN_a - g_a . d_a + d_a . (Hs d_a - c)
+//   S = sum N_a q_a = sum N_a dL/dN_a - r . c / 2             (tr B cancels tr(Hs H))
 //   lambda_bar = sum (q_a - S) e_a,  m = K lambda_bar          (implicit function theorem on r = 0)
-//   dL/dd_a = N_a [2 Hs d_a - g_a - m + (q_a - S - d_a . m)(lambda - 2 beta d_a)]
-// Three passes over the pairs with about 55 FP64 instructions each in all (about 115 when H is summed
-// again and the r terms, of relative size 1e-14, are carried): 4.69 -> 2.64 ms on 78,624 MPs.
+//   dL/dd_a = N_a [2 Hs d_a - c - g_a - m + (q_a - S - d_a . m)(lambda - 2 beta d_a)]
+// Three passes over the pairs with about 58 FP64 instructions in all (about 115 when H is summed again):
+// 4.69 -> 2.84 ms on 78,624 MPs (2.64 without the r terms, which then err by the caller's tolerance).
 __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_constant__ Dev D, const __grid_constant__ AdjDev A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -55,35 +57,40 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
     double *qa = sm, *wx = sm + S, *wy = sm + 2 * S, *wz = sm + 3 * S;
     const int n = D.cnt[p];
     const int64_t base = p * (int64_t)S;
-    // B and S
-    double v[10];
+    // B, S and r
+    double v[16];
 #pragma unroll
-    for (int i = 0; i < 10; i++) v[i] = 0.0;
+    for (int i = 0; i < 16; i++) v[i] = 0.0;
     for (int k = lane; k < n; k += kWarp) {
         const double4_32a sh = D.shape[base + k], pb = A.pb_cur[base + k];
         v[0] = fma(pb.y, sh.y, v[0]); v[1] = fma(pb.y, sh.z, v[1]); v[2] = fma(pb.y, sh.w, v[2]);
         v[3] = fma(pb.z, sh.y, v[3]); v[4] = fma(pb.z, sh.z, v[4]); v[5] = fma(pb.z, sh.w, v[5]);
         v[6] = fma(pb.w, sh.y, v[6]); v[7] = fma(pb.w, sh.z, v[7]); v[8] = fma(pb.w, sh.w, v[8]);
         v[9] = fma(sh.x, pb.x, v[9]);
+        v[10] += sh.y; v[11] += sh.z; v[12] += sh.w;
     }
-    const double t = warp_reduce_scatter10(v, lane);
-    const double Ssum = __shfl_sync(0xffffffffu, t, rs10_lane(9));
+    const double t = warp_reduce_scatter16(v, lane);   // value j at lanes 2j, 2j+1
     // lane 3 i + j: (B K)_ij, then its symmetric part
     const double *K = D.Kinv + 6 * p;
     const int li = lane < 9 ? lane / 3 : 0, lj = lane < 9 ? lane % 3 : 0;
     double bk = 0.0;
 #pragma unroll
-    for (int k = 0; k < 3; k++) bk = fma(__shfl_sync(0xffffffffu, t, rs10_lane(3 * li + k)), K[sym6(k, lj)], bk);
+    for (int k = 0; k < 3; k++) bk = fma(__shfl_sync(0xffffffffu, t, 2 * (3 * li + k)), K[sym6(k, lj)], bk);
     bk = 0.5 * (bk + __shfl_sync(0xffffffffu, bk, 3 * lj + li));
     const double s00 = __shfl_sync(0xffffffffu, bk, 0), s11 = __shfl_sync(0xffffffffu, bk, 4), s22 = __shfl_sync(0xffffffffu, bk, 8);
     const double s01 = __shfl_sync(0xffffffffu, bk, 1), s12 = __shfl_sync(0xffffffffu, bk, 5), s02 = __shfl_sync(0xffffffffu, bk, 2);
+    const double r0 = __shfl_sync(0xffffffffu, t, 20), r1 = __shfl_sync(0xffffffffu, t, 22), r2 = __shfl_sync(0xffffffffu, t, 24);
+    const double c0 = 2.0 * fma(s02, r2, fma(s01, r1, s00 * r0)), c1 = 2.0 * fma(s12, r2, fma(s11, r1, s01 * r0)),
+                 c2 = 2.0 * fma(s22, r2, fma(s12, r1, s02 * r0));
+    const double Ssum = fma(-0.5, fma(r2, c2, fma(r1, c1, r0 * c0)), __shfl_sync(0xffffffffu, t, 18));
     const double4_32a xp = D.xp[p];
     double lb[3] = {0.0, 0.0, 0.0};
     for (int k = lane; k < n; k += kWarp) {
         const double4_32a a = D.x[D.ids[base + k]], sh = D.shape[base + k], pb = A.pb_cur[base + k];
         const double x = xp.x - a.x, y = xp.y - a.y, z = xp.z - a.z;
-        const double h0 = fma(s02, z, fma(s01, y, s00 * x)), h1 = fma(s12, z, fma(s11, y, s01 * x)),
-                     h2 = fma(s22, z, fma(s12, y, s02 * x));
+        // Hs d - c; w below is short of c, which joins m
+        const double h0 = fma(s02, z, fma(s01, y, fma(s00, x, -c0))), h1 = fma(s12, z, fma(s11, y, fma(s01, x, -c1))),
+                     h2 = fma(s22, z, fma(s12, y, fma(s02, x, -c2)));
         const double g0 = h0 - pb.y, g1 = h1 - pb.z, g2 = h2 - pb.w;
         const double q = fma(z, g2, fma(y, g1, fma(x, g0, pb.x - Ssum)));
         qa[k] = q;
@@ -94,6 +101,7 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
     const double m0 = fma(K[0], lb0, fma(K[3], lb1, K[5] * lb2)), m1 = fma(K[3], lb0, fma(K[1], lb1, K[4] * lb2)),
                  m2 = fma(K[5], lb0, fma(K[4], lb1, K[2] * lb2));
     const double l0 = D.lam[3 * p], l1 = D.lam[3 * p + 1], l2 = D.lam[3 * p + 2], b2 = -2.0 * D.beta;
+    const double mc0 = m0 - c0, mc1 = m1 - c1, mc2 = m2 - c2;
     // scatter to the node and to x_p
     double px = 0, py = 0, pz = 0;
     for (int k = lane; k < n; k += kWarp) {
@@ -101,9 +109,9 @@ __global__ void __launch_bounds__(kAdjWarps * kWarp) k_adj_lme(const __grid_cons
         const double4_32a a = D.x[nid];
         const double x = xp.x - a.x, y = xp.y - a.y, z = xp.z - a.z, N = D.shape[base + k].x;
         const double c = fma(-x, m0, fma(-y, m1, fma(-z, m2, qa[k])));
-        const double o0 = N * fma(c, fma(b2, x, l0), wx[k] - m0);
-        const double o1 = N * fma(c, fma(b2, y, l1), wy[k] - m1);
-        const double o2 = N * fma(c, fma(b2, z, l2), wz[k] - m2);
+        const double o0 = N * fma(c, fma(b2, x, l0), wx[k] - mc0);
+        const double o1 = N * fma(c, fma(b2, y, l1), wy[k] - mc1);
+        const double o2 = N * fma(c, fma(b2, z, l2), wz[k] - mc2);
         px += o0; py += o1; pz += o2;
         A.sc1[(int64_t)D.noff[nid] + D.rank[base + k]] = make_double4_32a(o0, o1, o2, 0.0);
     }
