@@ -26,6 +26,7 @@
  *  - Fields come back in ascending ID order (erosion removes entries, never reorders them).
  *  - After an error the state is that of the failing step, partially updated (the oracle
  *    behaves the same way); otm_error_detail names the code and the smallest offending ID.
+ *    The SHAPE rows of an MP whose LME solve failed are unspecified then.
  *    otm_keep_last_good makes otm_step leave the state at the last good step instead.
  *  - Device reset: the library keeps two pieces of module data per device (the tables of its
  *    FP64 exponential and logarithm, and the allocation-free search's scratch address), set up by
@@ -341,7 +342,8 @@ int otm_support_search_noalloc(const double *node_x, int64_t n_nodes, const doub
 /* LME shape functions (Eq. 14) for n_mps points with given supports (ids/counts as produced
  * by otm_support_search). lambda (n_mps x 3, in: start, out: solution). shape: n_mps x
  * max_support x 4 doubles (N, dN/dx, dN/dy, dN/dz). iters (n_mps, optional). status: as above
- * (OTM_ERR_LME_NOCONV on failure). */
+ * (OTM_ERR_LME_NOCONV on failure). Slots past counts[p] and the rows of a point that fails are not
+ * written. */
 int otm_lme(const double *node_x, const double *mp_x, int64_t n_mps, const int32_t *ids,
             const int32_t *counts, int32_t max_support, double beta, double tol_abs,
             int32_t max_newton, double *lambda, double *shape, int32_t *iters, int32_t *status,

@@ -378,7 +378,6 @@ size_t scan_tmp_ints(int64_t n);
 bool carve_search_scratch(void *base, size_t bytes, int64_t nn, SearchScratch *S);
 cudaError_t build_search_grid(const double *node_x, int64_t nn, double cell, SearchScratch *S,
                               double *grid_out, cudaStream_t s);
-size_t lme_smem_bytes(int S, int warps);
 cudaError_t launch_adjoint_backward(const Dev &D, const AdjDev &A, cudaStream_t s, long long *launches);
 cudaError_t launch_rebuild_ranks(const Dev &D, cudaStream_t s, long long *launches);
 cudaError_t launch_csr_gather(const Dev &D, const int32_t *off, int32_t *ids, cudaStream_t s, long long *launches);

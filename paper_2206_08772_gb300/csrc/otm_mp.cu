@@ -82,8 +82,7 @@ __device__ __forceinline__ void df_add(float &sh, float &sl, float q, float f)
 //   exp(f) = 2^(n >> 10) * 2^((n & 1023) / 1024) * exp(s ln2 / 1024),
 // with exp(t) - 1 for |t| <= ln2/2048 by its Taylor polynomial of degree 3 (truncation below
 // 5.5e-16 relative). The 1024-entry table 2^(j/1024) is computed once on the host (C library
-// exp2) into g_exp2_table; the LME step kernel reads it through L1, the stand-alone kernels stage
-// it into shared memory. Valid for f in about
+// exp2) into g_exp2_table; the kernels read it through L1. Valid for f in about
 // [-707, 708]; below it returns 0 (a weight below 1e-307 of the largest), above +inf (the caller
 // then re-shifts). The scaling rounds y like any FP64 argument, so the result carries
 // |f| * 2^-53 relative error from it, plus about 3 ulps.
@@ -248,164 +247,13 @@ struct LmeSums {
     double shift;
 };
 
-// q[] and the multipliers passed here are in exponent units of ln2/1024 (see exp_scaled)
-template <bool SHIFTED>
-__device__ __forceinline__ void lme_accumulate(const double *dx, const double *dy, const double *dz, const double *q,
-                                               double *w, int n, double l0, double l1, double l2, double qs,
-                                               int lane, const double *T, double (&v)[16])
-{
-    for (int k = lane; k < n; k += kWarp) {
-        const double x = dx[k], y = dy[k], z = dz[k];
-        const double qk = SHIFTED ? q[k] + qs : q[k];
-        const double f = fma(l2, z, fma(l1, y, fma(l0, x, qk)));
-        const double wk = exp_scaled(f, T);
-        w[k] = wk;
-        const double wx = wk * x, wy = wk * y, wz = wk * z;
-        v[0] += wk;
-        v[1] += wx; v[2] += wy; v[3] += wz;
-        v[4] = fma(wx, x, v[4]); v[5] = fma(wy, y, v[5]); v[6] = fma(wz, z, v[6]);
-        v[7] = fma(wx, y, v[7]); v[8] = fma(wy, z, v[8]); v[9] = fma(wx, z, v[9]);
-    }
-}
-
-__device__ __forceinline__ void lme_sums(const double *dx, const double *dy, const double *dz, const double *q,
-                                         double *w, int n, double l0, double l1, double l2, double shift,
-                                         double q0shift, int lane, const double *T, LmeSums &E)
-{
-    double v[16];
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = 0.0;
-    // q[] holds (prior exponent - the solve's first shift) * 1024/ln2; a different shift (only
-    // after an over/underflow) is applied as a difference
-    const double qs = (q0shift - shift) * kExpScale;
-    const double s0 = l0 * kExpScale, s1 = l1 * kExpScale, s2 = l2 * kExpScale;
-    if (qs == 0.0)
-        lme_accumulate<false>(dx, dy, dz, q, w, n, s0, s1, s2, qs, lane, T, v);
-    else
-        lme_accumulate<true>(dx, dy, dz, q, w, n, s0, s1, s2, qs, lane, T, v);
-    const double t = warp_reduce_scatter16(v, lane);   // value j at lanes 2j, 2j+1
-    E.Z = __shfl_sync(0xffffffffu, t, 0);
-    E.r0 = __shfl_sync(0xffffffffu, t, 2);
-    E.r1 = __shfl_sync(0xffffffffu, t, 4);
-    E.r2 = __shfl_sync(0xffffffffu, t, 6);
-    E.a00 = __shfl_sync(0xffffffffu, t, 8);
-    E.a11 = __shfl_sync(0xffffffffu, t, 10);
-    E.a22 = __shfl_sync(0xffffffffu, t, 12);
-    E.a01 = __shfl_sync(0xffffffffu, t, 14);
-    E.a12 = __shfl_sync(0xffffffffu, t, 16);
-    E.a02 = __shfl_sync(0xffffffffu, t, 18);
-    E.shift = shift;
-}
-
-__device__ __forceinline__ double lme_fmax(const double *dx, const double *dy, const double *dz,
-                                           const double *q, int n, double l0, double l1, double l2,
-                                           double q0shift, int lane)
-{
-    const double s0 = l0 * kExpScale, s1 = l1 * kExpScale, s2 = l2 * kExpScale;
-    double m = -INFINITY;
-    for (int k = lane; k < n; k += kWarp) m = fmax(m, q[k] + (s0 * dx[k] + s1 * dy[k] + s2 * dz[k]));
-    return warp_max(m) * (1.0 / kExpScale) + q0shift;
-}
-
-// evaluation with the given shift; if the weights over- or underflow, again with max f
-__device__ __forceinline__ void lme_sums_safe(const double *dx, const double *dy, const double *dz,
-                                              const double *q, double *w, int n, double l0, double l1,
-                                              double l2, double shift, double q0shift, int lane, const double *T,
-                                              LmeSums &E)
-{
-    lme_sums(dx, dy, dz, q, w, n, l0, l1, l2, shift, q0shift, lane, T, E);
-    if (!(E.Z > 1e-200) || !(E.Z < 1e200)) {
-        const double fm = lme_fmax(dx, dy, dz, q, n, l0, l1, l2, q0shift, lane);
-        lme_sums(dx, dy, dz, q, w, n, l0, l1, l2, fm, q0shift, lane, T, E);
-    }
-}
-
 __device__ __forceinline__ double rn2(const LmeSums &E) { return E.r0 * E.r0 + E.r1 * E.r1 + E.r2 * E.r2; }
-
-// J' = A - r r^T / Z and its adjugate / determinant (cofactors); false if not positive definite.
-// iZ_out (optional) receives 1 / Z.
-__device__ __forceinline__ bool lme_jinv(const LmeSums &E, double inv[6], double *iZ_out = nullptr)
-{
-    const double iZ = 1.0 / E.Z;
-    if (iZ_out) *iZ_out = iZ;
-    const double s0 = E.r0 * iZ, s1 = E.r1 * iZ, s2 = E.r2 * iZ;
-    const double j00 = E.a00 - s0 * E.r0, j11 = E.a11 - s1 * E.r1, j22 = E.a22 - s2 * E.r2;
-    const double j01 = E.a01 - s0 * E.r1, j12 = E.a12 - s1 * E.r2, j02 = E.a02 - s0 * E.r2;
-    const double c00 = j11 * j22 - j12 * j12;
-    const double c01 = j02 * j12 - j01 * j22;
-    const double c02 = j01 * j12 - j02 * j11;
-    const double c11 = j00 * j22 - j02 * j02;
-    const double c12 = j01 * j02 - j00 * j12;
-    const double c22 = j00 * j11 - j01 * j01;
-    const double det = j00 * c00 + j01 * c01 + j02 * c02;
-    if (!(det > 0.0) || !isfinite(det)) return false;
-    const double id = 1.0 / det;
-    inv[0] = c00 * id; inv[1] = c11 * id; inv[2] = c22 * id;
-    inv[3] = c01 * id; inv[4] = c12 * id; inv[5] = c02 * id;   // (xx, yy, zz, xy, yz, xz) of J'^-1
-    return true;
-}
 
 // log Z(trial) < log Z(current)
 __device__ __forceinline__ bool logz_less(const LmeSums &t, const LmeSums &c)
 {
     if (t.shift == c.shift) return t.Z < c.Z;
     return t.shift + log(t.Z) < c.shift + log(c.Z);
-}
-
-// Damped Newton on the convex log Z(lambda): step -J^-1 (r/Z) = -J'^-1 r, halved until log Z or
-// the residual norm drops; stops when |r| / Z <= tol. All evaluations of one solve share the
-// initial shift (the previous step's log Z, so w ~ N), which makes the log Z comparison a
-// comparison of Z; q[] must hold the prior exponent minus that shift, times 1024/ln2. On return
-// w[] holds the weights of the accepted evaluation E. Warp-uniform.
-// Newton iterations from an evaluation E already taken at lambda (see lme_newton).
-__device__ int lme_newton_loop(const double *dx, const double *dy, const double *dz, const double *q, double *w,
-                               int n, double &l0, double &l1, double &l2, double shift, double tol, int max_it,
-                               int lane, const double *T, LmeSums &E, int &iters)
-{
-    const double tol2 = tol * tol;
-    for (;;) {
-        const double r2 = rn2(E);
-        if (!isfinite(r2) || !isfinite(E.Z)) return OTM_ERR_LME_NOCONV;
-        if (r2 <= tol2 * E.Z * E.Z) return OTM_OK;
-        if (iters >= max_it) return OTM_ERR_LME_NOCONV;
-        iters++;
-        double inv[6];
-        if (!lme_jinv(E, inv)) return OTM_ERR_LME_NOCONV;
-        const double s0 = -(inv[0] * E.r0 + inv[3] * E.r1 + inv[5] * E.r2);
-        const double s1 = -(inv[3] * E.r0 + inv[1] * E.r1 + inv[4] * E.r2);
-        const double s2 = -(inv[5] * E.r0 + inv[4] * E.r1 + inv[2] * E.r2);
-        double t = 1.0;
-        bool accepted = false;
-        LmeSums Et;
-        double m0 = l0, m1 = l1, m2 = l2;
-        for (int halving = 0; halving < 40; halving++) {
-            m0 = fma(t, s0, l0); m1 = fma(t, s1, l1); m2 = fma(t, s2, l2);
-            lme_sums_safe(dx, dy, dz, q, w, n, m0, m1, m2, E.shift, shift, lane, T, Et);
-            if (isfinite(Et.Z) && (logz_less(Et, E) || rn2(Et) * (E.Z * E.Z) < r2 * (Et.Z * Et.Z))) {
-                accepted = true;
-                break;
-            }
-            t *= 0.5;
-        }
-        if (!accepted) return OTM_ERR_LME_NOCONV;
-        l0 = m0; l1 = m1; l2 = m2;
-        E = Et;
-    }
-}
-
-// Damped Newton on the convex log Z(lambda): step -J^-1 (r/Z) = -J'^-1 r, halved until log Z or
-// the residual norm drops; stops when |r| / Z <= tol. All evaluations of one solve share the
-// initial shift (the previous step's log Z, so w ~ N), which makes the log Z comparison a
-// comparison of Z; q[] must hold the prior exponent minus that shift, times 1024/ln2. On return
-// w[] holds the weights of the accepted evaluation E. Warp-uniform.
-__device__ int lme_newton(const double *dx, const double *dy, const double *dz, const double *q, double *w,
-                          int n, double &l0, double &l1, double &l2, double shift, double tol, int max_it,
-                          int lane, const double *T, LmeSums &E, int &iters)
-{
-    iters = 0;
-    if (n <= 0) return OTM_ERR_LME_NOCONV;
-    lme_sums_safe(dx, dy, dz, q, w, n, l0, l1, l2, shift, shift, lane, T, E);
-    return lme_newton_loop(dx, dy, dz, q, w, n, l0, l1, l2, shift, tol, max_it, lane, T, E, iters);
 }
 
 // ======================================================================== support search
@@ -564,21 +412,11 @@ struct WarpSmem {
     double *dx, *dy, *dz, *q, *w;
 };
 
-__device__ __forceinline__ WarpSmem warp_smem(unsigned char *base, int S, int warp)
-{
-    unsigned char *b = base + (size_t)warp * 5 * (size_t)S * sizeof(double);
-    WarpSmem W;
-    W.dx = (double *)b;
-    W.dy = W.dx + S;
-    W.dz = W.dy + S;
-    W.q = W.dz + S;
-    W.w = W.q + S;
-    return W;
-}
-
 constexpr int kLmeWarps = 4;
 
-// The damped Newton solve of Eq. 14 for the block's MPs, block-synchronous: each round, every
+// The damped Newton solve of Eq. 14 for the block's MPs: the convex log Z(lambda) by steps -J^-1 (r/Z) = -J'^-1 r,
+// halved until log Z or the residual norm drops, to |r| / Z <= tol. All evaluations of a solve share its first
+// shift, which makes the log Z comparison a comparison of Z. Block-synchronous: each round, every
 // warp whose MP has an evaluation pending computes the sums (Z, r, A) at its trial lambda (the
 // pair loop); then one warp takes the scalar decisions of all of them (accept or halve the trial, the
 // convergence test, J'^-1, the next Newton step), eight lanes an MP. FP64 instructions cost the pipe
@@ -739,10 +577,9 @@ __device__ __forceinline__ void newton_fail(MpNewton &m)
     }
 }
 
-// One scalar round after an evaluation (the damped Newton of lme_newton_loop, as a state machine) for the block's
+// One scalar round after an evaluation (the damped Newton as a state machine) for the block's
 // four MPs, eight lanes each (called by one warp): every lane forms the shared scalars, and lane q its entry of
-// J', of the cofactors and of the step, in the operations and order of lme_jinv and lme_newton_loop; a
-// lane per MP issued 75 FP64 instructions a round, this 47 (mixed k_lme on 616 k MPs: 14.19 -> 13.33 ms, the same
+// J', of the cofactors and of the step; a lane per MP issued 75 FP64 instructions a round, this 47 (mixed k_lme on 616 k MPs: 14.19 -> 13.33 ms, the same
 // bits). True for the lanes of an MP with another evaluation to come.
 // ZOFF: the binary exponent the next solve's Z starts below (see the end)
 template <int ZOFF>
@@ -833,14 +670,6 @@ __device__ __forceinline__ bool newton_round(MpNewton *NS, double tol, int max_i
     __syncwarp();
     return m.state == kNewtonEval;
 }
-
-// shared memory of the stand-alone LME kernel (k_lme_only): the exp table and rows of S slots
-size_t lme_smem_bytes(int S, int warps)
-{
-    return kExpTable * sizeof(double) + (size_t)warps * 5 * (size_t)S * sizeof(double) +
-           (size_t)warps * sizeof(MpNewton);
-}
-
 
 // The new support of an MP into its row (IDs from the warp's list) and each pair's rank in its
 // node's influence list, by counting with atomics; three slots per lane at a time, so that three
@@ -1597,11 +1426,23 @@ struct NodeX3 {
     }
 };
 
-// the same evaluation in FP64, for trials outside the fixed-point range: coordinates from global
-// memory, the weights to w[0], w[ws], w[2 ws], ...; shift handling as lme_eval_block
+// the same evaluation in FP64, for trials outside the fixed-point range: coordinates from global memory, the
+// weights to w (if given); shift handling as lme_eval_block
+// exponent scale units of one pair's weight at lambda s / kExpScale with shift sh_s / kExpScale; d = x_p - x_a
+template <typename X>
+__device__ __forceinline__ double lme_weight64(X x, int id, double px, double py, double pz, double beta_s, double s0, double s1,
+                                               double s2, double sh_s, double &dx, double &dy, double &dz)
+{
+    double ax, ay, az;
+    x.get(id, ax, ay, az);
+    dx = px - ax; dy = py - ay; dz = pz - az;
+    const double q = fma(-beta_s, fma(dz, dz, fma(dy, dy, dx * dx)), -sh_s);
+    return exp_scaled(fma(s2, dz, fma(s1, dy, fma(s0, dx, q))), g_exp2_table);
+}
+
 template <typename X>
 __device__ __noinline__ void lme_eval64(X x, const int32_t *ids, double px, double py, double pz, double beta_s, double *w,
-                                        int ws, int n, MpNewton &m, int lane)
+                                        int n, MpNewton &m, int lane)
 {
     const double s0 = m.trial[0] * kExpScale, s1 = m.trial[1] * kExpScale, s2 = m.trial[2] * kExpScale;
     double sh = m.sh, v[10], t = 0.0;
@@ -1610,12 +1451,9 @@ __device__ __noinline__ void lme_eval64(X x, const int32_t *ids, double px, doub
 #pragma unroll
         for (int i = 0; i < 10; i++) v[i] = 0.0;
         for (int k = lane; k < n; k += kWarp) {
-            double ax, ay, az;
-            x.get(ids[k], ax, ay, az);
-            const double dx = px - ax, dy = py - ay, dz = pz - az;
-            const double q = fma(-beta_s, fma(dz, dz, fma(dy, dy, dx * dx)), -sh_s);
-            const double wk = exp_scaled(fma(s2, dz, fma(s1, dy, fma(s0, dx, q))), g_exp2_table);
-            w[k * ws] = wk;
+            double dx, dy, dz;
+            const double wk = lme_weight64(x, ids[k], px, py, pz, beta_s, s0, s1, s2, sh_s, dx, dy, dz);
+            if (w) w[k] = wk;
             const double wx = wk * dx, wy = wk * dy, wz = wk * dz;
             v[0] += wk;
             v[1] += wx; v[2] += wy; v[3] += wz;
@@ -1706,7 +1544,7 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4) k_lme_fix(const __grid_c
         if (M.state == kNewtonEval) {
             __syncwarp();
             if (!(X.ok && lme_eval_fix<!MIXED>(C, F, cnt, M, X, lane, T)))
-                lme_eval64(NodeX4{D.x}, D.ids + base, D.xp[p].x, D.xp[p].y, D.xp[p].z, D.beta * kExpScale, F.w, 1, cnt, M,
+                lme_eval64(NodeX4{D.x}, D.ids + base, D.xp[p].x, D.xp[p].y, D.xp[p].z, D.beta * kExpScale, F.w, cnt, M,
                            lane);
         }
         __syncthreads();
@@ -2468,66 +2306,13 @@ cudaError_t launch_search_only(const double *node_x, int64_t nn, const double *m
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kLmeWarps * kWarp)
-    k_lme_only(const double *node_x, const double *mp_x, int64_t nm, const int32_t *ids, const int32_t *counts,
-               int S, double beta, double tol, int max_newton, double *lam, double *shape, int32_t *iters_out,
-               int32_t *status)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *T = (double *)smem_raw;
-    exp_table_load(T);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t p = (int64_t)blockIdx.x * kLmeWarps + warp;
-    if (p >= nm) return;
-    WarpSmem W = warp_smem(smem_raw + kExpTable * sizeof(double), S, warp);
-    const int n = counts[p];
-    if (n > S || n <= 0) {
-        if (lane == 0) atomicCAS(status, 0, n > S ? OTM_ERR_CAPACITY : OTM_ERR_LME_NOCONV);
-        return;
-    }
-    const double px = mp_x[3 * p], py = mp_x[3 * p + 1], pz = mp_x[3 * p + 2];
-    const int64_t base = p * (int64_t)S;
-    for (int k = lane; k < n; k += kWarp) {
-        const int64_t id = ids[base + k];
-        const double x = px - node_x[3 * id], y = py - node_x[3 * id + 1], z = pz - node_x[3 * id + 2];
-        W.dx[k] = x; W.dy[k] = y; W.dz[k] = z;
-        W.q[k] = -(beta * kExpScale) * fma(z, z, fma(y, y, x * x));
-    }
-    __syncwarp();
-    double l0 = lam[3 * p], l1 = lam[3 * p + 1], l2 = lam[3 * p + 2];
-    const double shift = lme_fmax(W.dx, W.dy, W.dz, W.q, n, l0, l1, l2, 0.0, lane);
-    const double shift_s = shift * kExpScale;
-    for (int k = lane; k < n; k += kWarp) W.q[k] -= shift_s;
-    __syncwarp();
-    LmeSums E;
-    int iters = 0;
-    int st = lme_newton(W.dx, W.dy, W.dz, W.q, W.w, n, l0, l1, l2, shift, tol, max_newton, lane, T, E, iters);
-    double inv[6];
-    if (st == OTM_OK && !lme_jinv(E, inv)) st = OTM_ERR_LME_NOCONV;
-    if (lane == 0) {
-        if (iters_out) iters_out[p] = iters;
-        if (st != OTM_OK) atomicCAS(status, 0, st);
-        lam[3 * p] = l0; lam[3 * p + 1] = l1; lam[3 * p + 2] = l2;
-    }
-    if (st != OTM_OK) return;
-    const double iZ = 1.0 / E.Z;
-    for (int k = lane; k < n; k += kWarp) {
-        const double wk = W.w[k];
-        const double x = W.dx[k], y = W.dy[k], z = W.dz[k];
-        double *o = shape + 4 * (base + k);
-        o[0] = wk * iZ;
-        o[1] = -wk * (inv[0] * x + inv[3] * y + inv[5] * z);
-        o[2] = -wk * (inv[3] * x + inv[1] * y + inv[4] * z);
-        o[3] = -wk * (inv[5] * x + inv[4] * y + inv[2] * z);
-    }
-}
-
 // Stand-alone LME with fixed-point evaluations: the block solve of k_lme_fix over caller arrays. The support
 // radius is not an argument here, so the units are those of the default support tolerance (1e-6), every
-// separation is checked against the range, and points outside it, or with more than kLmeRows nodes,
-// are evaluated in FP64 (the weights then pass through their output rows). The exponent shift is
-// estimated in FP32 from the start. Measured (151,392 points of a rod, five evaluations each):
-// k_lme_only 9.7 ms, this kernel 3.3 ms.
+// separation is checked against the range, and points outside it, or with more than kLmeRows nodes, or
+// all of them where the length scale is outside the exponent arithmetic's (C.on = 0), are evaluated in FP64. The
+// weights of more than kLmeRows nodes have no place in shared memory and are formed again for the output. The
+// exponent shift is estimated in FP32 from the start. Measured (151,392 points of a rod, five evaluations
+// each): 9.7 ms with all in FP64, 3.3 ms so.
 __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
     k_lme_only_fix(const double *node_x, const double *mp_x, int64_t nm, const int32_t *ids, const int32_t *counts, int S,
                    double beta, const __grid_constant__ FixConst C, double tol, int max_newton, double *lam, double *shape,
@@ -2554,13 +2339,13 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
     if (active) {
         px = mp_x[3 * p]; py = mp_x[3 * p + 1]; pz = mp_x[3 * p + 2];
         i64 P[3], Ph[3];
-        bool ok = n <= kLmeRows;
+        bool ok = C.on && n <= kLmeRows;
         ok = fix_from_double_wide(px, C.fb, P[0], Ph[0]) && ok;
         ok = fix_from_double_wide(py, C.fb, P[1], Ph[1]) && ok;
         ok = fix_from_double_wide(pz, C.fb, P[2], Ph[2]) && ok;
         const double l0 = lam[3 * p], l1 = lam[3 * p + 1], l2 = lam[3 * p + 2];
         const float bf = (float)beta, lf0 = (float)l0, lf1 = (float)l1, lf2 = (float)l2, u32 = (float)(C.r_unit * 0x1p32);
-        i64 far = 0;                // largest |D| of any component
+        i64 far = 0;                // largest |D| of any component (less one unit for negative ones)
         float mx = -INFINITY, sum = 0.f;   // running log-sum of the exponents at the start
         constexpr int G = 4;        // passes of dependent gathers in flight (150 k points: 1 3.56, 2 3.47, 4 3.45 ms)
         for (int k0 = lane; k0 < n; k0 += G * kWarp) {
@@ -2583,7 +2368,7 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
                 ok = fix_from_double_wide(a[i], C.fb, lo, hi) && ok;
                 const i64 D = (i64)((u64)P[i] - (u64)lo);
                 ok = ok && (Ph[i] - hi - ((u64)P[i] < (u64)lo ? 1 : 0)) == (D >> 63);
-                far = max(far, D < 0 ? -D : D);
+                far = max(far, D ^ (D >> 63));
                 d[i] = (float)(int)(D >> 32) * u32;
                 if (k < kLmeRows) (i == 0 ? F.x0 : (i == 1 ? F.x1 : F.x2))[k] = lo;
             }
@@ -2620,14 +2405,13 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
     } else if (lane == 0) {
         M.state = kNewtonIdle;
     }
-    double *w = n <= kLmeRows ? F.w : shape + 4 * base;
-    const int ws = n <= kLmeRows ? 1 : 4;
+    double *w = n <= kLmeRows ? F.w : nullptr;
     __syncthreads();
     for (;;) {
         if (M.state == kNewtonEval) {
             __syncwarp();
             if (!(fixed && X.ok && lme_eval_fix<true>(C, F, n, M, X, lane, B.table)))
-                lme_eval64(nx, ids + base, px, py, pz, beta * kExpScale, w, ws, n, M, lane);
+                lme_eval64(nx, ids + base, px, py, pz, beta * kExpScale, w, n, M, lane);
         }
         __syncthreads();
         const bool pending = warp == 0 && fix_round(B.newton, B.fix, C, tol, max_newton, lane);
@@ -2647,14 +2431,20 @@ __global__ void __launch_bounds__(kLmeWarps * kWarp, 4)
 #pragma unroll
     for (int i = 0; i < 6; i++) K[i] = -M.inv[i] * Z;
     const bool wide = ((uintptr_t)shape & 31) == 0;
+    const double s0 = M.lam[0] * kExpScale, s1 = M.lam[1] * kExpScale, s2 = M.lam[2] * kExpScale, sh_s = M.C[10] * kExpScale;
 #pragma unroll 1
     for (int k = lane; k < n; k += kWarp) {
-        const double N = w[k * ws] * iZ;
-        double ex, ey, ez;
-        if (fixed) {
+        double N, ex, ey, ez;
+        if (!w) {
+            double dx, dy, dz;
+            N = lme_weight64(nx, ids[base + k], px, py, pz, beta * kExpScale, s0, s1, s2, sh_s, dx, dy, dz) * iZ;
+            ex = N * dx; ey = N * dy; ez = N * dz;
+        } else if (fixed) {
+            N = w[k] * iZ;
             fix_nd(N, X.xp[0] - F.x0[k], X.xp[1] - F.x1[k], X.xp[2] - F.x2[k], C.fb, C.r_unit, ex, ey, ez);
         } else {
             double ax, ay, az;
+            N = w[k] * iZ;
             nx.get(ids[base + k], ax, ay, az);
             ex = N * (px - ax); ey = N * (py - ay); ez = N * (pz - az);
         }
@@ -2675,20 +2465,12 @@ cudaError_t launch_lme_only(const double *node_x, const double *mp_x, int64_t nm
 {
     const unsigned blocks = (unsigned)((nm + kLmeWarps - 1) / kLmeWarps);
     if (blocks == 0) return cudaSuccess;
-    const FixConst C = make_fix_const(beta, 13.815510557964274 / beta);
-    if (C.on) {
-        const size_t smem = sizeof(FixBlock);
-        cudaError_t e = cudaFuncSetAttribute(k_lme_only_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_lme_only_fix<<<blocks, kLmeWarps * kWarp, smem, s>>>(node_x, mp_x, nm, ids, counts, S, beta, C, tol_abs,
-                                                              max_newton, lam, shape, iters, status);
-        return cudaGetLastError();
-    }
-    const size_t smem = lme_smem_bytes(S, kLmeWarps);
-    cudaError_t e = cudaFuncSetAttribute(k_lme_only, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(FixBlock);
+    const cudaError_t e = cudaFuncSetAttribute(k_lme_only_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_lme_only<<<blocks, kLmeWarps * kWarp, smem, s>>>(node_x, mp_x, nm, ids, counts, S, beta, tol_abs, max_newton,
-                                                       lam, shape, iters, status);
+    k_lme_only_fix<<<blocks, kLmeWarps * kWarp, smem, s>>>(node_x, mp_x, nm, ids, counts, S, beta,
+                                                          make_fix_const(beta, 13.815510557964274 / beta), tol_abs, max_newton,
+                                                          lam, shape, iters, status);
     return cudaGetLastError();
 }
 

@@ -130,3 +130,57 @@ def test_supports_beyond_the_search(orc, how, precision, eps):
         sim.freeze_topology()
         assert sim.step(2) == 0, sim.error()
         check()
+
+
+@pytest.mark.parametrize("n", [40, 336, 337, 400])
+def test_rows_of_a_failed_point_stay_as_they_were(orc, otm, n):
+    """Points outside the hull of their supports fail: their rows, and the unused slots of the others, keep what the
+    caller had there, on either side of the 336 nodes that the fixed-point kernel takes."""
+    import ctypes as C
+    import paper_2206_08772_gb300 as g
+    h = 1.3e-3
+    rng = np.random.default_rng(n)
+    x = np.stack(np.meshgrid(*[np.arange(-4, 5)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    x = (x[np.argsort((x ** 2).sum(1), kind="stable")][:n] + rng.uniform(-0.02, 0.02, (n, 3))) * h
+    m, S, tol, beta = 9, 416, 1e-14 * h, 0.8 / h ** 2
+    xp = rng.uniform(0.1, 0.3, (m, 3)) * h
+    bad = np.arange(m) % 3 == 1
+    xp[bad] += 6.0 * h
+    xd, pd, ids, cnt = dev(x), dev(xp), dev(np.tile(np.arange(S, dtype=np.int32) % n, (m, 1))), dev(np.full(m, n, np.int32))
+    shape = torch.full((m, S, 4), 7.25, dtype=torch.float64, device="cuda")
+    lam = torch.zeros(m, 3, dtype=torch.float64, device="cuda")
+    iters = torch.full((m,), -1, dtype=torch.int32, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    P = lambda t: C.c_void_p(t.data_ptr())
+    assert g.load().otm_lme(P(xd), P(pd), m, P(ids), P(cnt), S, beta, tol, 50, P(lam), P(shape), P(iters), P(status),
+                            C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    assert status.item() == -4
+    sh = shape.cpu().numpy()
+    assert (iters.cpu().numpy() >= 0).all()
+    for q in range(m):
+        st, N, dN, _, _ = orc.lme(xp[q] - x, beta, tol)
+        assert (st != 0) == bad[q]
+        assert (sh[q, n:] == 7.25).all()
+        if bad[q]:
+            assert (sh[q] == 7.25).all()
+        else:
+            assert np.abs(sh[q, :n, 0] - N).max() <= 1e-12 and np.abs(sh[q, :n, 1:] - dN).max() <= 1e-11 * np.abs(dN).max()
+
+
+@pytest.mark.parametrize("h", [1e-22, 1e40])
+@pytest.mark.parametrize("n", [60, 400])
+def test_length_scales_outside_the_fixed_point(orc, otm, h, n):
+    """Length scales beyond the exponent arithmetic's are evaluated in FP64; 1e-12 on N as elsewhere."""
+    rng = np.random.default_rng(n)
+    x = np.stack(np.meshgrid(*[np.arange(-4, 5)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    x = (x[np.argsort((x ** 2).sum(1), kind="stable")][:n] + rng.uniform(-0.02, 0.02, (n, 3))) * h
+    m, tol, beta = 5, 1e-14 * h, 0.8 / h ** 2
+    xp = rng.uniform(0.1, 0.3, (m, 3)) * h
+    shape, lam, _, st = otm.lme(dev(x), dev(xp), dev(np.tile(np.arange(n, dtype=np.int32), (m, 1))),
+                                dev(np.full(m, n, np.int32)), beta, tol)
+    assert st.item() == 0
+    sh = shape.cpu().numpy()
+    for q in range(m):
+        so, N, dN, _, _ = orc.lme(xp[q] - x, beta, tol)
+        assert so == 0
+        assert np.abs(sh[q, :, 0] - N).max() <= 1e-12 and np.abs(sh[q, :, 1:] - dN).max() <= 1e-11 * np.abs(dN).max()
