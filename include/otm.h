@@ -272,7 +272,8 @@ int otm_snapshot_bytes(otm_handle *h, size_t *bytes);
  * node-major lists from the stored state, reproducing them exactly. A snapshot loads into any
  * handle made with the same problem sizes, max_support and max_insert, of either precision
  * (otherwise OTM_ERR_ARG); the FP32 increments are rebuilt from the FP64 ones, and the shape functions
- * by the kind of evaluation (fixed point or FP64) that produced the stored state. */
+ * by the kind of evaluation (fixed point or FP64) that produced the stored state (FP64 for snapshots
+ * that do not name it). */
 int otm_snapshot_save(otm_handle *h, void *dst);
 int otm_snapshot_load(otm_handle *h, const void *src);
 

@@ -987,8 +987,11 @@ extern "C" void otm_destroy(otm_handle *h)
 struct SnapHeader {
     int64_t nn, nm, step, magic, n_inserted;
     int64_t nn_cap, nm_cap, S;     // the layout the snapshot was written with
-    int64_t state_fix;             // its shape functions' evaluations (otm_handle)
+    int64_t state_fix;             // its shape functions' evaluations (otm_handle); only with kSnapMagic
 };
+// snapshots with the first magic end before state_fix: whatever the buffer held lies there, and their shape
+// functions come from FP64 evaluations
+constexpr int64_t kSnapMagic = 0x4f544d54, kSnapMagicFp64 = 0x4f544d53;
 struct SnapField {
     void *p;
     size_t row;
@@ -1033,7 +1036,7 @@ extern "C" int otm_snapshot_save(otm_handle *h, void *dst)
     if (!h || !dst || (((uintptr_t)dst) & 255)) return OTM_ERR_ARG;
     SnapField f[32];
     const int n = snap_fields(h, f);
-    SnapHeader hd = {h->D.nn, h->D.nm, h->step, 0x4f544d53, h->n_inserted, h->nn_cap, h->nm0, h->D.S,
+    SnapHeader hd = {h->D.nn, h->D.nm, h->step, kSnapMagic, h->n_inserted, h->nn_cap, h->nm0, h->D.S,
                      h->state_fix};
     CK(cudaMemcpyAsync(dst, &hd, sizeof(hd), cudaMemcpyDefault, h->stream));
     char *o = (char *)dst + 256;
@@ -1056,14 +1059,14 @@ static int snapshot_load_impl(otm_handle *h, const void *src, const double4_32a 
     SnapHeader hd;
     CK(cudaStreamSynchronize(h->stream));
     CK(cudaMemcpy(&hd, src, sizeof(hd), cudaMemcpyDefault));
-    if (hd.magic != 0x4f544d53 || hd.nn > h->nn_cap || hd.nm > h->nm0) return OTM_ERR_ARG;
+    if ((hd.magic != kSnapMagic && hd.magic != kSnapMagicFp64) || hd.nn > h->nn_cap || hd.nm > h->nm0) return OTM_ERR_ARG;
     if (hd.nn_cap != h->nn_cap || hd.nm_cap != h->nm0 || hd.S != h->D.S) return OTM_ERR_ARG;
     if (want_step >= 0 && hd.step != want_step) return OTM_ERR_ARG;
     h->D.nn = hd.nn;
     h->D.nm = hd.nm;
     h->step = hd.step;
     h->n_inserted = hd.n_inserted;
-    h->state_fix = hd.state_fix == 2 ? 2 : (hd.state_fix ? 1 : 0);
+    h->state_fix = hd.magic == kSnapMagic ? (int)hd.state_fix : 0;
     SnapField f[32];
     const int n = snap_fields(h, f);
     const char *o = (const char *)src + 256;
