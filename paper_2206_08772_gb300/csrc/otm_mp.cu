@@ -1292,9 +1292,8 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
     const bool finite = isfinite(rn) && isfinite(Z);
     const bool conv = accept && finite && rn <= tol * tol * Z * Z;
     const bool newton = accept && finite && !conv && m.iters < max_it;
-    // J' = A - r r^T / Z at the accepted point, lane q its entry (xx, yy, zz, xy, yz, xz); r r^T / Z is
-    // second order in the residual, so the approximate 1/Z does
-    const double iZ = recip<0>(Z);
+    // J' = A - r r^T / Z at the accepted point, lane q its entry (xx, yy, zz, xy, yz, xz)
+    const double iZ = recip<2>(Z);
     const int ei = nib(0x010210), ej = nib(0x221210);
     const double ri = ei == 0 ? r0 : (ei == 1 ? r1 : r2), rj = ej == 0 ? r0 : (ej == 1 ? r1 : r2);
     const double J = q < 6 ? fma(-(ri * iZ), rj, m.E[4 + q]) : 0.0;
@@ -1340,7 +1339,7 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
         if (q < 6) m.inv[q] = inv;
         if (q == 0) {
             m.have_cur = 1;
-            m.iZ = recip<2>(Z);
+            m.iZ = iZ;
             // the next solve's shift: its Z then starts in [1/4, 1/2) (see newton_round)
             const int ez = ((__double2hiint(Z) >> 20) & 0x7ff) - 1023;
             m.logz = fma((double)(ez + 2), 0x1.62e42fefa39efp-1, sh);
