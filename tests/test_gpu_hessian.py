@@ -38,3 +38,21 @@ def test_inverse_hessian_at_any_newton_tolerance(tol):
         assert res.max() <= tol + 1e-14
         if tol > 1e-3 and steps == 0:
             assert res.max() > 0.05 * tol
+
+
+@pytest.mark.parametrize("tol", [1e-2, 1e-14])
+def test_double_float_hessian_sums_of_the_mixed_path(tol):
+    """The mixed handle's own solves (its first and after steps), whose A is summed in double-float, 1e-14 of its trace:
+    times the condition of H and three products, 1e-11. A snapshot of an FP64 handle regenerates in fixed point and
+    does not reach these sums."""
+    from paper_2206_08772_gb300.otm import OTM
+    p = scenarios.taylor_rod(h=0.8e-3, R=3.2e-3, L=6.4e-3, material=scenarios.copper_jc())
+    p.newton_tol = tol
+    sim = OTM(p, precision="mixed")
+    rows = np.arange(0, p.n_mps, 5)
+    for steps in (0, 3):
+        assert steps == 0 or sim.step(steps) == 0, sim.error()
+        K, _ = inverse_hessians(sim, p, rows)
+        err = (np.abs(sim.get("kinv")[rows] - K).max(1) / np.abs(K).max(1)).max()
+        print("mixed J^-1 against the exported N:", steps, err)
+        assert err <= 1e-11
