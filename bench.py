@@ -21,8 +21,10 @@ adjoint     : adjoint/forward time ratio of the hand-written GPU adjoint on the 
 e2e         : the same metric through the C ABI from page-locked host memory: the state at the
               window's start loaded from a host snapshot (H2D of every node, MP and support array),
               then every step followed by a D2H of the node positions (after one untimed load).
-roofline    : the dominant kernel of the step (largest phase time) against the FP64 peak, with
-              the method's algorithmic flops (frac) and the kernel's executed flops (frac_executed).
+roofline    : the dominant kernel of the step (largest phase time) against the pipe that binds it: the
+              integer pipe for the FP64 path's LME kernel (frac; its executed FP64 flops of the FP64 peak
+              beside it, frac_executed: the kernel's loops use the two pipes in turn), else FP64 or
+              FP32.
 cpu_baseline: the serial FP64 oracle on a bounded sample of the same workload (a contiguous
               block of material points in the middle of the rod, with the full node set), started
               from the GPU's state at the window's start; cpu_baseline_all_cores: the oracle's
@@ -64,12 +66,14 @@ MIXED_DTYPE = ("f32 scatter/node update/kinematics gather/row N d, double-float 
 #  lambda . d + prior: 6; Z, r, J = sum w d d^T: 1 + 6 + 12), once 15 (d_a and the prior term,
 #  N, grad N) and 17 (mass and force contributions): (1 + k) 25 + 32.
 #  executed in FP64 by the FP64 path's kernel: 17 once (N 1, mass 1, force Q e 15). Its evaluations
-#  (exponent, exp, Z, r, J) and e = N d run in fixed point on the integer pipes, so the algorithmic
-#  rate may exceed the FP64 peak.
+#  (exponent, exp, Z, r, J) and e = N d run in fixed point on the integer pipe: per evaluation 53 wide
+#  or high multiply-adds (32 lanes a clock and SM, counted as 2 operations) and about 75 others (64
+#  lanes), once 12 and about 60.
 LME_ALG_PER_EVAL, LME_ALG_ONCE = 25, 32
 LME_EXEC_PER_EVAL, LME_EXEC_ONCE = 0, 17
+LME_INT_PER_EVAL, LME_INT_ONCE = 2 * 53 + 75, 2 * 12 + 60
 #  k_search (FP32): 8 flops per candidate (3 sub, 1 mul, 2 fma); candidates ~ 3.73 x support.
-#  k_kinematics: 24 flops per pair (x_p: 3 fma, G = sum du (x) e: 9 fma; the FP64 path's in fixed point).
+#  k_kinematics: 24 flops per pair (x_p: 3 fma, G = sum du (x) e: 9 fma).
 SEARCH_PER_CAND, CAND_PER_PAIR = 8, 3.73
 KIN_PER_PAIR = 24
 # DRAM bytes per pair of one k_lme_fix launch, from the ncu capture of the h 0.4 mm rod
@@ -78,6 +82,7 @@ KIN_PER_PAIR = 24
 LME_DRAM_BYTES_PER_PAIR = (0.150299e9 + 1.289973e9) / (78624 * 256.6)
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12   # 2 FP64 FMA lanes / SM / clock at 2070 MHz
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
+INT_PEAK_TOPS = 152 * 64 * 2.070e9 / 1e12
 
 
 def aggregate(ms_local: float, n_mps: int, steps: int, world: int, dist, device="cpu"):
@@ -680,7 +685,9 @@ def main():
     pairs = n_bar * prob.n_mps
     lme_alg = pairs * (LME_ALG_PER_EVAL * (1 + k_bar) + LME_ALG_ONCE) / 1e12
     lme_exec = pairs * (LME_EXEC_PER_EVAL * (1 + k_bar) + LME_EXEC_ONCE) / 1e12
-    work = {"lme": (lme_alg, FP64_PEAK_TFLOPS, "fp64")}   # kernel -> (algorithmic TFLOP per launch, peak, kind)
+    lme_int = pairs * (LME_INT_PER_EVAL * (1 + k_bar) + LME_INT_ONCE) / 1e12
+    # kernel -> (TFLOP, or tera integer operations, per launch; peak; kind)
+    work = {"lme": (lme_int, INT_PEAK_TOPS, "int32") if args.precision == "fp64" else (lme_alg, FP64_PEAK_TFLOPS, "fp64")}
     if phases.get("kinematics", 0.0) > 0.0:     # separate kernels
         work["search"] = (pairs * CAND_PER_PAIR * SEARCH_PER_CAND / 1e12, FP32_PEAK_TFLOPS, "fp32")
         work["kinematics"] = (pairs * KIN_PER_PAIR / 1e12, FP64_PEAK_TFLOPS, "fp64")
@@ -689,24 +696,27 @@ def main():
     kernels = {}
     for k, (tf, peak, kind) in work.items():
         ms_k = phases[k]
-        kernels[k] = {"ms": ms_k, "achieved_tflops": tf / (ms_k / 1e3), "peak": peak, "kind": kind,
+        kernels[k] = {"ms": ms_k, "achieved": tf / (ms_k / 1e3), "peak": peak, "kind": kind,
                       "frac": tf / (ms_k / 1e3) / peak}
     dom = max(kernels, key=lambda k: kernels[k]["ms"])
     kd = kernels[dom]
-    roofline = {"kernel": "k_lme_fix" if dom == "lme" and args.precision == "fp64" else f"k_{dom}", "bound": "alu", "achieved": kd["achieved_tflops"], "peak": kd["peak"],
-                "unit": "TFLOP/s", "frac": kd["frac"],
+    roofline = {"kernel": "k_lme_fix" if dom == "lme" and args.precision == "fp64" else f"k_{dom}", "bound": "alu", "achieved": kd["achieved"], "peak": kd["peak"],
+                "unit": "Tops/s" if kd["kind"] == "int32" else "TFLOP/s", "frac": kd["frac"],
                 # the executed-flop count and the captured DRAM bytes are those of the FP64 path's kernel
-                "frac_executed": ((lme_exec / (kd["ms"] / 1e3) / kd["peak"])
+                "frac_executed": ((lme_exec / (kd["ms"] / 1e3) / FP64_PEAK_TFLOPS)
                                   if dom == "lme" and args.precision == "fp64" else None),
                 "flops_per_pair": {"algorithmic": LME_ALG_PER_EVAL * (1 + k_bar) + LME_ALG_ONCE,
+                                   "integer_ops": (LME_INT_PER_EVAL * (1 + k_bar) + LME_INT_ONCE
+                                                   if args.precision == "fp64" else None),
                                    "executed": (LME_EXEC_PER_EVAL * (1 + k_bar) + LME_EXEC_ONCE
                                                 if args.precision == "fp64" else None)},
                 "traffic": LME_DRAM_BYTES_PER_PAIR * pairs if dom == "lme" and args.precision == "fp64" else None,
                 "traffic_note": ("bytes per launch: DRAM bytes per pair of the ncu capture on the 78,624-MP rod "
                                  "(profiles/) x this launch's pairs"),
-                "peak_source": ("derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2070 MHz (no FP64 entry in the "
-                                "measured peaks)" if kd["kind"] == "fp64"
-                                else "derived: 152 SMs x 128 FP32 FMA/clk x 2 x 2070 MHz"),
+                "peak_source": {"fp64": "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2070 MHz (no FP64 entry in the "
+                                        "measured peaks)",
+                                "fp32": "derived: 152 SMs x 128 FP32 FMA/clk x 2 x 2070 MHz",
+                                "int32": "derived: 152 SMs x 64 integer operations/clk x 2070 MHz"}[kd["kind"]],
                 "kernel_ms": kd["ms"], "share_of_step": kd["ms"] / (ms / args.steps), "kernels": kernels}
     cpu = cpu_all = None
     if not args.no_cpu_baseline:
