@@ -60,7 +60,8 @@ extern "C" {
                                        * kinematics gather (x_p increment and G = sum du (x) N d);
                                        * the LME Newton's Hessian sums in double-float (FP32 pairs,
                                        * ~2^-47); the weights, N, Z, the residual, dF = 1 - G K, F
-                                       * and the return map in FP64 */
+                                       * and the return map in FP64. Takes about a quarter less
+                                       * memory; FP64 is the faster of the two */
 
 #define OTM_FLAG_FIXED 1              /* node flag: displacement increment held at zero */
 
@@ -81,7 +82,8 @@ typedef struct otm_params {
     double cell_size;    /* linked-cell edge, >= sqrt(rs2)/2 (stencil +-2 cells) */
     double dt;           /* time step */
     double T0;           /* initial temperature */
-    double newton_tol;   /* Newton stops when |sum N_a (x_p - x_a)| <= newton_tol * h */
+    double newton_tol;   /* Newton stops when |sum N_a (x_p - x_a)| <= newton_tol * h. The mixed path moves
+                          * x_p by sum N_a du_a, which is Eq. 9 up to this tolerance */
     double eps_stab;     /* stabilisation penalty of Eq. 7 (0 = off) */
     int32_t max_newton;  /* Newton iteration limit */
     int32_t n_materials; /* 1..4 */

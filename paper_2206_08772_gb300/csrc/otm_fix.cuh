@@ -1,4 +1,4 @@
-// otm_fix.cuh -- fixed-point arithmetic of the LME solve (Eq. 14).
+// otm_fix.cuh -- fixed-point arithmetic of the LME solve (Eq. 14), its force products and the node sums.
 //
 // Why: an FP64 instruction occupies an SM of this GPU for 16 cycles per warp (2 lanes per cycle), a
 // 32x32->64-bit integer multiply-add for 1 and a 32-bit integer operation for 0.5. The exponents,

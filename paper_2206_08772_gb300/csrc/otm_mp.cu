@@ -802,8 +802,8 @@ struct KinSum<true> {
 // new support in the same row. Used when no erosion can remove MPs between the two; the
 // return map (which only needs dF) follows.
 // Mixed: bound by latency; 12 blocks per SM (40 registers, a 24-byte spill) 2.64 ms, 10 blocks 2.84 ms on 616 k
-// MPs. FP64: bound by the gather's 12 FP64 FMAs a pair (1.1 of 1.60 ms on 202,752 MPs, where 6, 7 and 8 blocks
-// are within 0.3 % and 10 take 1.63); 8 blocks also suit the search's latency on few MPs (9,984: 0.110 ms, 6 blocks
+// MPs. FP64: bound by the gather's 12 FP64 FMAs a pair (FP64 pipe 90 % busy; 1.60 ms on 202,752 MPs, where 6, 7
+// and 8 blocks are within 0.3 % and 10 take 1.63); 8 blocks also suit the search's latency on few MPs (9,984: 0.110 ms, 6 blocks
 // 0.116). The sums in fixed point, in units of 2^-57 h, take 1.43 ms, but their error does not shrink with the
 // increments: 13 times the FP64 sums' at 0.013 h a step, 1e6 times at 1e-7 h.
 template <bool MIXED>
@@ -1003,7 +1003,7 @@ struct LmeStab<true> {
 // The same for the FP64 output loop of k_lme_fix, as c (e + dF N q) with e = N (x_p - x_a) at hand, q = x_a,n-1 -
 // x_p,n-1 and c = eps / |q|: the reciprocal root from the approximate one by a step of third order (5 FP64
 // instructions; the root and the division took about 35 of the term's 62), and x_prev one pass ahead. Bound by the
-// FP64 pipe, 27 of the loop's 38 instructions there; k_lme_fix on 78,624 stabilised MPs: 2.52 -> 1.91 ms.
+// FP64 pipe, 27 of the loop's 29 instructions there; k_lme_fix on 78,624 stabilised MPs: 2.52 -> 1.91 ms.
 struct StabFix {
     double xq0, xq1, xq2, F[9], eps, lim;
     double4_32a a;                     // x_prev of the pass's pair
