@@ -1256,13 +1256,18 @@ __device__ __forceinline__ bool fix_trial(const FixConst &C, double vmax, const 
 // STEPS Newton steps y += y (1 - x y), each of which doubles the bits. The division operator takes
 // about twice the FP64 instructions.
 template <int STEPS>
+__device__ __forceinline__ double recip_refine(double x, double y)
+{
+#pragma unroll
+    for (int i = 0; i < STEPS; i++) y = fma(y, fma(-x, y, 1.0), y);
+    return y;
+}
+template <int STEPS>
 __device__ __forceinline__ double recip(double x)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-#pragma unroll
-    for (int i = 0; i < STEPS; i++) y = fma(y, fma(-x, y, 1.0), y);
-    return y;
+    return recip_refine<STEPS>(x, y);
 }
 
 // One scalar round after the block's evaluations (the damped Newton of newton_round), for the block's
@@ -1292,8 +1297,10 @@ __device__ __forceinline__ bool fix_round(MpNewton *NS, MpFix *FS, const FixCons
     const bool finite = isfinite(rn) && isfinite(Z);
     const bool conv = accept && finite && rn <= tol * tol * Z * Z;
     const bool newton = accept && finite && !conv && m.iters < max_it;
-    // J' = A - r r^T / Z at the accepted point, lane q its entry (xx, yy, zz, xy, yz, xz)
-    const double iZ = recip<2>(Z);
+    // J' = A - r r^T / Z at the accepted point, lane q its entry (xx, yy, zz, xy, yz, xz). The approximate 1/Z does for
+    // the direction of a step; where the solve ends, K needs all of it (the caller's tolerance bounds r)
+    double iZ = recip<0>(Z);
+    if (conv) iZ = recip_refine<2>(Z, iZ);
     const int ei = nib(0x010210), ej = nib(0x221210);
     const double ri = ei == 0 ? r0 : (ei == 1 ? r1 : r2), rj = ej == 0 ? r0 : (ej == 1 ? r1 : r2);
     const double J = q < 6 ? fma(-(ri * iZ), rj, m.E[4 + q]) : 0.0;
